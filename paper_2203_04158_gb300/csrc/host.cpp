@@ -129,6 +129,9 @@ void stag_fill(StagDesc &d, std::vector<uint64_t> &tab) {
             }
         }
     }
+    // a rank is the sum of its chunks' entries: entries that each fit 32 bits
+    // are not enough when the sector itself is larger (35 choose 17)
+    mx = std::max(mx, binom(d.M, d.N) - 1);
     d.wide = mx > 0xFFFFFFFFull ? 1 : 0;
 }
 

@@ -82,6 +82,18 @@ def test_comb_large_sectors_against_oracle(G, M, N, R):
     assert np.all(as_u64(pats[:2]) == np.uint64(0xFFFFFFFFFFFFFFFF))
 
 
+@pytest.mark.parametrize("M,N,R", [(35, 17, 8), (35, 18, 8), (36, 14, 12), (34, 17, 8)])
+def test_comb_rank_sums_beyond_32_bits(G, M, N, R):
+    """Sectors around 2^32 states whose table entries may each fit 32 bits:
+    the highest ranks come out whole."""
+    D = math.comb(M, N)
+    u = np.unique(np.concatenate([np.arange(D - 50, D), np.arange(2**32 - 50, min(D, 2**32 + 50)), [0]])).astype(np.uint64)
+    u = u[u < D]
+    pats = np.array([oracle.unrank(M, N, int(i)) for i in u], dtype=np.uint64)
+    _, r64 = rank_both(G, G.gbr_comb_create(M, N, R), to_dev_u64(pats), check=1)
+    assert np.array_equal(r64, u)
+
+
 @pytest.mark.parametrize("n", [0, 1, 7, 1023, 1024, 1025, 4097, 100003])
 def test_comb_ragged_lengths(G, n):
     import torch
