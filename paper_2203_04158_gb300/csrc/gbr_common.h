@@ -118,7 +118,7 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
 struct gbr_comb {
     gbr::StagDesc desc;
     gbr::DevBuf table;      // entries (uint32 or uint64)
-    gbr::DevBuf binom;      // 65 x 65 uint64 binomials (unranking)
+    gbr::DevBuf binom;      // 65 x 65 uint64 binomials, then the low patterns by popcount (unranking)
     uint64_t dim;
 };
 

@@ -94,6 +94,33 @@ def test_comb_rank_sums_beyond_32_bits(G, M, N, R):
     assert np.array_equal(r64, u)
 
 
+@pytest.mark.parametrize("M", [13, 14, 15, 31, 32, 33, 34, 35, 36, 63])
+@pytest.mark.parametrize("part", [0, 1, 3, 2])
+def test_comb_unrank_around_its_switches(G, M, part):
+    """Unranking looks the last 14 positions up and computes in 64 bits above
+    position 34: sectors around both, empty to half filled, in both index
+    widths, a ragged count over several tiles, first and last index."""
+    import torch
+    N = 0 if part == 0 else max(1, M * part // 4 if part > 1 else M - 1)
+    D = math.comb(M, N)
+    n = 2048 * 3 + 5
+    u = S.bounded(13, np.arange(n, dtype=np.uint64), D)
+    u[:4] = [0, D - 1, D // 2, D // 3]
+    c = G.gbr_comb_create(M, N, 8)
+    outs = []
+    for dt in (np.int64, np.int32)[:2 if D < 2**32 else 1]:
+        r = torch.from_numpy(u.astype(np.uint32).view(np.int32) if dt is np.int32 else u.view(np.int64)).cuda()
+        pats = torch.empty(n, dtype=torch.int64, device="cuda")
+        G.gbr_comb_unrank(c, r, pats)
+        outs.append(as_u64(pats))
+    for p in outs:
+        for ui, a in zip(u[:300], p[:300]):
+            assert int(a) == oracle.unrank(M, N, int(ui)), (M, N, int(ui))
+        assert np.array_equal(p, outs[0])
+    _, r64 = rank_both(G, c, to_dev_u64(outs[0]), check=1)
+    assert np.array_equal(r64, u)
+
+
 @pytest.mark.parametrize("n", [0, 1, 7, 1023, 1024, 1025, 4097, 100003])
 def test_comb_ragged_lengths(G, n):
     import torch
