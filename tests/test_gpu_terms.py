@@ -96,3 +96,32 @@ def test_open_set_projection_and_radices(G):
         y, x, _ = run(G, 2 * L, terms, sub, R=R)
         y_ref, drop = oracle.hv_ops(terms, sub, x)
         assert drop > 0 and rel_inf(y, y_ref) <= TOL64
+
+
+def _ladder_terms(M, count, seed):
+    """`count` hops and pair hops between random orbitals, diagonal ones among them."""
+    rng = np.random.default_rng(seed)
+    out = []
+    for _ in range(count):
+        p, q = (int(o) for o in rng.integers(0, M, 2))
+        if rng.random() < 0.5 or M < 6:
+            out.append((float(rng.uniform(-1, 1)), [2 * p + 1, 2 * q]))
+        else:
+            a, b, c, d = (int(o) for o in rng.choice(M, 4, replace=False))
+            out.append((float(rng.uniform(-1, 1)), [2 * a + 1, 2 * b + 1, 2 * c, 2 * d]))
+    return out
+
+
+@pytest.mark.parametrize("nterms", [1, 31, 127, 128, 129, 300])
+@pytest.mark.parametrize("M,N", [(5, 2), (16, 6), (16, 7), (33, 2), (64, 2)])
+def test_term_tiles_and_members_per_warp(G, M, N, nterms):
+    """Term counts around the tiles of 128, member counts on both sides of the
+    switch between one and four members a warp (8,008 and 11,440 against 64 a
+    multiprocessor) with ragged ends, and both mask widths."""
+    st = oracle.enumerate_sector(M, N) if M < 20 else np.array(
+        sorted((1 << a) | (1 << b) for a in range(0, M, 4) for b in range(a)), dtype=np.uint64)
+    terms = _ladder_terms(M, nterms, 100 * M + nterms)
+    for fp in (64, 32):
+        y, x, _ = run(G, M, terms, st, fp=fp)
+        y_ref, _ = oracle.hv_ops(terms, st, x)
+        assert rel_inf(y, y_ref) <= (TOL64 if fp == 64 else TOL32), (M, N, nterms, fp)
