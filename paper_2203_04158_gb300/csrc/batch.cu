@@ -158,8 +158,13 @@ __device__ void hv_small(const SectorDesc &sd, int hmax, const SpinLists &up, co
 
 struct BatchSmem {
     int maxD, maxDs, hmax, iters;
+    int tri_smem;      // 1: the tridiagonal solver's arrays in shared memory (short recurrences)
     int64_t slot;      // doubles of global scratch per CTA: x, Hx (maxD each), solver work 3 (iters + 2)
 };
+// Longest recurrence whose solver arrays (12 KiB) go to shared memory: the
+// solver's chains read one entry a step, which from L2 costs several times the
+// arithmetic of the step.
+constexpr int kBatchTriSmem = 512;
 
 // xg: per-CTA scratch of lay.slot doubles for the FP64 Ritz vector, its H·v
 // and the tridiagonal solver's work (global memory; each CTA reuses its own
@@ -193,7 +198,8 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
     double *alpha = (double *)take((size_t)(kmax + 2) * 8);
     double *beta = (double *)take((size_t)(kmax + 2) * 8);
     double *svec = (double *)take((size_t)(kmax + 2) * 8);
-    double *work = xg + (size_t)blockIdx.x * lay.slot + 2 * (size_t)maxD;   // 3 (kmax + 2) doubles
+    // 3 (kmax + 2) doubles
+    double *work = lay.tri_smem ? (double *)take((size_t)(kmax + 2) * 24) : xg + (size_t)blockIdx.x * lay.slot + 2 * (size_t)maxD;
     __shared__ double red[NT / 32];
     __shared__ double hs[kBatchMaxL * kBatchMaxL];
     __shared__ double bc64[kBatchMaxL * kBatchMaxL];
@@ -329,35 +335,41 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
                         }
                         __syncthreads();
                         if (!conv_s && kdone == next_check && k + 1 < Kc) {
-                            // residual estimate from the last eigenvector component alone
-                            const double lam = tridiag_lowest_warm(alpha, beta, kdone, &lam_hint, &gap_hint);
-                            if (threadIdx.x == 0) {
+                            // residual estimate from the last eigenvector component alone; one warp
+                            if (threadIdx.x < 32) {
+                                const Tri t = tri_stage(alpha, beta, kdone, scale, work);
+                                const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint);
                                 const double thr = 1e-6 * scale;
-                                const double r = b * tridiag_last_component(alpha, beta, kdone, lam, work);
-                                if (r <= thr) {
-                                    conv_s = 1;
-                                } else {
-                                    // next test at half the distance the geometric decrease since
-                                    // the last test predicts, 4 to 16 steps ahead
-                                    int gap = 4;
-                                    if (r_last > 0.0 && r < r_last) {
-                                        const double per_step = log(r / r_last) / (double)(kdone - k_last);
-                                        const double steps = log(thr / r) / per_step;
-                                        gap = 4 * max(1, min(4, (int)(0.5 * steps / 4.0)));
+                                const double r = b * tri_last_component(t, lam);
+                                if (threadIdx.x == 0) {
+                                    if (r <= thr) {
+                                        conv_s = 1;
+                                    } else {
+                                        // next test at half the distance the geometric decrease since
+                                        // the last test predicts, 4 to 16 steps ahead
+                                        int gap = 4;
+                                        if (r_last > 0.0 && r < r_last) {
+                                            const double per_step = log(r / r_last) / (double)(kdone - k_last);
+                                            const double steps = log(thr / r) / per_step;
+                                            gap = 4 * max(1, min(4, (int)(0.5 * steps / 4.0)));
+                                        }
+                                        next_check = kdone + gap;
+                                        r_last = r;
+                                        k_last = kdone;
                                     }
-                                    next_check = kdone + gap;
-                                    r_last = r;
-                                    k_last = kdone;
                                 }
                             }
                             __syncthreads();
                         }
                         if (conv_s || k + 1 >= Kc) {
                             // the Ritz pair of the final T for the second pass
-                            const double lam = tridiag_lowest_warm(alpha, beta, kdone, &lam_hint, &gap_hint);
-                            if (threadIdx.x == 0) {
-                                tridiag_vector_thread(alpha, beta, kdone, lam, svec, work);
-                                if (b * fabs(svec[kdone - 1]) <= 1e-6 * scale) conv_s = 1;
+                            if (threadIdx.x < 32) {
+                                const Tri t = tri_stage(alpha, beta, kdone, scale, work);
+                                const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint) / t.unit;
+                                if (threadIdx.x == 0) {
+                                    tridiag_vector_thread(alpha, beta, kdone, lam, svec, work);
+                                    if (b * fabs(svec[kdone - 1]) <= 1e-6 * scale) conv_s = 1;
+                                }
                             }
                             __syncthreads();
                             break;
@@ -485,17 +497,18 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
             for (int q = 0; q < L; ++q)
                 if (p != q && models[m].h[p * L + q] != 0.0) ++nb;
         if (nb > 0x7FFF) return set_error(GBR_EINVAL, "too many bonds");
-        // largest hop count of any per-spin state: N (L - N) bounds it
-        for (int N = 0; N <= L; ++N) hmax = std::max(hmax, N * (L - N));
+        // largest hop count of any per-spin state: N (L - N) bounds it, and so do the
+        // bonds, each of which lets at most one of its ends hop
+        for (int N = 0; N <= L; ++N) hmax = std::max(hmax, std::min(N * (L - N), nb / 2));
         maxDs = std::max<int>(maxDs, (int)binom(L, L / 2));
     }
     for (const SectorDesc &s : secs) maxD = std::max(maxD, s.Dup * s.Ddn);
     const int K = std::min(iters, maxD);
-    BatchSmem lay{maxD, maxDs, hmax, K, 2 * (int64_t)maxD + 3 * (int64_t)(K + 2)};
+    BatchSmem lay{maxD, maxDs, hmax, K, K <= kBatchTriSmem ? 1 : 0, 2 * (int64_t)maxD + 3 * (int64_t)(K + 2)};
     auto r16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
     size_t smem = 3 * r16((size_t)maxD * 4) + 2 * r16((size_t)maxDs * 4) +
                   2 * r16((size_t)maxDs) + 2 * r16((size_t)maxDs * hmax * 4) + 2 * r16((size_t)maxDs * 4) +
-                  3 * r16((size_t)(K + 2) * 8);
+                  3 * r16((size_t)(K + 2) * 8) + (lay.tri_smem ? r16((size_t)(K + 2) * 24) : 0);
     int dev = 0, optin = 0;
     GBR_CUDA_TRY(cudaGetDevice(&dev));
     GBR_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));

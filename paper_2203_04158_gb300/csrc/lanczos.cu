@@ -337,68 +337,91 @@ __global__ void __launch_bounds__(kRedThreads) k_multiaxpy(const LzState *st, T 
     }
 }
 
-// per-step and final tridiagonal solves share the device routine of tridiag.cuh
+// per-step and final tridiagonal solves share the device routines of tridiag.cuh
 #include "tridiag.cuh"
 
-__global__ void __launch_bounds__(kRedThreads) k_tridiag(const LzState *st, const double *alpha, const double *beta,
-                                                         int kfixed, double *out, double *s, double *work) {
-    const int k = kfixed > 0 ? kfixed : (st->k + 1);
-    const double lam = tridiag_lowest_block(alpha, beta, k);
-    if (threadIdx.x == 0) {
-        out[0] = lam;
-        if (s) tridiag_vector_thread(alpha, beta, k, lam, s, work);
-    }
+// Largest T whose scaled copy (3 doubles a row) a tridiagonal kernel keeps in
+// shared memory; longer ones go to the global work array.
+constexpr int kTriSmemRows = 2000;
+static size_t tri_smem(int rows) { return rows <= kTriSmemRows ? (size_t)rows * 24 : 0; }
+
+// lowest eigenvalue of T_{k+1} of the current step into ritz[k]; one warp
+__global__ void __launch_bounds__(32) k_step_ritz(const LzState *st, const double *alpha, const double *beta, double *work,
+                                                  int in_smem, double *ritz) {
+    extern __shared__ __align__(16) double tri_sm[];
+    const int k = st->k + 1;
+    const Tri t = tri_stage(alpha, beta, k, st->scale, in_smem ? tri_sm : work);
+    const double lam = tri_lowest(t) / t.unit;
+    if (threadIdx.x == 0) ritz[st->k] = lam;
 }
 
 // Convergence test every 8 steps (after beta_{k+1} is known): residual
 // estimate of the lowest Ritz pair, beta_{k+1} |s_k|, against tol * scale.
-// One warp does the eigenvalue search (warm-started from the previous test);
-// thread 0 the last eigenvector component.
+// One warp, its search warm-started from the previous test.
 __global__ void __launch_bounds__(32) k_conv_check(LzState *st, const double *alpha, const double *beta, double tol,
-                                                   double *work) {
+                                                   double *work, int in_smem) {
+    extern __shared__ __align__(16) double tri_sm[];
     const int k = st->k + 1;
     if (st->converged || (k % 8) != 0) return;
-    const double lam = tridiag_lowest_warm(alpha, beta, k, &st->lam_hint, &st->gap_hint);
-    if (threadIdx.x == 0) {
-        const double res = beta[k] * tridiag_last_component(alpha, beta, k, lam, work);
-        if (res <= tol * st->scale) {
-            st->stop = 1;
-            st->converged = 1;
-        }
+    const Tri t = tri_stage(alpha, beta, k, st->scale, in_smem ? tri_sm : work);
+    const double lam = tri_lowest_warm(t, &st->lam_hint, &st->gap_hint);
+    const double res = beta[k] * tri_last_component(t, lam);
+    if (threadIdx.x == 0 && res <= tol * st->scale) {
+        st->stop = 1;
+        st->converged = 1;
     }
 }
 
-// The prefix of the recurrence whose Ritz vector the refinement forms: the
-// shortest T_k (k = 8, 16, ... below kdone) whose lowest Ritz pair has the
-// residual estimate beta_{k+1} |s_k| <= u * max_j(|alpha_j|, beta_j), u the
-// unit roundoff of the vectors' precision; kdone if there is none.  A run
-// without re-orthogonalisation that goes on past that point grows copies of
+__global__ void __launch_bounds__(32) k_tri_stage(const LzState *st, const double *alpha, const double *beta, int k,
+                                                  double *work) {
+    tri_stage(alpha, beta, k, st->scale, work);
+}
+
+// Lowest Ritz value of the whole T_kdone (block gridDim.x - 1, into out[0]) and, for
+// the refinement, the prefix of the recurrence whose Ritz vector it forms: the
+// shortest T_k (k = 8, 16, ... below kdone; block k / 8 - 1) whose lowest Ritz pair has
+// the residual estimate beta_{k+1} |s_k| <= u * max_j(|alpha_j|, beta_j), u the
+// unit roundoff of the vectors' precision (*kout, the smallest by atomicMin).
+// A run without re-orthogonalisation that goes on past that point grows copies of
 // the converged state in T, and the Ritz vector of the longer T loses
 // accuracy, while the stored vectors cannot make it more accurate than at
-// that prefix.  One warp; *kout receives the prefix length.
+// that prefix.  One warp a block; the candidates are independent, so they run side
+// by side (one after the other, warm-started and through pivots, they took 2.0 ms of
+// the 8-site ring's 100-step solve).  lam[c]: candidate c's eigenvalue.
 __global__ void __launch_bounds__(32) k_ritz_prefix(const LzState *st, const double *alpha, const double *beta,
-                                                    int kdone, double u, double *work, int *kout) {
-    __shared__ double lam_prev, gap;
-    __shared__ int found;
-    if (threadIdx.x == 0) {
-        lam_prev = 0.0;
-        gap = 0.0;
-        found = kdone;
-    }
-    __syncthreads();
-    const double thr = u * st->scale;
-    for (int k = 8; k < kdone; k += 8) {
-        const double lam = tridiag_lowest_warm(alpha, beta, k, &lam_prev, &gap);
-        if (threadIdx.x == 0 && beta[k] * tridiag_last_component(alpha, beta, k, lam, work) <= thr) found = k;
-        __syncthreads();
-        if (found != kdone) break;
-    }
-    if (threadIdx.x == 0) *kout = found;
+                                                    int kdone, double u, double *work, int in_smem, double *lam,
+                                                    double *out, int *kout) {
+    extern __shared__ __align__(16) double tri_sm[];
+    const bool whole = blockIdx.x + 1 == gridDim.x;
+    const int k = whole ? kdone : 8 * ((int)blockIdx.x + 1);
+    // too long for shared memory: k_tri_stage has left T_kdone's arrays in work, of
+    // which T_k's are the leading parts
+    const Tri t = in_smem ? tri_stage(alpha, beta, k, st->scale, tri_sm)
+                          : Tri{work, work + kdone, work + 2 * (int64_t)kdone, k, tri_unit(st->scale)};
+    const double l = tri_lowest(t);
+    const double res = whole ? 0.0 : beta[k] * tri_last_component(t, l);
+    if (threadIdx.x != 0) return;
+    lam[blockIdx.x] = l / t.unit;
+    if (whole) out[0] = l / t.unit;
+    else if (res <= u * st->scale) atomicMin(kout, k);
 }
 
-// per-step Ritz value into ritz[k]
-__global__ void k_copy_ritz(const LzState *st, const double *val, double *ritz) {
-    if (threadIdx.x == 0) ritz[st->k] = val[0];
+// eigenvector s of T_k for the eigenvalue *lam
+__global__ void __launch_bounds__(32) k_ritz_vector(const double *alpha, const double *beta, int k, const double *lam,
+                                                    double *s, double *work, int in_smem) {
+    extern __shared__ __align__(16) double tri_sm[];
+    if (in_smem) {
+        // alpha, beta and the two work arrays
+        double *a = tri_sm, *b = tri_sm + k;
+        for (int i = threadIdx.x; i < k; i += 32) {
+            a[i] = alpha[i];
+            b[i] = beta[i];
+        }
+        __syncwarp();
+        if (threadIdx.x == 0) tridiag_vector_thread(a, b, k, *lam, s, tri_sm + 2 * k);
+    } else if (threadIdx.x == 0) {
+        tridiag_vector_thread(alpha, beta, k, *lam, s, work);
+    }
 }
 
 // x (FP64) = sum_j s_j v_j = sum_j (s_j / g_j) u_j over the stored
@@ -743,14 +766,14 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
     }
     if (!pass2) finalize(nparts2, 1);
     if (z.tol > 0.0 && !pass2) {
-        k_conv_check<<<1, 32, 0, z.st>>>(st, z.alpha.as<double>(), z.beta.as<double>(), z.tol, z.work.as<double>());
+        k_conv_check<<<1, 32, tri_smem(z.iters), z.st>>>(st, z.alpha.as<double>(), z.beta.as<double>(), z.tol,
+                                                         z.work.as<double>(), z.iters <= kTriSmemRows);
         ++nk;
     }
     if (want_ritz) {
-        k_tridiag<<<1, kRedThreads, 0, z.st>>>(st, z.alpha.as<double>(), z.beta.as<double>(), 0, z.tri.as<double>(),
-                                               nullptr, nullptr);
-        k_copy_ritz<<<1, 32, 0, z.st>>>(st, z.tri.as<double>(), z.ritz_tmp.as<double>());
-        nk += 2;
+        k_step_ritz<<<1, 32, tri_smem(z.iters), z.st>>>(st, z.alpha.as<double>(), z.beta.as<double>(), z.work.as<double>(),
+                                                        z.iters <= kTriSmemRows, z.ritz_tmp.as<double>());
+        ++nk;
     }
     k_advance<<<1, 32, 0, z.st>>>(st);
     nk += 1;
@@ -866,15 +889,28 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
     res->breakdown = hs.breakdown;
     res->converged = hs.converged;
     res->stored_basis = z.store;
-    // lowest Ritz value of T_kdone
-    double *tri = z.tri.as<double>();
-    k_tridiag<<<1, kRedThreads, 0, s>>>(z.state.as<LzState>(), z.alpha.as<double>(), z.beta.as<double>(), kdone, tri,
-                                       nullptr, z.work.as<double>());
+    // lowest Ritz value of T_kdone and (refinement) the converged prefix T_kr
+    double *tri = z.tri.as<double>(), *lam = z.coef.as<double>();
+    int *kbuf = reinterpret_cast<int *>(tri + 1);
+    const double unit = sizeof(T) == 4 ? 5.9604644775390625e-8 : 1.1102230246251565e-16;
+    const int ncand = o->refine ? (kdone - 1) / 8 + 1 : 1;   // k = 8, 16, ... below kdone, then kdone
+    GBR_CUDA_TRY(cudaMemsetAsync(kbuf, 0x7F, sizeof(int), s));
+    if (kdone > kTriSmemRows) {
+        k_tri_stage<<<1, 32, 0, s>>>(z.state.as<LzState>(), z.alpha.as<double>(), z.beta.as<double>(), kdone,
+                                     z.work.as<double>());
+        count_launches(1);
+    }
+    k_ritz_prefix<<<ncand, 32, tri_smem(kdone), s>>>(z.state.as<LzState>(), z.alpha.as<double>(), z.beta.as<double>(), kdone,
+                                                     unit, z.work.as<double>(), kdone <= kTriSmemRows, lam, tri, kbuf);
     GBR_LAUNCH_CHECK();
     count_launches(1);
-    double Er = 0.0;
-    GBR_CUDA_TRY(cudaMemcpyAsync(&Er, tri, 8, cudaMemcpyDeviceToHost, s));
+    double et[2];
+    GBR_CUDA_TRY(cudaMemcpyAsync(et, tri, sizeof(et), cudaMemcpyDeviceToHost, s));
     GBR_CUDA_TRY(cudaStreamSynchronize(s));
+    const double Er = et[0];
+    int kr = 0;
+    memcpy(&kr, et + 1, sizeof(int));
+    if (kr < 1 || kr > kdone) kr = kdone;
     res->E_ritz = Er;
     res->E0 = Er;
     res->residual = -1.0;
@@ -883,18 +919,11 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
         if ((rc = grow(x, (size_t)n * 8))) return rc;
         if ((rc = grow(hx, (size_t)n * 8))) return rc;
         double *sv = z.svec.as<double>();
-        // the Ritz vector of the converged prefix T_kr, then its eigenvector s
-        int *kbuf = reinterpret_cast<int *>(tri + 8);
-        const double unit = sizeof(T) == 4 ? 5.9604644775390625e-8 : 1.1102230246251565e-16;
-        k_ritz_prefix<<<1, 32, 0, s>>>(z.state.as<LzState>(), z.alpha.as<double>(), z.beta.as<double>(), kdone, unit,
-                                       z.work.as<double>(), kbuf);
-        int kr = kdone;
-        GBR_CUDA_TRY(cudaMemcpyAsync(&kr, kbuf, sizeof(int), cudaMemcpyDeviceToHost, s));
-        GBR_CUDA_TRY(cudaStreamSynchronize(s));
-        if (kr < 1 || kr > kdone) kr = kdone;
-        k_tridiag<<<1, kRedThreads, 0, s>>>(z.state.as<LzState>(), z.alpha.as<double>(), z.beta.as<double>(), kr,
-                                           tri + 4, sv, z.work.as<double>());
-        count_launches(2);
+        const bool vsm = 4 * kr <= 3 * kTriSmemRows;
+        k_ritz_vector<<<1, 32, vsm ? (size_t)kr * 32 : 0, s>>>(z.alpha.as<double>(), z.beta.as<double>(), kr,
+                                                             lam + (kr == kdone ? ncand - 1 : kr / 8 - 1), sv,
+                                                             z.work.as<double>(), vsm);
+        count_launches(1);
         GBR_LAUNCH_CHECK();
         // terms of the Ritz sum: drop the trailing coefficients whose norm is
         // at most ritz_tail (s is normalised by the tridiagonal solver)
