@@ -35,16 +35,33 @@ struct ModelDev {
     double U[kBatchMaxL];
 };
 
-__device__ __forceinline__ double bsum(double v, double *red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
+// Sum over the block of the threads' two-float sums, in FP64 by the first warp
+// alone (valid in its threads): the FP64 pipe takes 16 clocks of the whole
+// multiprocessor for every warp instruction, so every warp doing its own
+// shuffles and the final sum (and square roots and the like after it) cost 6,600
+// clocks of that pipe a Lanczos step, more than the step's vector work.  red: one float2
+// per thread.  Ends with the sum in registers of warp 0 and no barrier behind it.
+__device__ __forceinline__ double bsum0(float hi, float lo, float2 *red) {
+    red[threadIdx.x] = make_float2(hi, lo);
     __syncthreads();
     double r = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += red[i];
+    if (threadIdx.x < 32) {
+        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) r += (double)red[i].x + (double)red[i].y;
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
+    }
+    return r;
+}
+
+// the same for FP64 values (the final Rayleigh quotient); red: one double per thread
+__device__ __forceinline__ double bsum0(double v, double *red) {
+    red[threadIdx.x] = v;
     __syncthreads();
-    return r;   // all threads
+    double r = 0.0;
+    if (threadIdx.x < 32) {
+        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) r += red[i];
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
+    }
+    return r;
 }
 
 __device__ __forceinline__ void ffp(float &hi, float &lo, float a, float b) {
@@ -126,34 +143,33 @@ __device__ __forceinline__ double diag64(uint32_t a, const double *h, int L) {
     return d;
 }
 
-// y = H x on the sector, one element per thread iteration (hs: the L x L
-// one-body matrix, for the FP64 diagonal)
+// (H x)_i of element i = (ru, rd), x in shared or global memory (hs: the L x L
+// one-body matrix, for the FP64 diagonal; umask: sites with U != 0)
 template <typename T>
-__device__ void hv_small(const SectorDesc &sd, int hmax, const SpinLists &up, const SpinLists &dn, const T *bc,
-                         const T *U, const double *hs, const T *x, T *y) {
-    const int D = sd.Dup * sd.Ddn;
-    for (int i = threadIdx.x; i < D; i += blockDim.x) {
-        const int ru = i / sd.Ddn, rd = i - ru * sd.Ddn;
-        const uint32_t au = up.st[ru], ad = dn.st[rd];
-        T dg = (sizeof(T) == 8) ? (T)(diag64(au, hs, sd.L) + diag64(ad, hs, sd.L)) : (T)(up.d32[ru] + dn.d32[rd]);
-        const uint32_t both = au & ad;
-        for (int p = 0; p < sd.L; ++p)
-            if ((both >> p) & 1u) dg += U[p];
-        T acc = dg * x[i];
-        for (int k = 0; k < up.cnt[ru]; ++k) {
-            const uint32_t e = up.ent[ru * hmax + k];
-            const T c = bc[(e >> 16) & 0x7FFFu];
-            const T v = x[(int)(e & 0xFFFFu) * sd.Ddn + rd];
-            acc += (e >> 31) ? -c * v : c * v;
-        }
-        for (int k = 0; k < dn.cnt[rd]; ++k) {
-            const uint32_t e = dn.ent[rd * hmax + k];
-            const T c = bc[(e >> 16) & 0x7FFFu];
-            const T v = x[ru * sd.Ddn + (int)(e & 0xFFFFu)];
-            acc += (e >> 31) ? -c * v : c * v;
-        }
-        y[i] = acc;
+__device__ __forceinline__ T hv_small(const SectorDesc &sd, int hmax, const SpinLists &up, const SpinLists &dn, const T *bc,
+                                      const T *U, uint32_t umask, const double *hs, const T *x, int ru, int rd) {
+    const uint32_t au = up.st[ru], ad = dn.st[rd];
+    T dg = (sizeof(T) == 8) ? (T)(diag64(au, hs, sd.L) + diag64(ad, hs, sd.L)) : (T)(up.d32[ru] + dn.d32[rd]);
+    uint32_t both = au & ad & umask;
+    while (both) {
+        dg += U[__ffs(both) - 1];
+        both &= both - 1u;
     }
+    const T *row = x + ru * sd.Ddn, *col = x + rd;
+    T acc = dg * row[rd];
+    const uint32_t *e = up.ent + ru * hmax;
+    int n = up.cnt[ru];
+    for (int k = 0; k < n; ++k) {
+        const T c = bc[(e[k] >> 16) & 0x7FFFu], v = col[(int)(e[k] & 0xFFFFu) * sd.Ddn];
+        acc += (e[k] >> 31) ? -c * v : c * v;
+    }
+    e = dn.ent + rd * hmax;
+    n = dn.cnt[rd];
+    for (int k = 0; k < n; ++k) {
+        const T c = bc[(e[k] >> 16) & 0x7FFFu], v = row[e[k] & 0xFFFFu];
+        acc += (e[k] >> 31) ? -c * v : c * v;
+    }
+    return acc;
 }
 
 struct BatchSmem {
@@ -165,6 +181,10 @@ struct BatchSmem {
 // solver's chains read one entry a step, which from L2 costs several times the
 // arithmetic of the step.
 constexpr int kBatchTriSmem = 512;
+__host__ __device__ __forceinline__ size_t batch_scratch(int threads, int iters, int tri_smem) {
+    const size_t r = (size_t)threads * 8, t = tri_smem ? (size_t)(iters + 2) * 24 : 0;
+    return r > t ? r : t;
+}
 
 // xg: per-CTA scratch of lay.slot doubles for the FP64 Ritz vector, its H·v
 // and the tridiagonal solver's work (global memory; each CTA reuses its own
@@ -198,9 +218,11 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
     double *alpha = (double *)take((size_t)(kmax + 2) * 8);
     double *beta = (double *)take((size_t)(kmax + 2) * 8);
     double *svec = (double *)take((size_t)(kmax + 2) * 8);
-    // 3 (kmax + 2) doubles
-    double *work = lay.tri_smem ? (double *)take((size_t)(kmax + 2) * 24) : xg + (size_t)blockIdx.x * lay.slot + 2 * (size_t)maxD;
-    __shared__ double red[NT / 32];
+    // reduction slots (one double or float2 per thread) and, for short recurrences, the
+    // solver's 3 (kmax + 2) doubles in the same place: both are warp 0's between barriers
+    double *red = (double *)take(batch_scratch(NT, kmax, lay.tri_smem));
+    double *work = lay.tri_smem ? red : xg + (size_t)blockIdx.x * lay.slot + 2 * (size_t)maxD;
+    __shared__ uint32_t umask_s;
     __shared__ double hs[kBatchMaxL * kBatchMaxL];
     __shared__ double bc64[kBatchMaxL * kBatchMaxL];
     __shared__ float bc32[kBatchMaxL * kBatchMaxL];
@@ -230,6 +252,9 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
         for (int i = threadIdx.x; i < L; i += blockDim.x) { U64[i] = m.U[i]; U32[i] = (float)m.U[i]; }
         __syncthreads();
         if (threadIdx.x == 0) {
+            uint32_t um = 0;
+            for (int a = 0; a < L; ++a) um |= U64[a] != 0.0 ? 1u << a : 0u;
+            umask_s = um;
             int nb = 0;
             for (int a = 0; a < L; ++a)
                 for (int b = 0; b < L; ++b)
@@ -256,149 +281,169 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
         // (at most three cycles).  Each cycle runs the recurrence twice: once
         // for the scalars, once more (bit identical) to accumulate the Ritz
         // vector x in FP64.
-        __shared__ int conv_s;
+        __shared__ int conv_s, end_s;
         __shared__ double lam_hint, gap_hint;   // warm start of the convergence test's eigenvalue search
-        __shared__ int next_check, k_last;       // step of the next test; step and residual of the last one
-        __shared__ double r_last;
-        int kdone = 0;
+        __shared__ double inv_n0;
+        __shared__ float ak_s, bk_s, inv_s;     // alpha_k, beta_{k+1} and 1 / beta_{k+1} of the step
+        __shared__ int kdone;
+        // this thread's elements i = threadIdx.x + j NT as (ru, rd)
+        const int dru = NT / sd.Ddn, drd = NT - dru * sd.Ddn;
+        const int ru0 = (int)threadIdx.x / sd.Ddn, rd0 = (int)threadIdx.x - ru0 * sd.Ddn;
+        const uint32_t umask = umask_s;
+        auto next = [&](int &ru, int &rd) {
+            ru += dru;
+            rd += drd;
+            if (rd >= sd.Ddn) {
+                rd -= sd.Ddn;
+                ++ru;
+            }
+        };
         for (int cyc = 0; cyc < 3; ++cyc) {
             if (cyc > 0) {
-                for (int i = threadIdx.x; i < D; i += blockDim.x) hx[i] = x[i];
+                for (int i = threadIdx.x; i < D; i += NT) hx[i] = x[i];
                 __syncthreads();
             }
-            const int Kc = K;
+            auto source = [&](int i) { return (float)(cyc == 0 ? start[sd.off + i] : hx[i]); };
             float fh = 0.f, fl = 0.f;
-            for (int i = threadIdx.x; i < D; i += blockDim.x) {
-                const float s = (float)(cyc == 0 ? start[sd.off + i] : hx[i]);
-                ffp(fh, fl, s, s);
+            for (int i = threadIdx.x; i < D; i += NT) {
+                const float f = source(i);
+                ffp(fh, fl, f, f);
             }
-            const double n0 = sqrt(bsum((double)fh + (double)fl, red));
-            double scale = 0.0;
-            kdone = 0;
+            const double n2 = bsum0(fh, fl, reinterpret_cast<float2 *>(red));
             if (threadIdx.x == 0) {
+                inv_n0 = 1.0 / sqrt(n2);
                 conv_s = 0;
+                end_s = 0;
                 lam_hint = 0.0;
                 gap_hint = 0.0;
-                next_check = 4;
-                k_last = 0;
-                r_last = 0.0;
             }
             __syncthreads();
-            for (int pass = 0; pass < 2; ++pass) {
-                for (int i = threadIdx.x; i < D; i += blockDim.x) {
-                    const float s = (float)(cyc == 0 ? start[sd.off + i] : hx[i]);
-                    v[i] = (float)((double)s / n0);
-                    vp[i] = 0.f;
+            // the first run: scalars
+            for (int i = threadIdx.x; i < D; i += NT) v[i] = (float)((double)source(i) * inv_n0);
+            __syncthreads();
+            // warp 0's: step of the next test, step and residual of the last one
+            int next_check = 4, k_last = 0;
+            double r_last = 0.0, scale = 0.0;
+            for (int k = 0; k < K; ++k) {
+                const float bk = bk_s;   // beta_k (k > 0)
+                float ah = 0.f, al = 0.f;
+                for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
+                    float wi = hv_small<float>(sd, hmax, up, dn, bc32, U32, umask, hs, v, ru, rd);
+                    if (k) wi = __fmaf_rn(-bk, vp[i], wi);
+                    w[i] = wi;
+                    ffp(ah, al, wi, v[i]);
+                }
+                const double a = bsum0(ah, al, reinterpret_cast<float2 *>(red));
+                if (threadIdx.x == 0) {
+                    alpha[k] = a;
+                    ak_s = (float)a;
+                }
+                scale = fmax(scale, fabs(a));
+                __syncthreads();
+                const float ak = ak_s;
+                float bh = 0.f, bl = 0.f;
+                for (int i = threadIdx.x; i < D; i += NT) {
+                    const float wi = __fmaf_rn(-ak, v[i], w[i]);
+                    w[i] = wi;
+                    ffp(bh, bl, wi, wi);
+                }
+                const double b2 = bsum0(bh, bl, reinterpret_cast<float2 *>(red));
+                if (threadIdx.x < 32) {
+                    const double b = sqrt(fmax(b2, 0.0));
+                    const int kd = k + 1;
+                    scale = fmax(scale, b);
+                    bool conv = b <= 1e-13 * scale;
+                    if (threadIdx.x == 0) {
+                        beta[kd] = b;
+                        bk_s = (float)b;
+                        inv_s = 1.0f / (float)b;   // FP32: the FP64 divide is slow here
+                    }
+                    __syncwarp();
+                    if (!conv && kd == next_check && kd < K) {
+                        // residual estimate from the last eigenvector component alone
+                        const Tri t = tri_stage(alpha, beta, kd, scale, work);
+                        const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint);
+                        const double thr = 1e-6 * scale;
+                        const double r = b * tri_last_component(t, lam);
+                        if (r <= thr) {
+                            conv = true;
+                        } else {
+                            // next test at half the distance the geometric decrease since
+                            // the last test predicts, 4 to 16 steps ahead
+                            int gap = 4;
+                            if (r_last > 0.0 && r < r_last) {
+                                const double per_step = log(r / r_last) / (double)(kd - k_last);
+                                const double steps = log(thr / r) / per_step;
+                                gap = 4 * max(1, min(4, (int)(0.5 * steps / 4.0)));
+                            }
+                            next_check = kd + gap;
+                            r_last = r;
+                            k_last = kd;
+                        }
+                    }
+                    if (conv || kd >= K) {
+                        // the Ritz pair of the final T for the second run
+                        const Tri t = tri_stage(alpha, beta, kd, scale, work);
+                        const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint) / t.unit;
+                        if (threadIdx.x == 0) {
+                            tridiag_vector_thread(alpha, beta, kd, lam, svec, work);
+                            if (conv || b * fabs(svec[kd - 1]) <= 1e-6 * scale) conv_s = 1;
+                            kdone = kd;
+                            end_s = 1;
+                        }
+                    }
                 }
                 __syncthreads();
-                const int ksteps = pass == 0 ? Kc : kdone;
-                for (int k = 0; k < ksteps; ++k) {
-                    if (pass == 1) {
-                        for (int i = threadIdx.x; i < D; i += blockDim.x) x[i] = fma(svec[k], (double)v[i], k ? x[i] : 0.0);
-                        if (k + 1 == ksteps) break;
-                    }
-                    hv_small<float>(sd, hmax, up, dn, bc32, U32, hs, v, w);
-                    __syncthreads();
-                    const float bk = k ? (float)beta[k] : 0.f;
-                    float ah = 0.f, al = 0.f;
-                    for (int i = threadIdx.x; i < D; i += blockDim.x) {
-                        float wi = w[i];
-                        if (k) wi -= bk * vp[i];
-                        w[i] = wi;
-                        ffp(ah, al, wi, v[i]);
-                    }
-                    __syncthreads();
-                    if (pass == 0) {
-                        const double a = bsum((double)ah + (double)al, red);
-                        if (threadIdx.x == 0) alpha[k] = a;
-                        scale = fmax(scale, fabs(a));
-                    }
-                    __syncthreads();
-                    const float ak = (float)alpha[k];
-                    float bh = 0.f, bl = 0.f;
-                    for (int i = threadIdx.x; i < D; i += blockDim.x) {
-                        const float wi = w[i] - ak * v[i];
-                        w[i] = wi;
-                        ffp(bh, bl, wi, wi);
-                    }
-                    __syncthreads();
-                    if (pass == 0) {
-                        const double b = sqrt(fmax(bsum((double)bh + (double)bl, red), 0.0));
-                        if (threadIdx.x == 0) beta[k + 1] = b;
-                        kdone = k + 1;
-                        scale = fmax(scale, b);
-                        __syncthreads();
-                        // lowest Ritz pair of T_{k+1} and its residual estimate,
-                        // every 4 steps and at the end of the cycle
-                        if (b <= 1e-13 * scale) {
-                            if (threadIdx.x == 0) conv_s = 1;
-                        }
-                        __syncthreads();
-                        if (!conv_s && kdone == next_check && k + 1 < Kc) {
-                            // residual estimate from the last eigenvector component alone; one warp
-                            if (threadIdx.x < 32) {
-                                const Tri t = tri_stage(alpha, beta, kdone, scale, work);
-                                const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint);
-                                const double thr = 1e-6 * scale;
-                                const double r = b * tri_last_component(t, lam);
-                                if (threadIdx.x == 0) {
-                                    if (r <= thr) {
-                                        conv_s = 1;
-                                    } else {
-                                        // next test at half the distance the geometric decrease since
-                                        // the last test predicts, 4 to 16 steps ahead
-                                        int gap = 4;
-                                        if (r_last > 0.0 && r < r_last) {
-                                            const double per_step = log(r / r_last) / (double)(kdone - k_last);
-                                            const double steps = log(thr / r) / per_step;
-                                            gap = 4 * max(1, min(4, (int)(0.5 * steps / 4.0)));
-                                        }
-                                        next_check = kdone + gap;
-                                        r_last = r;
-                                        k_last = kdone;
-                                    }
-                                }
-                            }
-                            __syncthreads();
-                        }
-                        if (conv_s || k + 1 >= Kc) {
-                            // the Ritz pair of the final T for the second pass
-                            if (threadIdx.x < 32) {
-                                const Tri t = tri_stage(alpha, beta, kdone, scale, work);
-                                const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint) / t.unit;
-                                if (threadIdx.x == 0) {
-                                    tridiag_vector_thread(alpha, beta, kdone, lam, svec, work);
-                                    if (b * fabs(svec[kdone - 1]) <= 1e-6 * scale) conv_s = 1;
-                                }
-                            }
-                            __syncthreads();
-                            break;
-                        }
-                    }
-                    __syncthreads();
-                    const float inv = 1.0f / (float)beta[k + 1];   // FP32: the FP64 divide is slow here
-                    for (int i = threadIdx.x; i < D; i += blockDim.x) {
-                        const float vn = w[i] * inv;
-                        vp[i] = v[i];
-                        v[i] = vn;
-                    }
-                    __syncthreads();
-                }
+                if (end_s) break;
+                // v_{k+1} takes the place of v_{k-1}
+                const float inv = inv_s;
+                for (int i = threadIdx.x; i < D; i += NT) vp[i] = w[i] * inv;
+                float *t = vp;
+                vp = v;
+                v = t;
+                __syncthreads();
+            }
+            // the second run, one pass a step: the same vectors with the stored
+            // scalars, summed into x (the solver's arrays are free: they hold the
+            // scalars in FP32, as the first run used them)
+            float4 *sf = reinterpret_cast<float4 *>(work);
+            const int steps = kdone;
+            for (int k = threadIdx.x; k + 1 < steps; k += NT)
+                sf[k] = make_float4(k ? (float)beta[k] : 0.f, (float)alpha[k], 1.0f / (float)beta[k + 1], 0.f);
+            for (int i = threadIdx.x; i < D; i += NT) {
+                const float f = (float)((double)source(i) * inv_n0);
+                v[i] = f;
+                x[i] = svec[0] * (double)f;
             }
             __syncthreads();
+            for (int k = 0; k + 1 < steps; ++k) {
+                const float4 c = sf[k];
+                const double sk = svec[k + 1];
+                for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
+                    float wi = hv_small<float>(sd, hmax, up, dn, bc32, U32, umask, hs, v, ru, rd);
+                    if (k) wi = __fmaf_rn(-c.x, vp[i], wi);
+                    wi = __fmaf_rn(-c.y, v[i], wi) * c.z;
+                    vp[i] = wi;   // read by this thread alone
+                    x[i] = fma(sk, (double)wi, x[i]);
+                }
+                float *t = vp;
+                vp = v;
+                v = t;
+                __syncthreads();
+            }
             if (conv_s) break;
         }
         __syncthreads();
         // FP64 Rayleigh quotient of the Ritz vector
-        hv_small<double>(sd, hmax, up, dn, bc64, U64, hs, x, hx);
-        __syncthreads();
         double xhx = 0.0, xx = 0.0;
-        for (int i = threadIdx.x; i < D; i += blockDim.x) {
-            xhx = fma(x[i], hx[i], xhx);
-            xx = fma(x[i], x[i], xx);
+        for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
+            const double xi = x[i];
+            xhx = fma(xi, hv_small<double>(sd, hmax, up, dn, bc64, U64, umask, hs, x, ru, rd), xhx);
+            xx = fma(xi, xi, xx);
         }
-        const double num = bsum(xhx, red);
-        const double den = bsum(xx, red);
+        const double num = bsum0(xhx, red);
+        __syncthreads();
+        const double den = bsum0(xx, red);
         if (threadIdx.x == 0) {
             outE[si] = num / den;
             if (outK) outK[si] = kdone;
@@ -508,7 +553,7 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
     auto r16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
     size_t smem = 3 * r16((size_t)maxD * 4) + 2 * r16((size_t)maxDs * 4) +
                   2 * r16((size_t)maxDs) + 2 * r16((size_t)maxDs * hmax * 4) + 2 * r16((size_t)maxDs * 4) +
-                  3 * r16((size_t)(K + 2) * 8) + (lay.tri_smem ? r16((size_t)(K + 2) * 24) : 0);
+                  3 * r16((size_t)(K + 2) * 8) + r16(batch_scratch(threads, K, lay.tri_smem));
     int dev = 0, optin = 0;
     GBR_CUDA_TRY(cudaGetDevice(&dev));
     GBR_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));

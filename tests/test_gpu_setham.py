@@ -125,3 +125,28 @@ def test_both_trie_orders_give_the_same_bits(G, fp):
         assert torch.equal(ys[0], ys[1])
         y_ref, _ = oracle.hv_set(L, h, U, st, x.double().cpu().numpy())
         assert rel_inf(ys[1].double().cpu().numpy(), y_ref) <= (TOL64 if fp == 64 else TOL32)
+
+
+@pytest.mark.parametrize("kind", ["dense9", "wide17", "two_threads", "one_thread"])
+def test_hop_masks_and_threads_per_member(G, kind):
+    """More bonds than one 32-bit mask a thread holds (every pair of 9 sites),
+    words of 34 orbitals, and set sizes that take two and one thread a member."""
+    rng = np.random.default_rng(17)
+    if kind == "dense9":
+        L, st = 9, oracle.fixed_N_states(9, 4)
+        h = rng.uniform(-1, 1, (9, 9))
+        h = h + h.T
+    elif kind == "wide17":
+        L = 17
+        h = S.chain(17) + np.diag(np.linspace(-1, 1, 17))
+        st = np.array(sorted((1 << a) | (1 << b) for a in range(34) for b in range(a)), dtype=np.uint64)
+    else:
+        L, N = (11, 6) if kind == "two_threads" else (11, 8)
+        h, st = S.chain(11), S.popcount_states(22, N)
+        rng.shuffle(st)
+        st = np.sort(st[:st.size - 5])          # an open set with a ragged end
+    U = S.uniform_U(L, 3.0)
+    for fp in (64, 32):
+        y, x, _ = run(G, L, h, U, st, 8, 1, fp)
+        y_ref, _ = oracle.hv_set(L, h, U, st, x)
+        assert rel_inf(y, y_ref) <= (TOL64 if fp == 64 else TOL32), (kind, fp)
