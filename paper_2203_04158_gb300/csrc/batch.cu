@@ -35,33 +35,30 @@ struct ModelDev {
     double U[kBatchMaxL];
 };
 
-// Sum over the block of the threads' two-float sums, in FP64 by the first warp
-// alone (valid in its threads): the FP64 pipe takes 16 clocks of the whole
-// multiprocessor for every warp instruction, so every warp doing its own
-// shuffles and the final sum (and square roots and the like after it) cost 6,600
-// clocks of that pipe a Lanczos step, more than the step's vector work.  red: one float2
-// per thread.  Ends with the sum in registers of warp 0 and no barrier behind it.
-__device__ __forceinline__ double bsum0(float hi, float lo, float2 *red) {
-    red[threadIdx.x] = make_float2(hi, lo);
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x < 32) {
-        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) r += (double)red[i].x + (double)red[i].y;
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
-    }
-    return r;
+// A team: T consecutive threads of a CTA that solve one sector, with a named
+// barrier of their own (a warp needs none).
+template <int T> __device__ __forceinline__ void team_sync(int bar) {
+    if (T == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(T) : "memory");
 }
 
-// the same for FP64 values (the final Rayleigh quotient); red: one double per thread
-__device__ __forceinline__ double bsum0(double v, double *red) {
-    red[threadIdx.x] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x < 32) {
-        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) r += red[i];
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
+// Sum over the team in FP64, valid in the first warp.  A dependent FP64 operation
+// takes about 150 clocks on this GPU, so each warp sums its own threads (five
+// steps) and only the first warp what the others left in red; ends without a
+// barrier behind it.
+template <int T> __device__ __forceinline__ double team_sum(double v, double *red, int bar) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if (T == 32) return v;
+    const int lane = threadIdx.x & 31, w = (threadIdx.x % T) >> 5;
+    if (lane == 0) red[w] = v;
+    team_sync<T>(bar);
+    if (w == 0) {
+        v = lane < T / 32 ? red[lane] : 0.0;
+#pragma unroll
+        for (int o = T / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        v = __shfl_sync(0xFFFFFFFFu, v, 0);
     }
-    return r;
+    return v;
 }
 
 __device__ __forceinline__ void ffp(float &hi, float &lo, float a, float b) {
@@ -102,14 +99,17 @@ __device__ __forceinline__ int rank_small(uint32_t a, const uint32_t *bin) {
 struct SpinLists {
     uint32_t *st;      // states
     uint8_t *cnt;      // hops per state
-    uint32_t *ent;     // [state][hmax]: target | bond << 16 | sign << 31
+    uint32_t *ent;     // [state][hm]: offset of the target's element | (2 bond + sign) << 16
     float *d32;        // one-body diagonal (the FP64 one is summed on the fly)
+    int hm;            // stride of ent (odd: neighbouring states in different banks)
 };
 
-// builds the per-spin state list and hop lists of one spin species
-__device__ void build_spin(int L, int N, int D, int hmax, const double *h, const uint8_t *bidx, const uint32_t *bin,
-                           SpinLists s) {
-    for (int r = threadIdx.x; r < D; r += blockDim.x) {
+// builds the per-spin state list and hop lists of one spin species; mul: distance
+// in the vector between neighbouring ranks of this spin
+template <int T>
+__device__ void build_spin(int L, int N, int D, int mul, const double *h, const uint8_t *bidx, const uint32_t *bin,
+                           const SpinLists &s) {
+    for (int r = threadIdx.x % T; r < D; r += T) {
         const uint32_t a = unrank_small(L, N, r, bin);
         s.st[r] = a;
         double d = 0.0;
@@ -123,11 +123,11 @@ __device__ void build_spin(int L, int N, int D, int hmax, const double *h, const
                 const int lo = min(p, q), hi = max(p, q);
                 const uint32_t between = ((1u << hi) - 1u) & ~((1u << (lo + 1)) - 1u);
                 const uint32_t sg = (uint32_t)(__popc(a & between) & 1);
-                if (k < hmax) s.ent[r * hmax + k] = (uint32_t)rank_small(b, bin) | ((uint32_t)bidx[p * L + q] << 16) | (sg << 31);
+                if (k < s.hm) s.ent[r * s.hm + k] = (uint32_t)(rank_small(b, bin) * mul) | ((2u * bidx[p * L + q] + sg) << 16);
                 ++k;
             }
         }
-        s.cnt[r] = (uint8_t)min(k, hmax);
+        s.cnt[r] = (uint8_t)min(k, s.hm);
         s.d32[r] = (float)d;
     }
 }
@@ -144,9 +144,11 @@ __device__ __forceinline__ double diag64(uint32_t a, const double *h, int L) {
 }
 
 // (H x)_i of element i = (ru, rd), x in shared or global memory (hs: the L x L
-// one-body matrix, for the FP64 diagonal; umask: sites with U != 0)
+// one-body matrix, for the FP64 diagonal; umask: sites with U != 0; cf: the bonds'
+// coefficients with both signs).  An entry holds the target's element and the
+// signed coefficient's place, so that a hop is three loads and one FMA.
 template <typename T>
-__device__ __forceinline__ T hv_small(const SectorDesc &sd, int hmax, const SpinLists &up, const SpinLists &dn, const T *bc,
+__device__ __forceinline__ T hv_small(const SectorDesc &sd, const SpinLists &up, const SpinLists &dn, const T *cf,
                                       const T *U, uint32_t umask, const double *hs, const T *x, int ru, int rd) {
     const uint32_t au = up.st[ru], ad = dn.st[rd];
     T dg = (sizeof(T) == 8) ? (T)(diag64(au, hs, sd.L) + diag64(ad, hs, sd.L)) : (T)(up.d32[ru] + dn.d32[rd]);
@@ -157,81 +159,355 @@ __device__ __forceinline__ T hv_small(const SectorDesc &sd, int hmax, const Spin
     }
     const T *row = x + ru * sd.Ddn, *col = x + rd;
     T acc = dg * row[rd];
-    const uint32_t *e = up.ent + ru * hmax;
+    const uint32_t *e = up.ent + ru * up.hm;
     int n = up.cnt[ru];
-    for (int k = 0; k < n; ++k) {
-        const T c = bc[(e[k] >> 16) & 0x7FFFu], v = col[(int)(e[k] & 0xFFFFu) * sd.Ddn];
-        acc += (e[k] >> 31) ? -c * v : c * v;
-    }
-    e = dn.ent + rd * hmax;
+    for (int k = 0; k < n; ++k) acc += cf[e[k] >> 16] * col[e[k] & 0xFFFFu];
+    e = dn.ent + rd * dn.hm;
     n = dn.cnt[rd];
-    for (int k = 0; k < n; ++k) {
-        const T c = bc[(e[k] >> 16) & 0x7FFFu], v = row[e[k] & 0xFFFFu];
-        acc += (e[k] >> 31) ? -c * v : c * v;
-    }
+    for (int k = 0; k < n; ++k) acc += cf[e[k] >> 16] * row[e[k] & 0xFFFFu];
     return acc;
 }
 
-struct BatchSmem {
-    int maxD, maxDs, hmax, iters;
-    int tri_smem;      // 1: the tridiagonal solver's arrays in shared memory (short recurrences)
-    int64_t slot;      // doubles of global scratch per CTA: x, Hx (maxD each), solver work 3 (iters + 2)
+struct TeamVars {
+    double lam_hint, gap_hint, inv_n0;   // warm start of the convergence test's eigenvalue search; 1 / |start|
+    float ak, bk, inv;                   // alpha_k, beta_{k+1} and 1 / beta_{k+1} of the step
+    int cur, conv, end, kdone;
+    uint32_t umask;                      // sites with U != 0
 };
+
 // Longest recurrence whose solver arrays (12 KiB) go to shared memory: the
 // solver's chains read one entry a step, which from L2 costs several times the
 // arithmetic of the step.
 constexpr int kBatchTriSmem = 512;
-__host__ __device__ __forceinline__ size_t batch_scratch(int threads, int iters, int tri_smem) {
-    const size_t r = (size_t)threads * 8, t = tri_smem ? (size_t)(iters + 2) * 24 : 0;
-    return r > t ? r : t;
+
+// A team's shared memory for one sector (host and device lay it out alike).
+struct TeamLay {
+    int v, vp, w, st_up, st_dn, cnt_up, cnt_dn, ent_up, ent_dn, d_up, d_dn, alpha, beta, svec, scratch, hs, cf64, cf32, U64,
+        U32, bidx, bytes;
+    int hm_up, hm_dn;
+};
+__host__ __device__ inline TeamLay team_lay(const SectorDesc &sd, int T, int hmax, int nb, int iters, int tri_smem) {
+    TeamLay l;
+    int at = (int)((sizeof(TeamVars) + 15) & ~(size_t)15);
+    auto take = [&](int bytes) { const int q = at; at += (bytes + 15) & ~15; return q; };
+    const int D = sd.Dup * sd.Ddn, K = iters < D ? iters : D, L = sd.L;
+    auto hops = [&](int N) { const int m = N * (L - N); return (m < hmax ? m : hmax) | 1; };
+    l.hm_up = hops(sd.Nup);
+    l.hm_dn = hops(sd.Ndn);
+    l.v = take(D * 4);
+    l.vp = take(D * 4);
+    l.w = take(D * 4);
+    l.st_up = take(sd.Dup * 4);
+    l.st_dn = take(sd.Ddn * 4);
+    l.cnt_up = take(sd.Dup);
+    l.cnt_dn = take(sd.Ddn);
+    l.ent_up = take(sd.Dup * l.hm_up * 4);
+    l.ent_dn = take(sd.Ddn * l.hm_dn * 4);
+    l.d_up = take(sd.Dup * 4);
+    l.d_dn = take(sd.Ddn * 4);
+    l.alpha = take((K + 2) * 8);
+    l.beta = take((K + 2) * 8);
+    l.svec = take((K + 2) * 8);
+    // one double per warp for the sums and, for short recurrences, the solver's
+    // 3 (K + 2) doubles in the same place: both are the first warp's between barriers
+    const int red = T / 32 * 8, tri = tri_smem ? (K + 2) * 24 : 0;
+    l.scratch = take(red > tri ? red : tri);
+    l.hs = take(L * L * 8);
+    l.cf64 = take(2 * nb * 8);
+    l.cf32 = take(2 * nb * 4);
+    l.U64 = take(L * 8);
+    l.U32 = take(L * 4);
+    l.bidx = take(L * L);
+    l.bytes = at;
+    return l;
 }
 
-// xg: per-CTA scratch of lay.slot doubles for the FP64 Ritz vector, its H·v
-// and the tridiagonal solver's work (global memory; each CTA reuses its own
-// slot, which stays in L2), so that the shared memory holds only the FP32
+// Size classes of the sectors: 0 = the whole CTA (as many threads as it has),
+// then teams of 128, 64 and 32 threads, several in a CTA.
+constexpr int kBatchClasses = 4;
+struct BatchLay {
+    int hmax, nb, iters, tri_smem, bytes;   // bytes: shared memory of a CTA
+    int beg[kBatchClasses + 1];             // sectors of each class in the sorted list
+    int64_t slot;                           // doubles of global scratch per CTA
+};
+// doubles of global scratch of a sector: x, the restart's source (D each), the solver's 3 (K + 2)
+__host__ __device__ inline int64_t team_slot(int64_t D, int iters) { return 2 * D + 3 * ((iters < D ? iters : D) + 2); }
+
+template <int T>
+__device__ void solve_sector(const SectorDesc sd, const ModelDev &m, const double *__restrict__ start, const BatchLay &bl,
+                             unsigned char *smem, double *xg, int bar, const uint32_t *bin, double *outE, int *outK) {
+    const TeamLay l = team_lay(sd, T, bl.hmax, bl.nb, bl.iters, bl.tri_smem);
+    const int tid = threadIdx.x % T;
+    TeamVars &tv = *reinterpret_cast<TeamVars *>(smem);
+    float *v = (float *)(smem + l.v), *vp = (float *)(smem + l.vp);
+    float *const w = (float *)(smem + l.w);
+    const SpinLists up{(uint32_t *)(smem + l.st_up), smem + l.cnt_up, (uint32_t *)(smem + l.ent_up), (float *)(smem + l.d_up), l.hm_up};
+    const SpinLists dn{(uint32_t *)(smem + l.st_dn), smem + l.cnt_dn, (uint32_t *)(smem + l.ent_dn), (float *)(smem + l.d_dn), l.hm_dn};
+    double *alpha = (double *)(smem + l.alpha), *beta = (double *)(smem + l.beta), *svec = (double *)(smem + l.svec);
+    double *red = (double *)(smem + l.scratch);
+    double *hs = (double *)(smem + l.hs), *cf64 = (double *)(smem + l.cf64), *U64 = (double *)(smem + l.U64);
+    float *cf32 = (float *)(smem + l.cf32), *U32 = (float *)(smem + l.U32);
+    uint8_t *bidx = smem + l.bidx;
+    const int L = sd.L, D = sd.Dup * sd.Ddn, K = min(bl.iters, D);
+    double *x = xg, *hx = xg + D;
+    double *work = bl.tri_smem ? red : xg + 2 * (int64_t)D;
+    for (int i = tid; i < L * L; i += T) hs[i] = m.h[i];
+    for (int i = tid; i < L; i += T) {
+        U64[i] = m.U[i];
+        U32[i] = (float)m.U[i];
+    }
+    team_sync<T>(bar);
+    if (tid == 0) {
+        uint32_t um = 0;
+        for (int a = 0; a < L; ++a) um |= U64[a] != 0.0 ? 1u << a : 0u;
+        tv.umask = um;
+        int nb = 0;
+        for (int a = 0; a < L; ++a)
+            for (int b = 0; b < L; ++b) {
+                const double c = hs[a * L + b];
+                if (a == b || c == 0.0) continue;
+                bidx[a * L + b] = (uint8_t)nb;
+                cf64[2 * nb] = c;
+                cf64[2 * nb + 1] = -c;
+                cf32[2 * nb] = (float)c;
+                cf32[2 * nb + 1] = -(float)c;
+                ++nb;
+            }
+    }
+    team_sync<T>(bar);
+    build_spin<T>(L, sd.Nup, sd.Dup, sd.Ddn, hs, bidx, bin, up);
+    build_spin<T>(L, sd.Ndn, sd.Ddn, 1, hs, bidx, bin, dn);
+    // Restarted Lanczos: each cycle stops as soon as the lowest Ritz pair
+    // of T has converged to FP32 level (residual estimate
+    // beta_{k+1} |s_k| <= 1e-6 max(|alpha|, beta), tested after 4 steps and
+    // then at half the distance the decrease so far predicts (4 to 16
+    // steps), with a warm-started eigenvalue search and the last
+    // eigenvector component alone, and at the last step of the cycle), which keeps the FP32
+    // recurrence from running on after convergence and spoiling the Ritz
+    // vector; a cycle that ends unconverged restarts from its Ritz vector
+    // (at most three cycles).  Each cycle runs the recurrence twice: once
+    // for the scalars, once more (bit identical) to accumulate the Ritz
+    // vector x in FP64.
+    //
+    // this thread's elements i = tid + j T as (ru, rd)
+    const int dru = T / sd.Ddn, drd = T - dru * sd.Ddn;
+    const int ru0 = tid / sd.Ddn, rd0 = tid - ru0 * sd.Ddn;
+    auto next = [&](int &ru, int &rd) {
+        ru += dru;
+        rd += drd;
+        if (rd >= sd.Ddn) {
+            rd -= sd.Ddn;
+            ++ru;
+        }
+    };
+    for (int cyc = 0; cyc < 3; ++cyc) {
+        if (cyc > 0)
+            for (int i = tid; i < D; i += T) hx[i] = x[i];
+        team_sync<T>(bar);
+        auto source = [&](int i) { return (float)(cyc == 0 ? start[sd.off + i] : hx[i]); };
+        const uint32_t umask = tv.umask;
+        float fh = 0.f, fl = 0.f;
+        for (int i = tid; i < D; i += T) {
+            const float f = source(i);
+            ffp(fh, fl, f, f);
+        }
+        const double n2 = team_sum<T>((double)fh + (double)fl, red, bar);
+        if (tid == 0) {
+            tv.inv_n0 = 1.0 / sqrt(n2);
+            tv.conv = 0;
+            tv.end = 0;
+            tv.lam_hint = 0.0;
+            tv.gap_hint = 0.0;
+        }
+        team_sync<T>(bar);
+        // the first run: scalars
+        for (int i = tid; i < D; i += T) v[i] = (float)((double)source(i) * tv.inv_n0);
+        team_sync<T>(bar);
+        // the first warp's: step of the next test, step and residual of the last one
+        int next_check = 4, k_last = 0;
+        float r_last = 0.f;
+        double scale = 0.0;
+        for (int k = 0; k < K; ++k) {
+            const float bk = tv.bk;   // beta_k (k > 0)
+            float ah = 0.f, al = 0.f;
+            for (int i = tid, ru = ru0, rd = rd0; i < D; i += T, next(ru, rd)) {
+                float wi = hv_small<float>(sd, up, dn, cf32, U32, umask, hs, v, ru, rd);
+                if (k) wi = __fmaf_rn(-bk, vp[i], wi);
+                w[i] = wi;
+                ffp(ah, al, wi, v[i]);
+            }
+            const double a = team_sum<T>((double)ah + (double)al, red, bar);
+            if (tid == 0) {
+                alpha[k] = a;
+                tv.ak = (float)a;
+            }
+            scale = fmax(scale, fabs(a));
+            team_sync<T>(bar);
+            const float ak = tv.ak;
+            float bh = 0.f, blo = 0.f;
+            for (int i = tid; i < D; i += T) {
+                const float wi = __fmaf_rn(-ak, v[i], w[i]);
+                w[i] = wi;
+                ffp(bh, blo, wi, wi);
+            }
+            const double b2 = team_sum<T>((double)bh + (double)blo, red, bar);
+            if (tid < 32) {
+                const double b = sqrt(fmax(b2, 0.0));
+                const int kd = k + 1;
+                scale = fmax(scale, b);
+                bool conv = b <= 1e-13 * scale;
+                if (tid == 0) {
+                    beta[kd] = b;
+                    tv.bk = (float)b;
+                    tv.inv = 1.0f / (float)b;   // FP32: the FP64 divide is slow here
+                }
+                __syncwarp();
+                if (!conv && kd == next_check && kd < K) {
+                    // residual estimate from the last eigenvector component alone
+                    const Tri t = tri_stage(alpha, beta, kd, scale, work);
+                    const double lam = tri_lowest_warm(t, &tv.lam_hint, &tv.gap_hint);
+                    // relative to the scale, which the prediction needs in FP32 only
+                    const double r = b * tri_last_component(t, lam);
+                    const float rr = (float)(r * tri_unit(scale)), thr = (float)(1e-6 * (scale * tri_unit(scale)));
+                    if (r <= 1e-6 * scale) {
+                        conv = true;
+                    } else {
+                        // next test at half the distance the geometric decrease since
+                        // the last test predicts, 4 to 16 steps ahead
+                        int gap = 4;
+                        if (r_last > 0.f && rr < r_last) {
+                            const float per_step = logf(rr / r_last) / (float)(kd - k_last);
+                            const float steps = logf(thr / rr) / per_step;
+                            gap = 4 * max(1, min(4, (int)(0.5f * steps / 4.0f)));
+                        }
+                        next_check = kd + gap;
+                        r_last = rr;
+                        k_last = kd;
+                    }
+                }
+                if (conv || kd >= K) {
+                    // the Ritz pair of the final T for the second run (the vectors'
+                    // memory is free: it takes the recurrence from below)
+                    const Tri t = tri_stage(alpha, beta, kd, scale, work);
+                    const double lam = tri_lowest_warm(t, &tv.lam_hint, &tv.gap_hint);
+                    if (!tri_vector_twisted(t, beta, lam, svec, (double *)(smem + l.v)) && tid == 0)
+                        tridiag_vector_thread(alpha, beta, kd, lam / t.unit, svec, work);
+                    if (tid == 0) {
+                        if (conv || b * fabs(svec[kd - 1]) <= 1e-6 * scale) tv.conv = 1;
+                        tv.kdone = kd;
+                        tv.end = 1;
+                    }
+                }
+            }
+            team_sync<T>(bar);
+            if (tv.end) break;
+            // v_{k+1} takes the place of v_{k-1}
+            const float inv = tv.inv;
+            for (int i = tid; i < D; i += T) vp[i] = w[i] * inv;
+            float *t = vp;
+            vp = v;
+            v = t;
+            team_sync<T>(bar);
+        }
+        // the second run, one pass a step: the same vectors with the stored
+        // scalars, summed into x (the solver's arrays are free: they hold the
+        // scalars in FP32, as the first run used them)
+        float4 *sf = reinterpret_cast<float4 *>(work);
+        const int steps = tv.kdone;
+        for (int k = tid; k + 1 < steps; k += T)
+            sf[k] = make_float4(k ? (float)beta[k] : 0.f, (float)alpha[k], 1.0f / (float)beta[k + 1], 0.f);
+        for (int i = tid; i < D; i += T) {
+            const float f = (float)((double)source(i) * tv.inv_n0);
+            v[i] = f;
+            x[i] = svec[0] * (double)f;
+        }
+        team_sync<T>(bar);
+        for (int k = 0; k + 1 < steps; ++k) {
+            const float4 c = sf[k];
+            const double sk = svec[k + 1];
+            for (int i = tid, ru = ru0, rd = rd0; i < D; i += T, next(ru, rd)) {
+                const double xi = x[i];
+                float wi = hv_small<float>(sd, up, dn, cf32, U32, umask, hs, v, ru, rd);
+                if (k) wi = __fmaf_rn(-c.x, vp[i], wi);
+                wi = __fmaf_rn(-c.y, v[i], wi) * c.z;
+                vp[i] = wi;   // read by this thread alone
+                x[i] = fma(sk, (double)wi, xi);
+            }
+            float *t = vp;
+            vp = v;
+            v = t;
+            team_sync<T>(bar);
+        }
+        if (tv.conv) break;
+    }
+    team_sync<T>(bar);
+    // FP64 Rayleigh quotient of the Ritz vector
+    double xhx = 0.0, xx = 0.0;
+    for (int i = tid, ru = ru0, rd = rd0; i < D; i += T, next(ru, rd)) {
+        const double xi = x[i];
+        xhx = fma(xi, hv_small<double>(sd, up, dn, cf64, U64, tv.umask, hs, x, ru, rd), xhx);
+        xx = fma(xi, xi, xx);
+    }
+    const double num = team_sum<T>(xhx, red, bar);
+    team_sync<T>(bar);
+    const double den = team_sum<T>(xx, red, bar);
+    if (tid == 0) {
+        *outE = num / den;
+        *outK = tv.kdone;
+    }
+    team_sync<T>(bar);
+}
+
+template <int NT, int T>
+__device__ void batch_class(int cls, const SectorDesc *__restrict__ secs, const ModelDev *__restrict__ models,
+                            const double *__restrict__ start, const BatchLay &bl, unsigned char *smem, double *xg,
+                            int *counter, const uint32_t *bin, double *outE, int *outK) {
+    if (bl.beg[cls] == bl.beg[cls + 1]) return;
+    constexpr int teams = NT / T;
+    const int team = threadIdx.x / T, bar = 1 + team;
+    smem += team * (bl.bytes / teams & ~15);
+    xg += team * (bl.slot / teams);
+    TeamVars &tv = *reinterpret_cast<TeamVars *>(smem);
+    while (true) {
+        if (threadIdx.x % T == 0) tv.cur = bl.beg[cls] + atomicAdd(counter + cls, 1);
+        team_sync<T>(bar);
+        const int si = tv.cur;
+        if (si >= bl.beg[cls + 1]) break;
+        const SectorDesc sd = secs[si];
+        solve_sector<T>(sd, models[sd.model], start, bl, smem, xg, bar, bin, outE + si, outK + si);
+    }
+    __syncthreads();   // the next class lays the shared memory out anew
+}
+
+// One persistent launch over all sectors, largest class first, each class's
+// sectors from a device work queue.
+//
+// A sector is a long chain of short steps (FP64 sums and tridiagonal searches
+// whose dependent operations take about 150 clocks each, barriers, and vector
+// loops that a small sector does not fill the CTA with), so small ones go to
+// teams: several sectors side by side in a CTA, in the shared memory that a whole
+// CTA's sector has.  256 impurity models (16,620 sectors of up to 4,900 states):
+// 12.3 ms in the kernel at 256 threads, against 19.3 ms with one sector a CTA; 128
+// threads 16.1, 512 threads 22.0 ms.  Three models (192 sectors, no queue): 1.6 ms,
+// the largest sector's own time.
+//
+// xg: per-CTA scratch of bl.slot doubles for the FP64 Ritz vector, the restart's
+// source and, for long recurrences, the tridiagonal solver's work (global memory; each CTA
+// reuses its own slot, which stays in L2), so that the shared memory holds only the FP32
 // recurrence and three CTAs fit on an SM.
 //
 // NT threads per CTA (128, 256 or 512; the autotuner's choice), at most
 // 64 K / (NT x 3 x 256 / NT) registers a thread so that three CTAs fit on an SM
 // at 256 and the register budget per SM stays the same at the other sizes.
 template <int NT>
-__global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const SectorDesc *__restrict__ secs, int nsec,
+__global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const SectorDesc *__restrict__ secs,
                                                          const ModelDev *__restrict__ models,
-                                                         const double *__restrict__ start, int iters, BatchSmem lay,
+                                                         const double *__restrict__ start, const BatchLay bl,
                                                          int *counter, double *__restrict__ outE, int *__restrict__ outK,
                                                          double *__restrict__ xg) {
     extern __shared__ __align__(16) unsigned char smr[];
-    // layout
-    unsigned char *p = smr;
-    auto take = [&](size_t bytes) { unsigned char *q = p; p += (bytes + 15) & ~(size_t)15; return q; };
-    const int maxD = lay.maxD, maxDs = lay.maxDs, hmax = lay.hmax, kmax = lay.iters;
-    float *v = (float *)take((size_t)maxD * 4);
-    float *vp = (float *)take((size_t)maxD * 4);
-    float *w = (float *)take((size_t)maxD * 4);
-    double *x = xg + (size_t)blockIdx.x * lay.slot;
-    double *hx = x + maxD;
-    SpinLists up, dn;
-    up.st = (uint32_t *)take((size_t)maxDs * 4); dn.st = (uint32_t *)take((size_t)maxDs * 4);
-    up.cnt = (uint8_t *)take((size_t)maxDs); dn.cnt = (uint8_t *)take((size_t)maxDs);
-    up.ent = (uint32_t *)take((size_t)maxDs * hmax * 4); dn.ent = (uint32_t *)take((size_t)maxDs * hmax * 4);
-    up.d32 = (float *)take((size_t)maxDs * 4); dn.d32 = (float *)take((size_t)maxDs * 4);
-    double *alpha = (double *)take((size_t)(kmax + 2) * 8);
-    double *beta = (double *)take((size_t)(kmax + 2) * 8);
-    double *svec = (double *)take((size_t)(kmax + 2) * 8);
-    // reduction slots (one double or float2 per thread) and, for short recurrences, the
-    // solver's 3 (kmax + 2) doubles in the same place: both are warp 0's between barriers
-    double *red = (double *)take(batch_scratch(NT, kmax, lay.tri_smem));
-    double *work = lay.tri_smem ? red : xg + (size_t)blockIdx.x * lay.slot + 2 * (size_t)maxD;
-    __shared__ uint32_t umask_s;
-    __shared__ double hs[kBatchMaxL * kBatchMaxL];
-    __shared__ double bc64[kBatchMaxL * kBatchMaxL];
-    __shared__ float bc32[kBatchMaxL * kBatchMaxL];
-    __shared__ double U64[kBatchMaxL];
-    __shared__ float U32[kBatchMaxL];
-    __shared__ uint8_t bidx[kBatchMaxL * kBatchMaxL];
     __shared__ uint32_t bin[(kBatchMaxL + 1) * (kBatchMaxL + 1)];
-    __shared__ int cur;
-    for (int i = threadIdx.x; i < (kBatchMaxL + 1) * (kBatchMaxL + 1); i += blockDim.x) {
+    for (int i = threadIdx.x; i < (kBatchMaxL + 1) * (kBatchMaxL + 1); i += NT) {
         const int n = i / (kBatchMaxL + 1), k = i % (kBatchMaxL + 1);
         // C(n, k) by the multiplicative formula (small n)
         uint32_t c = (k > n) ? 0u : 1u;
@@ -239,217 +515,11 @@ __global__ void __launch_bounds__(NT, (NT >= 512 ? 1 : 768 / NT)) k_batch(const 
         bin[i] = c;
     }
     __syncthreads();
-    while (true) {
-        if (threadIdx.x == 0) cur = atomicAdd(counter, 1);
-        __syncthreads();
-        const int si = cur;
-        __syncthreads();
-        if (si >= nsec) break;
-        const SectorDesc sd = secs[si];
-        const ModelDev &m = models[sd.model];
-        const int L = sd.L;
-        for (int i = threadIdx.x; i < L * L; i += blockDim.x) hs[i] = m.h[i];
-        for (int i = threadIdx.x; i < L; i += blockDim.x) { U64[i] = m.U[i]; U32[i] = (float)m.U[i]; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t um = 0;
-            for (int a = 0; a < L; ++a) um |= U64[a] != 0.0 ? 1u << a : 0u;
-            umask_s = um;
-            int nb = 0;
-            for (int a = 0; a < L; ++a)
-                for (int b = 0; b < L; ++b)
-                    if (a != b && hs[a * L + b] != 0.0) {
-                        bidx[a * L + b] = (uint8_t)nb;
-                        bc64[nb] = hs[a * L + b];
-                        bc32[nb] = (float)hs[a * L + b];
-                        ++nb;
-                    }
-        }
-        __syncthreads();
-        build_spin(L, sd.Nup, sd.Dup, hmax, hs, bidx, bin, up);
-        build_spin(L, sd.Ndn, sd.Ddn, hmax, hs, bidx, bin, dn);
-        const int D = sd.Dup * sd.Ddn;
-        const int K = min(iters, D);
-        // Restarted Lanczos: each cycle stops as soon as the lowest Ritz pair
-        // of T has converged to FP32 level (residual estimate
-        // beta_{k+1} |s_k| <= 1e-6 max(|alpha|, beta), tested after 4 steps and
-        // then at half the distance the decrease so far predicts (4 to 16
-        // steps), with a warm-started eigenvalue search and the last
-        // eigenvector component alone, and at the last step of the cycle), which keeps the FP32
-        // recurrence from running on after convergence and spoiling the Ritz
-        // vector; a cycle that ends unconverged restarts from its Ritz vector
-        // (at most three cycles).  Each cycle runs the recurrence twice: once
-        // for the scalars, once more (bit identical) to accumulate the Ritz
-        // vector x in FP64.
-        __shared__ int conv_s, end_s;
-        __shared__ double lam_hint, gap_hint;   // warm start of the convergence test's eigenvalue search
-        __shared__ double inv_n0;
-        __shared__ float ak_s, bk_s, inv_s;     // alpha_k, beta_{k+1} and 1 / beta_{k+1} of the step
-        __shared__ int kdone;
-        // this thread's elements i = threadIdx.x + j NT as (ru, rd)
-        const int dru = NT / sd.Ddn, drd = NT - dru * sd.Ddn;
-        const int ru0 = (int)threadIdx.x / sd.Ddn, rd0 = (int)threadIdx.x - ru0 * sd.Ddn;
-        const uint32_t umask = umask_s;
-        auto next = [&](int &ru, int &rd) {
-            ru += dru;
-            rd += drd;
-            if (rd >= sd.Ddn) {
-                rd -= sd.Ddn;
-                ++ru;
-            }
-        };
-        for (int cyc = 0; cyc < 3; ++cyc) {
-            if (cyc > 0) {
-                for (int i = threadIdx.x; i < D; i += NT) hx[i] = x[i];
-                __syncthreads();
-            }
-            auto source = [&](int i) { return (float)(cyc == 0 ? start[sd.off + i] : hx[i]); };
-            float fh = 0.f, fl = 0.f;
-            for (int i = threadIdx.x; i < D; i += NT) {
-                const float f = source(i);
-                ffp(fh, fl, f, f);
-            }
-            const double n2 = bsum0(fh, fl, reinterpret_cast<float2 *>(red));
-            if (threadIdx.x == 0) {
-                inv_n0 = 1.0 / sqrt(n2);
-                conv_s = 0;
-                end_s = 0;
-                lam_hint = 0.0;
-                gap_hint = 0.0;
-            }
-            __syncthreads();
-            // the first run: scalars
-            for (int i = threadIdx.x; i < D; i += NT) v[i] = (float)((double)source(i) * inv_n0);
-            __syncthreads();
-            // warp 0's: step of the next test, step and residual of the last one
-            int next_check = 4, k_last = 0;
-            double r_last = 0.0, scale = 0.0;
-            for (int k = 0; k < K; ++k) {
-                const float bk = bk_s;   // beta_k (k > 0)
-                float ah = 0.f, al = 0.f;
-                for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
-                    float wi = hv_small<float>(sd, hmax, up, dn, bc32, U32, umask, hs, v, ru, rd);
-                    if (k) wi = __fmaf_rn(-bk, vp[i], wi);
-                    w[i] = wi;
-                    ffp(ah, al, wi, v[i]);
-                }
-                const double a = bsum0(ah, al, reinterpret_cast<float2 *>(red));
-                if (threadIdx.x == 0) {
-                    alpha[k] = a;
-                    ak_s = (float)a;
-                }
-                scale = fmax(scale, fabs(a));
-                __syncthreads();
-                const float ak = ak_s;
-                float bh = 0.f, bl = 0.f;
-                for (int i = threadIdx.x; i < D; i += NT) {
-                    const float wi = __fmaf_rn(-ak, v[i], w[i]);
-                    w[i] = wi;
-                    ffp(bh, bl, wi, wi);
-                }
-                const double b2 = bsum0(bh, bl, reinterpret_cast<float2 *>(red));
-                if (threadIdx.x < 32) {
-                    const double b = sqrt(fmax(b2, 0.0));
-                    const int kd = k + 1;
-                    scale = fmax(scale, b);
-                    bool conv = b <= 1e-13 * scale;
-                    if (threadIdx.x == 0) {
-                        beta[kd] = b;
-                        bk_s = (float)b;
-                        inv_s = 1.0f / (float)b;   // FP32: the FP64 divide is slow here
-                    }
-                    __syncwarp();
-                    if (!conv && kd == next_check && kd < K) {
-                        // residual estimate from the last eigenvector component alone
-                        const Tri t = tri_stage(alpha, beta, kd, scale, work);
-                        const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint);
-                        const double thr = 1e-6 * scale;
-                        const double r = b * tri_last_component(t, lam);
-                        if (r <= thr) {
-                            conv = true;
-                        } else {
-                            // next test at half the distance the geometric decrease since
-                            // the last test predicts, 4 to 16 steps ahead
-                            int gap = 4;
-                            if (r_last > 0.0 && r < r_last) {
-                                const double per_step = log(r / r_last) / (double)(kd - k_last);
-                                const double steps = log(thr / r) / per_step;
-                                gap = 4 * max(1, min(4, (int)(0.5 * steps / 4.0)));
-                            }
-                            next_check = kd + gap;
-                            r_last = r;
-                            k_last = kd;
-                        }
-                    }
-                    if (conv || kd >= K) {
-                        // the Ritz pair of the final T for the second run
-                        const Tri t = tri_stage(alpha, beta, kd, scale, work);
-                        const double lam = tri_lowest_warm(t, &lam_hint, &gap_hint) / t.unit;
-                        if (threadIdx.x == 0) {
-                            tridiag_vector_thread(alpha, beta, kd, lam, svec, work);
-                            if (conv || b * fabs(svec[kd - 1]) <= 1e-6 * scale) conv_s = 1;
-                            kdone = kd;
-                            end_s = 1;
-                        }
-                    }
-                }
-                __syncthreads();
-                if (end_s) break;
-                // v_{k+1} takes the place of v_{k-1}
-                const float inv = inv_s;
-                for (int i = threadIdx.x; i < D; i += NT) vp[i] = w[i] * inv;
-                float *t = vp;
-                vp = v;
-                v = t;
-                __syncthreads();
-            }
-            // the second run, one pass a step: the same vectors with the stored
-            // scalars, summed into x (the solver's arrays are free: they hold the
-            // scalars in FP32, as the first run used them)
-            float4 *sf = reinterpret_cast<float4 *>(work);
-            const int steps = kdone;
-            for (int k = threadIdx.x; k + 1 < steps; k += NT)
-                sf[k] = make_float4(k ? (float)beta[k] : 0.f, (float)alpha[k], 1.0f / (float)beta[k + 1], 0.f);
-            for (int i = threadIdx.x; i < D; i += NT) {
-                const float f = (float)((double)source(i) * inv_n0);
-                v[i] = f;
-                x[i] = svec[0] * (double)f;
-            }
-            __syncthreads();
-            for (int k = 0; k + 1 < steps; ++k) {
-                const float4 c = sf[k];
-                const double sk = svec[k + 1];
-                for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
-                    float wi = hv_small<float>(sd, hmax, up, dn, bc32, U32, umask, hs, v, ru, rd);
-                    if (k) wi = __fmaf_rn(-c.x, vp[i], wi);
-                    wi = __fmaf_rn(-c.y, v[i], wi) * c.z;
-                    vp[i] = wi;   // read by this thread alone
-                    x[i] = fma(sk, (double)wi, x[i]);
-                }
-                float *t = vp;
-                vp = v;
-                v = t;
-                __syncthreads();
-            }
-            if (conv_s) break;
-        }
-        __syncthreads();
-        // FP64 Rayleigh quotient of the Ritz vector
-        double xhx = 0.0, xx = 0.0;
-        for (int i = threadIdx.x, ru = ru0, rd = rd0; i < D; i += NT, next(ru, rd)) {
-            const double xi = x[i];
-            xhx = fma(xi, hv_small<double>(sd, hmax, up, dn, bc64, U64, umask, hs, x, ru, rd), xhx);
-            xx = fma(xi, xi, xx);
-        }
-        const double num = bsum0(xhx, red);
-        __syncthreads();
-        const double den = bsum0(xx, red);
-        if (threadIdx.x == 0) {
-            outE[si] = num / den;
-            if (outK) outK[si] = kdone;
-        }
-        __syncthreads();
-    }
+    xg += (size_t)blockIdx.x * bl.slot;
+    batch_class<NT, NT>(0, secs, models, start, bl, smr, xg, counter, bin, outE, outK);
+    if (NT > 128) batch_class<NT, NT == 128 ? 64 : 128>(1, secs, models, start, bl, smr, xg, counter, bin, outE, outK);
+    batch_class<NT, 64>(2, secs, models, start, bl, smr, xg, counter, bin, outE, outK);
+    batch_class<NT, 32>(3, secs, models, start, bl, smr, xg, counter, bin, outE, outK);
 }
 
 static int sector_list(int n_models, const gbr_model_desc *models, std::vector<SectorDesc> &secs, int64_t *n_states) {
@@ -494,23 +564,48 @@ namespace gbr {
 static int g_batch_threads = kBatchThreads, g_batch_per_sm = 0;
 
 template <int NT>
-static int launch_batch(int grid_req_per_sm, size_t smem, int nsec, const SectorDesc *secs, const ModelDev *md,
-                        const double *d_start, int K, const BatchSmem &lay, int *ctr, double *E, int *Kout,
-                        DevBuf &dx, cudaStream_t st, int *grid_out) {
+static int launch_batch(int grid_req_per_sm, int nsec, const SectorDesc *secs, const ModelDev *md, const double *d_start,
+                        const BatchLay &bl, int *ctr, double *E, int *Kout, DevBuf &dx, cudaStream_t st) {
     auto kern = k_batch<NT>;
-    GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bl.bytes));
     int per_sm = 0;
-    GBR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
+    GBR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, (size_t)bl.bytes));
     per_sm = std::max(1, per_sm);
     if (grid_req_per_sm > 0) per_sm = std::min(per_sm, grid_req_per_sm);
     const int grid = std::max(1, std::min<int>(nsec, sm_count() * per_sm));
     int rc;
-    if ((rc = dx.alloc((size_t)grid * (size_t)lay.slot * 8))) return rc;
-    kern<<<grid, NT, smem, st>>>(secs, nsec, md, d_start, K, lay, ctr, E, Kout, dx.as<double>());
+    if ((rc = dx.alloc((size_t)grid * (size_t)bl.slot * 8))) return rc;
+    kern<<<grid, NT, (size_t)bl.bytes, st>>>(secs, md, d_start, bl, ctr, E, Kout, dx.as<double>());
     GBR_LAUNCH_CHECK();
     count_launches(1);
-    if (grid_out) *grid_out = grid;
     return GBR_OK;
+}
+
+// Class of every sector and the CTA's shared memory: what the largest sector needs
+// for the whole CTA; a smaller one goes to the smallest team whose size suits it
+// and whose share of that memory holds it.
+// The limits keep a team's vector loops (ten elements a thread at most) below its FP64 chains.
+constexpr int kBatchTeam[kBatchClasses] = {0, 128, 64, 32};
+constexpr int kBatchTeamMax[kBatchClasses] = {0, 1200, 400, 64};   // states
+static void batch_plan(const std::vector<SectorDesc> &secs, int threads, BatchLay *bl, std::vector<int> *cls) {
+    bl->bytes = 0;
+    for (const SectorDesc &s : secs) bl->bytes = std::max(bl->bytes, team_lay(s, threads, bl->hmax, bl->nb, bl->iters, bl->tri_smem).bytes);
+    cls->assign(secs.size(), 0);
+    bl->slot = 0;
+    for (size_t i = 0; i < secs.size(); ++i) {
+        const SectorDesc &s = secs[i];
+        const int D = s.Dup * s.Ddn;
+        int teams = 1;
+        for (int c = kBatchClasses - 1; c >= 1; --c) {
+            const int T = kBatchTeam[c], n = threads / T;
+            if (T >= threads || D > kBatchTeamMax[c]) continue;
+            if (team_lay(s, T, bl->hmax, bl->nb, bl->iters, bl->tri_smem).bytes > (bl->bytes / n & ~15)) continue;
+            (*cls)[i] = c;
+            teams = n;
+            break;
+        }
+        bl->slot = std::max(bl->slot, teams * team_slot(D, bl->iters));
+    }
 }
 
 static int batch_run(int n_models, const gbr_model_desc *models, const double *d_start, int iters, double *h_E0,
@@ -523,7 +618,7 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
     int rc = sector_list(n_models, models, secs, &n_states);
     if (rc) return rc;
     std::vector<ModelDev> md((size_t)n_models);
-    int maxD = 1, maxDs = 1, hmax = 1;
+    int maxD = 1, hmax = 1, nbmax = 1;
     for (int m = 0; m < n_models; ++m) {
         const int L = models[m].L;
         memset(&md[(size_t)m], 0, sizeof(ModelDev));
@@ -545,27 +640,34 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
         // largest hop count of any per-spin state: N (L - N) bounds it, and so do the
         // bonds, each of which lets at most one of its ends hop
         for (int N = 0; N <= L; ++N) hmax = std::max(hmax, std::min(N * (L - N), nb / 2));
-        maxDs = std::max<int>(maxDs, (int)binom(L, L / 2));
+        nbmax = std::max(nbmax, nb);
     }
     for (const SectorDesc &s : secs) maxD = std::max(maxD, s.Dup * s.Ddn);
     const int K = std::min(iters, maxD);
-    BatchSmem lay{maxD, maxDs, hmax, K, K <= kBatchTriSmem ? 1 : 0, 2 * (int64_t)maxD + 3 * (int64_t)(K + 2)};
-    auto r16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    size_t smem = 3 * r16((size_t)maxD * 4) + 2 * r16((size_t)maxDs * 4) +
-                  2 * r16((size_t)maxDs) + 2 * r16((size_t)maxDs * hmax * 4) + 2 * r16((size_t)maxDs * 4) +
-                  3 * r16((size_t)(K + 2) * 8) + r16(batch_scratch(threads, K, lay.tri_smem));
+    BatchLay bl;
+    bl.hmax = hmax;
+    bl.nb = nbmax;
+    bl.iters = K;
     int dev = 0, optin = 0;
     GBR_CUDA_TRY(cudaGetDevice(&dev));
     GBR_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (smem + 8192 > (size_t)optin)
-        return set_error(GBR_EINVAL, "largest sector needs %zu bytes of shared memory (limit %d)", smem, optin);
-    // largest sectors first
+    std::vector<int> cls;
+    // the solver's arrays in shared memory if they fit there
+    for (bl.tri_smem = K <= kBatchTriSmem ? 1 : 0;; bl.tri_smem = 0) {
+        batch_plan(secs, threads, &bl, &cls);
+        if (bl.bytes + 1024 <= optin) break;
+        if (!bl.tri_smem) return set_error(GBR_EINVAL, "largest sector needs %d bytes of shared memory (limit %d)", bl.bytes, optin);
+    }
+    // by class, the largest sectors first
     std::vector<SectorDesc> order(secs);
     std::vector<int> idx(secs.size());
     for (size_t i = 0; i < idx.size(); ++i) idx[i] = (int)i;
     std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) {
+        if (cls[(size_t)a] != cls[(size_t)b]) return cls[(size_t)a] < cls[(size_t)b];
         return (int64_t)secs[(size_t)a].Dup * secs[(size_t)a].Ddn > (int64_t)secs[(size_t)b].Dup * secs[(size_t)b].Ddn;
     });
+    for (int c = 0; c <= kBatchClasses; ++c)
+        bl.beg[c] = (int)std::count_if(cls.begin(), cls.end(), [&](int k) { return k < c; });
     for (size_t i = 0; i < idx.size(); ++i) order[i] = secs[(size_t)idx[i]];
     DevBuf dsec, dmod, dE, dK, dctr, dx;
     if ((rc = dsec.upload(order.data(), order.size() * sizeof(SectorDesc)))) return rc;
@@ -582,14 +684,14 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
     }
     const int nsec = (int)order.size();
     if (threads == 128)
-        rc = launch_batch<128>(per_sm_req, smem, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, K, lay,
-                               dctr.as<int>(), dE.as<double>(), dK.as<int>(), dx, st, nullptr);
+        rc = launch_batch<128>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
+                               dE.as<double>(), dK.as<int>(), dx, st);
     else if (threads == 512)
-        rc = launch_batch<512>(per_sm_req, smem, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, K, lay,
-                               dctr.as<int>(), dE.as<double>(), dK.as<int>(), dx, st, nullptr);
+        rc = launch_batch<512>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
+                               dE.as<double>(), dK.as<int>(), dx, st);
     else
-        rc = launch_batch<256>(per_sm_req, smem, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, K, lay,
-                               dctr.as<int>(), dE.as<double>(), dK.as<int>(), dx, st, nullptr);
+        rc = launch_batch<256>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
+                               dE.as<double>(), dK.as<int>(), dx, st);
     if (rc) return rc;
     if (ms_out) {
         cudaEventRecord(e1, st);

@@ -406,22 +406,20 @@ __global__ void __launch_bounds__(32) k_ritz_prefix(const LzState *st, const dou
     else if (res <= u * st->scale) atomicMin(kout, k);
 }
 
-// eigenvector s of T_k for the eigenvalue *lam
-__global__ void __launch_bounds__(32) k_ritz_vector(const double *alpha, const double *beta, int k, const double *lam,
-                                                    double *s, double *work, int in_smem) {
+// eigenvector s of T_k for the eigenvalue *lam; in shared memory five arrays
+// (the scaled T, and the two recurrences)
+__global__ void __launch_bounds__(32) k_ritz_vector(const LzState *st, const double *alpha, const double *beta, int k,
+                                                    const double *lam, double *s, double *work, int in_smem) {
     extern __shared__ __align__(16) double tri_sm[];
+    bool ok = false;
     if (in_smem) {
-        // alpha, beta and the two work arrays
-        double *a = tri_sm, *b = tri_sm + k;
-        for (int i = threadIdx.x; i < k; i += 32) {
-            a[i] = alpha[i];
-            b[i] = beta[i];
-        }
-        __syncwarp();
-        if (threadIdx.x == 0) tridiag_vector_thread(a, b, k, *lam, s, tri_sm + 2 * k);
-    } else if (threadIdx.x == 0) {
-        tridiag_vector_thread(alpha, beta, k, *lam, s, work);
+        double *f = tri_sm + 3 * k, *g = tri_sm + 4 * k;
+        const Tri t = tri_stage(alpha, beta, k, st->scale, tri_sm);
+        ok = tri_vector_twisted(t, beta, *lam * t.unit, f, g);
+        if (ok)
+            for (int i = threadIdx.x; i < k; i += 32) s[i] = f[i];
     }
+    if (!ok && threadIdx.x == 0) tridiag_vector_thread(alpha, beta, k, *lam, s, work);
 }
 
 // x (FP64) = sum_j s_j v_j = sum_j (s_j / g_j) u_j over the stored
@@ -919,8 +917,9 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
         if ((rc = grow(x, (size_t)n * 8))) return rc;
         if ((rc = grow(hx, (size_t)n * 8))) return rc;
         double *sv = z.svec.as<double>();
-        const bool vsm = 4 * kr <= 3 * kTriSmemRows;
-        k_ritz_vector<<<1, 32, vsm ? (size_t)kr * 32 : 0, s>>>(z.alpha.as<double>(), z.beta.as<double>(), kr,
+        const bool vsm = 5 * kr <= 3 * kTriSmemRows;
+        k_ritz_vector<<<1, 32, vsm ? (size_t)kr * 40 : 0, s>>>(z.state.as<LzState>(), z.alpha.as<double>(),
+                                                             z.beta.as<double>(), kr,
                                                              lam + (kr == kdone ? ncand - 1 : kr / 8 - 1), sv,
                                                              z.work.as<double>(), vsm);
         count_launches(1);
