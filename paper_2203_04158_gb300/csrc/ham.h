@@ -90,7 +90,7 @@ struct gbr_ham {
     gbr::DevBuf bonds;         // nbond x {p, q} uint8 pairs (as uint16), bond order
     gbr::DevBuf bond_coef64;   // nbond doubles
     gbr::DevBuf bond_coef32;   // nbond floats
-    gbr::DevBuf hcoef64;       // L x L doubles (fused path lookups)
+    gbr::DevBuf ubonds;        // undirected bonds p < q as masks (fused path)
     gbr::DevBuf binom;         // (L+1) x (L+1) uint32 binomials (CNS ranking)
     // tuned launch shape (0 = default): rows per CTA of the gather passes
     int tune_up_rows[2] = {0, 0};
@@ -101,8 +101,8 @@ struct gbr_ham {
     // spin-down, spin-up and fused-update passes (32 or 64; 0 = 64)
     int win_dn[2] = {-1, -1}, win_up[2] = {0, 0}, win_lz[2] = {0, 0};
     // chunk width R of the per-spin staggered tables (8 or 4) and threads per
-    // state of the fused per-element kernel (1, 2 or 4)
-    int rank_R[2] = {8, 8}, fused_tps[2] = {1, 1};
+    // state of the fused per-element kernel (1, 2 or 4; 0 = by the sector's size)
+    int rank_R[2] = {8, 8}, fused_tps[2] = {0, 0};
     // threads per CTA of the plain gather passes (spin-down, spin-up, fused
     // update): 128, or 64 for column chunks half as wide
     int gather_nt[3][2] = {{128, 128}, {128, 128}, {128, 128}};

@@ -105,48 +105,99 @@ __device__ __forceinline__ void stage_u32(uint32_t *s, const uint32_t *__restric
     for (int i = threadIdx.x; i < n; i += blockDim.x) s[i] = __ldg(g + i);
 }
 
+// the same in 16-byte packs, for a table whose buffer is padded to whole packs
+__host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
+__device__ __forceinline__ void stage_packs(uint32_t *s, const uint32_t *__restrict__ g, int n) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < pad4(n) / 4; i += blockDim.x)
+        reinterpret_cast<uint4 *>(s)[i] = __ldg(reinterpret_cast<const uint4 *>(g) + i);
+}
+
 // ---------------------------------------------------------------- hop lists
 //
-// One thread per per-spin state r: unrank (list), then for every occupied
-// site p (ascending) and every empty site q connected to it (ascending):
+// For every per-spin state r (unrank: list) and every occupied site p
+// (ascending) and empty site q connected to it (ascending):
 // target = rank(a ^ (2^p | 2^q)), sign = parity of the occupied sites
 // strictly between p and q (Eq. Talpha, gather form Eq. Talpha2).
-__global__ void k_hop_lists(const SpinK s, const HamK hk, const uint32_t *__restrict__ states,
-                            const uint32_t *__restrict__ gtab, const uint32_t *__restrict__ gbinom,
-                            const uint16_t *__restrict__ gbond_index, uint16_t *__restrict__ cnt,
-                            uint32_t *__restrict__ tgt, uint16_t *__restrict__ bond, int hmax) {
-    extern __shared__ __align__(16) uint32_t sm[];
+//
+// One thread per state and site, both spin species in one launch (the first
+// nblk0 blocks take s0).  A thread finds the place of its site's hops in the list
+// by counting those of the lower sites, a few instructions a site; a thread per
+// state ranked its ~10 to 30 hops one after the other on a handful of CTAs.
+// Bound: latency (table staging, one chain of look-ups).  HOPLIST_FIGURES
+constexpr int kHopThreads = 256;
+
+struct HopOut {
+    const uint32_t *states, *tab;
+    uint16_t *cnt;
+    uint32_t *tgt;
+    uint16_t *bond;
+    int hmax;
+};
+
+// hops of the occupied sites of a below site p
+__device__ __forceinline__ int hops_below(const HamK &hk, uint32_t a, int p) {
+    uint32_t occ = a & ((1u << p) - 1u);
+    int k = 0;
+    while (occ) {
+        k += __popc(hk.nbr[__ffs(occ) - 1] & ~a);
+        occ &= occ - 1u;
+    }
+    return k;
+}
+
+struct HopArgs {
+    SpinK s0, s1;
+    HopOut o0, o1;
+    int nblk0, nblk;             // blocks of the first species, of both
+    const uint32_t *binom;
+    const uint16_t *bond_index;
+};
+
+__device__ __forceinline__ void hop_lists_block(const HopArgs &ha, const HamK &hk, uint32_t *sm, int blk) {
+    const bool first = blk < ha.nblk0;
+    const SpinK &s = first ? ha.s0 : ha.s1;
+    const HopOut &o = first ? ha.o0 : ha.o1;
     uint32_t *tab = sm;
     const int nb = (hk.L + 1) * (hk.L + 1);
-    uint32_t *binom = sm + s.tab_entries;
+    uint32_t *binom = sm + pad4(s.tab_entries);
     uint16_t *bidx = reinterpret_cast<uint16_t *>(binom + nb);
-    stage_u32(tab, gtab, s.tab_entries);
-    stage_u32(binom, gbinom, nb);
-    for (int i = threadIdx.x; i < hk.L * hk.L; i += blockDim.x) bidx[i] = gbond_index[i];
-    __syncthreads();
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < s.D; r += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t a = states[r];
-        int k = 0;
-        uint32_t occ = a;
-        while (occ) {
-            const int p = __ffs(occ) - 1;
-            occ &= occ - 1u;
-            uint32_t emp = hk.nbr[p] & ~a;
-            while (emp) {
-                const int q = __ffs(emp) - 1;
-                emp &= emp - 1u;
-                const uint32_t b = a ^ ((1u << p) | (1u << q));
-                const uint32_t t = spin_rank(s, hk.rank_method, tab, binom, b);
-                const uint32_t sg = (uint32_t)(__popc(a & between_mask(p, q)) & 1);
-                if (k < hmax) {
-                    tgt[(int64_t)k * s.D + r] = t | (sg << 31);
-                    bond[(int64_t)k * s.D + r] = bidx[p * hk.L + q];
-                }
-                ++k;
-            }
-        }
-        cnt[r] = (uint16_t)min(k, hmax);
+    if (hk.rank_method == GBR_RANK_CNS) {
+        stage_u32(binom, ha.binom, nb);
+    } else {
+        stage_packs(tab, o.tab, s.tab_entries);
     }
+    for (int i = threadIdx.x; i < hk.L * hk.L; i += kHopThreads) bidx[i] = ha.bond_index[i];
+    __syncthreads();
+    const int64_t at = (int64_t)(blk - (first ? 0 : ha.nblk0)) * kHopThreads + threadIdx.x;
+    const int p = (int)(at / s.D);
+    if (p >= hk.L) return;
+    const int64_t r = at - p * s.D;
+    const uint32_t a = o.states[r];
+    if (p == 0) {
+        const int n = hops_below(hk, a, hk.L - 1) + ((a >> (hk.L - 1)) & 1u ? __popc(hk.nbr[hk.L - 1] & ~a) : 0);
+        o.cnt[r] = (uint16_t)min(n, o.hmax);
+    }
+    if (!((a >> p) & 1u)) return;
+    uint32_t emp = hk.nbr[p] & ~a;
+    int k = emp ? hops_below(hk, a, p) : 0;
+    while (emp) {
+        const int q = __ffs(emp) - 1;
+        emp &= emp - 1u;
+        const uint32_t b = a ^ ((1u << p) | (1u << q));
+        const uint32_t t = spin_rank(s, hk.rank_method, tab, binom, b);
+        const uint32_t sg = (uint32_t)(__popc(a & between_mask(p, q)) & 1);
+        if (k < o.hmax) {
+            o.tgt[(int64_t)k * s.D + r] = t | (sg << 31);
+            o.bond[(int64_t)k * s.D + r] = bidx[p * hk.L + q];
+        }
+        ++k;
+    }
+}
+
+__global__ void __launch_bounds__(kHopThreads) k_hop_lists(const HopArgs ha, const HamK hk) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    hop_lists_block(ha, hk, sm, (int)blockIdx.x);
 }
 
 template <typename T> struct Vec;
@@ -189,12 +240,12 @@ __global__ void __launch_bounds__(256) k_hv_fused(const SpinK su, const SpinK sd
                                                   T *__restrict__ y) {
     extern __shared__ __align__(16) uint32_t sm[];
     uint32_t *tu = sm;
-    uint32_t *td = tu + su.tab_entries;
+    uint32_t *td = tu + pad4(su.tab_entries);
     const int nb = (hk.L + 1) * (hk.L + 1);
-    uint32_t *binom = td + sd.tab_entries;
-    T *hc = reinterpret_cast<T *>(binom + nb + (nb & 1));   // 8-byte aligned
-    stage_u32(tu, tab_up, su.tab_entries);
-    stage_u32(td, tab_dn, sd.tab_entries);
+    uint32_t *binom = td + pad4(sd.tab_entries);
+    T *hc = reinterpret_cast<T *>(binom + pad4(nb));
+    stage_packs(tu, tab_up, su.tab_entries);
+    stage_packs(td, tab_dn, sd.tab_entries);
     stage_u32(binom, gbinom, nb);
     for (int i = threadIdx.x; i < hk.L * hk.L; i += blockDim.x) hc[i] = hcoef[i];
     T uval[kMaxUClasses];
@@ -250,6 +301,106 @@ __global__ void __launch_bounds__(256) k_hv_fused(const SpinK su, const SpinK sd
     }
 }
 
+// The same for small sectors, kWideTps threads per element: the bonds p < q of both
+// spins (spin down first) are dealt round-robin to the group's threads.
+// A thread first tests its bonds -- a hop exists where exactly one end is occupied,
+// in either direction with the same coefficient, h being symmetric -- and keeps the
+// answers as a 32-bit mask, then works off the set bits, two hops a round, so that
+// no lane waits for another's empty sites.
+//
+// Bound: latency.  8-site ring (4,900 states): 4.6 us FP32, 5.8 us FP64, against 7.0
+// and 8.2 us with one thread per element; 3x3 torus with diagonal hops (15,876):
+// 11.7 and 13.8 against 14.5 and 16.8 us.  Larger sectors (48,400 states: 9.9 us
+// against 7.7) keep k_hv_fused, whose warps share the spin-up pattern and so walk
+// its hops together.
+constexpr int kFusedThreads = 256;
+constexpr int kWideTps = 8;
+
+// an undirected bond: its two sites and the sites strictly between them
+struct alignas(8) BondMasks { uint32_t ends, between; };
+
+template <typename T>
+__global__ void __launch_bounds__(kFusedThreads) k_hv_fused_wide(const SpinK su, const SpinK sd, const HamK hk, const int nub,
+                                                  const uint32_t *__restrict__ st_up, const uint32_t *__restrict__ st_dn,
+                                                  const uint32_t *__restrict__ tab_up, const uint32_t *__restrict__ tab_dn,
+                                                  const uint32_t *__restrict__ gbinom, const BondMasks *__restrict__ gbonds,
+                                                  const T *__restrict__ gcoef, const T *__restrict__ dup,
+                                                  const T *__restrict__ ddn, const T *__restrict__ uv,
+                                                  const T *__restrict__ x, T *__restrict__ y) {
+    constexpr int TPS = kWideTps;
+    extern __shared__ __align__(16) uint32_t sm[];
+    uint32_t *tu = sm;
+    uint32_t *td = tu + pad4(su.tab_entries);
+    const int nb = (hk.L + 1) * (hk.L + 1);
+    uint32_t *binom = td + pad4(sd.tab_entries);
+    BondMasks *bonds = reinterpret_cast<BondMasks *>(binom + pad4(nb));
+    T *coef = reinterpret_cast<T *>(bonds + nub);
+    if (hk.rank_method == GBR_RANK_CNS) {
+        stage_u32(binom, gbinom, nb);
+    } else {
+        stage_packs(tu, tab_up, su.tab_entries);
+        stage_packs(td, tab_dn, sd.tab_entries);
+    }
+    for (int i = threadIdx.x; i < nub; i += kFusedThreads) {
+        bonds[i] = gbonds[i];
+        coef[i] = gcoef[i];
+    }
+    __syncthreads();
+    const int g = (int)(threadIdx.x % TPS);
+    const int64_t D = su.D * sd.D;
+    const int64_t stride = (int64_t)gridDim.x * (kFusedThreads / TPS);
+    const int64_t rounds = (D + stride - 1) / stride;   // every lane takes part in the butterfly
+    for (int64_t rnd = 0; rnd < rounds; ++rnd) {
+        const int64_t i = rnd * stride + (int64_t)blockIdx.x * (kFusedThreads / TPS) + threadIdx.x / TPS;
+        const bool live = i < D;
+        const int64_t ru = live ? (D <= 0xFFFFFFFFll ? (int64_t)((uint32_t)i / (uint32_t)sd.D) : i / sd.D) : 0;
+        const int64_t rd = live ? i - ru * sd.D : 0;
+        const uint32_t au = st_up[ru], ad = st_dn[rd];
+        T acc = 0;
+        if (live && g == 0) {
+            T dg = dup[ru] + ddn[rd];
+            for (int c = 0; c < hk.nucls; ++c) dg += uv[c] * (T)__popc(au & ad & hk.umask[c]);
+            acc = dg * x[i];
+        }
+        for (int e0 = 0; e0 < 2 * nub; e0 += 32 * TPS) {
+            // bit j: entry e0 + j TPS + g; an entry below nub is a spin-down bond
+            uint32_t act = 0;
+            const int left = (2 * nub - e0 - g + TPS - 1) / TPS, ne = left < 32 ? left : 32;
+            for (int j = 0; j < ne; ++j) {
+                const int e = e0 + j * TPS + g;
+                const bool dn = e < nub;
+                const uint32_t ends = bonds[dn ? e : e - nub].ends, m = (dn ? ad : au) & ends;
+                if (m != 0 && m != ends) act |= 1u << j;
+            }
+            if (!live) act = 0;
+            while (act) {
+                T c[2], v[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const bool on = act != 0;
+                    const int e = on ? e0 + (__ffs(act) - 1) * TPS + g : 0;
+                    act &= act - 1u;
+                    const bool dn = e < nub;
+                    const int b = dn ? e : e - nub;
+                    const BondMasks bm = bonds[b];
+                    const uint32_t a = dn ? ad : au;
+                    const uint32_t t = dn ? spin_rank(sd, hk.rank_method, td, binom, a ^ bm.ends)
+                                          : spin_rank(su, hk.rank_method, tu, binom, a ^ bm.ends);
+                    c[u] = (__popc(a & bm.between) & 1) ? -coef[b] : coef[b];
+                    v[u] = T(0);
+                    if (on) v[u] = x[dn ? ru * sd.D + (int64_t)t : (int64_t)t * sd.D + rd];
+                    else c[u] = T(0);
+                }
+                acc += c[0] * v[0];
+                acc += c[1] * v[1];
+            }
+        }
+#pragma unroll
+        for (int o = TPS / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        if (live && g == 0) y[i] = acc;
+    }
+}
+
 // ------------------------------------------------------------ factored path
 //
 // Y = H_up X + Dg o X + (H_dn X^T)^T.  Both off-diagonal products are row
@@ -261,61 +412,71 @@ __global__ void __launch_bounds__(256) k_hv_fused(const SpinK su, const SpinK sd
 // and consecutive CTAs share a column chunk so the gathered rows of that
 // chunk stay in L2.
 
-template <typename T, int TILE>
-__global__ void __launch_bounds__(TILE * 4) k_transpose(const T *__restrict__ in, T *__restrict__ out, int64_t rows,
-                                                        int64_t cols) {
-    __shared__ T tile[TILE][TILE + 1];
-    const int64_t c0 = (int64_t)blockIdx.x * TILE, r0 = (int64_t)blockIdx.y * TILE;
-    for (int i = threadIdx.y; i < TILE; i += blockDim.y) {
-        const int64_t r = r0 + i, c = c0 + threadIdx.x;
-        if (r < rows && c < cols) tile[i][threadIdx.x] = __ldcs(in + r * cols + c);
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < TILE; i += blockDim.y) {
-        const int64_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[c * rows + r] = tile[threadIdx.x][i];
-    }
-}
+// One 64 x 64 tile of the transpose by 256 threads.  PACKS: 16-byte packs on both
+// sides: the tile is read as row packs and written as packs of V consecutive
+// elements of one output row (V = 4 FP32, 2 FP64), which needs cols and rows multiples of V
+// and 16-byte aligned vectors; partial edge tiles, and everything without
+// PACKS, go element by element.
+constexpr int kTransposeTile = 64, kTransposeThreads = 256;
+template <typename T> struct TransposeTile { T e[kTransposeTile][kTransposeTile + 1]; };
 
-// The same transpose with 16-byte packs on both sides: a 64 x 64 tile is
-// read as row packs and written as packs of V consecutive elements of one
-// output row (V = 4 FP32, 2 FP64).  Needs cols and rows multiples of V and
-// 16-byte aligned vectors; partial edge tiles fall back to single elements.
-template <typename T>
-__global__ void __launch_bounds__(256) k_transpose16(const T *__restrict__ in, T *__restrict__ out, int64_t rows,
-                                                     int64_t cols) {
-    constexpr int TILE = 64, V = 16 / (int)sizeof(T), RP = TILE / V, PAD = 1;
+template <typename T, bool PACKS>
+__device__ __forceinline__ void transpose_block(const T *__restrict__ in, T *__restrict__ out, int64_t rows, int64_t cols,
+                                                int64_t tile_c, int64_t tile_r, TransposeTile<T> &tile) {
+    constexpr int TILE = kTransposeTile, V = PACKS ? 16 / (int)sizeof(T) : 1, RP = TILE / V;
     typedef typename Vec<T>::v4 P16;
-    __shared__ T tile[TILE][TILE + PAD];
-    const int64_t c0 = (int64_t)blockIdx.x * TILE, r0 = (int64_t)blockIdx.y * TILE;
+    const int64_t c0 = tile_c * TILE, r0 = tile_r * TILE;
     const bool full = r0 + TILE <= rows && c0 + TILE <= cols;
-    for (int idx = threadIdx.x; idx < TILE * RP; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < TILE * RP; idx += kTransposeThreads) {
         const int i = idx / RP, j = idx % RP;
         const int64_t r = r0 + i, c = c0 + (int64_t)j * V;
-        T o[V];
-        if (full) {
-            unpack16(__ldcs(reinterpret_cast<const P16 *>(in + r * cols + c)), o);
+        T o[PACKS ? 16 / (int)sizeof(T) : 1];
+        if (PACKS && full) {
+            if constexpr (PACKS) unpack16(__ldcs(reinterpret_cast<const P16 *>(in + r * cols + c)), o);
         } else {
 #pragma unroll
             for (int e = 0; e < V; ++e) o[e] = (r < rows && c + e < cols) ? __ldcs(in + r * cols + c + e) : T(0);
         }
 #pragma unroll
-        for (int e = 0; e < V; ++e) tile[i][j * V + e] = o[e];
+        for (int e = 0; e < V; ++e) tile.e[i][j * V + e] = o[e];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < TILE * RP; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < TILE * RP; idx += kTransposeThreads) {
         const int c = idx / RP, j = idx % RP;
-        T o[V];
+        T o[PACKS ? 16 / (int)sizeof(T) : 1];
 #pragma unroll
-        for (int e = 0; e < V; ++e) o[e] = tile[j * V + e][c];
+        for (int e = 0; e < V; ++e) o[e] = tile.e[j * V + e][c];
         const int64_t oc = c0 + c, orow = r0 + (int64_t)j * V;
-        if (full) {
-            *reinterpret_cast<P16 *>(out + oc * rows + orow) = pack16(o);
+        if (PACKS && full) {
+            if constexpr (PACKS) *reinterpret_cast<P16 *>(out + oc * rows + orow) = pack16(o);
         } else if (oc < cols) {
 #pragma unroll
             for (int e = 0; e < V; ++e)
                 if (orow + e < rows) out[oc * rows + orow + e] = o[e];
         }
+    }
+}
+
+template <typename T, bool PACKS>
+__global__ void __launch_bounds__(kTransposeThreads) k_transpose(const T *__restrict__ in, T *__restrict__ out, int64_t rows,
+                                                                 int64_t cols) {
+    __shared__ TransposeTile<T> tile;
+    transpose_block<T, PACKS>(in, out, rows, cols, blockIdx.x, blockIdx.y, tile);
+}
+
+// Hop lists and X^T, which do not depend on one another, in one launch: the first
+// ha.nblk blocks rank, the others transpose a tile each.
+// PREP_FIGURES
+template <typename T, bool PACKS>
+__global__ void __launch_bounds__(kTransposeThreads) k_prepare(const HopArgs ha, const HamK hk, const T *__restrict__ in,
+                                                               T *__restrict__ out, int64_t rows, int64_t cols,
+                                                               unsigned tiles_c) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    if ((int)blockIdx.x < ha.nblk) {
+        hop_lists_block(ha, hk, sm, (int)blockIdx.x);
+    } else {
+        const unsigned t = blockIdx.x - (unsigned)ha.nblk;
+        transpose_block<T, PACKS>(in, out, rows, cols, t % tiles_c, t / tiles_c, *reinterpret_cast<TransposeTile<T> *>(sm));
     }
 }
 
@@ -898,60 +1059,90 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
 
 struct HamDev {
     // precision-specific copies of the diagonal and coefficients
-    const void *dup, *ddn, *uval, *bcoef, *hcoef;
+    const void *dup, *ddn, *uval, *bcoef, *hcoef, *ucoef;
 };
-
-template <typename T>
-static int launch_hop_lists(const gbr_ham *H, const SpinSector &s, cudaStream_t st) {
-    const int R = H->rank_R[sizeof(T) == 8 ? 1 : 0];
-    const SpinK sk = spin_k(s, R);
-    const int nb = (H->L + 1) * (H->L + 1);
-    const size_t smem = (size_t)(sk.tab_entries + nb) * 4 + (size_t)H->L * H->L * 2 + 16;
-    const int threads = 128;
-    int64_t blocks = (s.D + threads - 1) / threads;
-    blocks = std::min<int64_t>(blocks, (int64_t)sm_count() * 8);
-    if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(k_hop_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_hop_lists<<<(int)std::max<int64_t>(blocks, 1), threads, smem, st>>>(
-        sk, H->k, s.states.as<uint32_t>(), spin_tab(s, R), H->binom.as<uint32_t>(),
-        reinterpret_cast<const uint16_t *>(H->bonds.p) + 2 * H->k.nbond, s.hop_cnt.as<uint16_t>(),
-        s.hop_tgt.as<uint32_t>(), s.hop_bond.as<uint16_t>(), s.hmax);
-    GBR_LAUNCH_CHECK();
-    const_cast<SpinSector &>(s).lists_ready = 1;
-    count_launches(1);
-    return GBR_OK;
-}
-
-template <typename T>
-static int launch_fused(const gbr_ham *H, const T *x, T *y, cudaStream_t st, const HamDev &hd) {
-    const int fpi = sizeof(T) == 8 ? 1 : 0;
-    const int R = H->rank_R[fpi], tps = H->fused_tps[fpi];
-    const SpinK su = spin_k(H->up, R), sd = spin_k(H->dn, R);
-    const int nb = (H->L + 1) * (H->L + 1);
-    const size_t smem = (size_t)(su.tab_entries + sd.tab_entries + nb + 1) * 4 + (size_t)H->L * H->L * sizeof(T) + 16;
-    const int threads = 256;
-    int64_t blocks = (H->D * tps + threads - 1) / threads;
-    blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * 8));
-    auto kern = tps == 4 ? k_hv_fused<T, 4> : (tps == 2 ? k_hv_fused<T, 2> : k_hv_fused<T, 1>);
-    if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(int)blocks, threads, smem, st>>>(su, sd, H->k, H->up.states.as<uint32_t>(), H->dn.states.as<uint32_t>(),
-                                             spin_tab(H->up, R), spin_tab(H->dn, R),
-                                             H->binom.as<uint32_t>(), (const T *)hd.hcoef, (const T *)hd.dup,
-                                             (const T *)hd.ddn, (const T *)hd.uval, x, y);
-    GBR_LAUNCH_CHECK();
-    count_launches(1);
-    return GBR_OK;
-}
 
 // When N_up == N_dn both spin species share one sector and one set of hop
 // lists (the hopping is spin independent).
 static const SpinSector &dn_lists(const gbr_ham *H) { return H->Nup == H->Ndn ? H->up : H->dn; }
 
+// Launch arguments and shared memory of the ranking pass.
+template <typename T>
+static int hop_args(const gbr_ham *H, HopArgs *ha, size_t *smem) {
+    const int R = H->rank_R[sizeof(T) == 8 ? 1 : 0];
+    const bool two = H->Nup != H->Ndn;
+    ha->s0 = spin_k(H->up, R);
+    ha->s1 = spin_k(H->dn, R);
+    auto out = [&](const SpinSector &s) {
+        return HopOut{s.states.as<uint32_t>(), spin_tab(s, R), s.hop_cnt.as<uint16_t>(), s.hop_tgt.as<uint32_t>(),
+                      s.hop_bond.as<uint16_t>(), s.hmax};
+    };
+    ha->o0 = out(H->up);
+    ha->o1 = out(H->dn);
+    auto blocks = [&](const SpinSector &s) { return (s.D * H->L + kHopThreads - 1) / kHopThreads; };
+    const int64_t b0 = blocks(H->up), b1 = two ? blocks(H->dn) : 0;
+    if (b0 + b1 > 0x3FFFFFFF) return set_error(GBR_EINVAL, "per-spin sectors too large for the ranking grid");
+    ha->nblk0 = (int)b0;
+    ha->nblk = (int)(b0 + b1);
+    ha->binom = H->binom.as<uint32_t>();
+    ha->bond_index = reinterpret_cast<const uint16_t *>(H->bonds.p) + 2 * H->k.nbond;
+    const int nb = (H->L + 1) * (H->L + 1), ent = std::max(ha->s0.tab_entries, ha->s1.tab_entries);
+    *smem = (size_t)(pad4(ent) + nb) * 4 + (size_t)H->L * H->L * 2 + 16;
+    return GBR_OK;
+}
+
+static void lists_done(const gbr_ham *H) {
+    const_cast<SpinSector &>(H->up).lists_ready = 1;
+    if (H->Nup != H->Ndn) const_cast<SpinSector &>(H->dn).lists_ready = 1;
+}
+
 template <typename T>
 static int stage_hop_lists(const gbr_ham *H, cudaStream_t st) {
-    int rc = launch_hop_lists<T>(H, H->up, st);
+    HopArgs ha;
+    size_t smem = 0;
+    int rc = hop_args<T>(H, &ha, &smem);
     if (rc) return rc;
-    if (H->Nup != H->Ndn) rc = launch_hop_lists<T>(H, H->dn, st);
-    return rc;
+    if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(k_hop_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_hop_lists<<<ha.nblk, kHopThreads, smem, st>>>(ha, H->k);
+    GBR_LAUNCH_CHECK();
+    lists_done(H);
+    count_launches(1);
+    return GBR_OK;
+}
+
+// Whether the fused path takes eight threads per element: no other number was
+// chosen for the handle, and the chip (2,048 threads a multiprocessor) holds them all.
+static bool fused_wide(const gbr_ham *H, int fpi) { return H->fused_tps[fpi] == 0 && H->D * kWideTps <= (int64_t)sm_count() * 2048; }
+
+template <typename T>
+static int launch_fused(const gbr_ham *H, const T *x, T *y, cudaStream_t st, const HamDev &hd) {
+    const int fpi = sizeof(T) == 8 ? 1 : 0;
+    const int R = H->rank_R[fpi], tps = std::max(1, H->fused_tps[fpi]);
+    const bool wide = fused_wide(H, fpi);
+    const SpinK su = spin_k(H->up, R), sd = spin_k(H->dn, R);
+    const int nb = (H->L + 1) * (H->L + 1), nub = H->k.nbond / 2;
+    const size_t tables = (size_t)(pad4(su.tab_entries) + pad4(sd.tab_entries) + pad4(nb)) * 4;
+    const size_t smem = tables + (wide ? (size_t)nub * (sizeof(BondMasks) + sizeof(T)) : (size_t)H->L * H->L * sizeof(T));
+    const int64_t per = kFusedThreads / (wide ? kWideTps : tps);
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((H->D + per - 1) / per, (int64_t)sm_count() * 8));
+    if (wide) {
+        auto kern = k_hv_fused_wide<T>;
+        if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<blocks, kFusedThreads, smem, st>>>(su, sd, H->k, nub, H->up.states.as<uint32_t>(), H->dn.states.as<uint32_t>(),
+                                                  spin_tab(H->up, R), spin_tab(H->dn, R), H->binom.as<uint32_t>(),
+                                                  H->ubonds.as<BondMasks>(), (const T *)hd.ucoef, (const T *)hd.dup,
+                                                  (const T *)hd.ddn, (const T *)hd.uval, x, y);
+    } else {
+        auto kern = tps == 4 ? k_hv_fused<T, 4> : (tps == 2 ? k_hv_fused<T, 2> : k_hv_fused<T, 1>);
+        if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<blocks, kFusedThreads, smem, st>>>(su, sd, H->k, H->up.states.as<uint32_t>(), H->dn.states.as<uint32_t>(),
+                                                  spin_tab(H->up, R), spin_tab(H->dn, R), H->binom.as<uint32_t>(),
+                                                  (const T *)hd.hcoef, (const T *)hd.dup, (const T *)hd.ddn,
+                                                  (const T *)hd.uval, x, y);
+    }
+    GBR_LAUNCH_CHECK();
+    count_launches(1);
+    return GBR_OK;
 }
 
 // scratch of the factored path: X^T and Z^T, owned by the handle unless the
@@ -972,7 +1163,7 @@ static int ensure_ws(const gbr_ham *H, size_t bytes) {
 // the partial-sum sizing of the fused Lanczos epilogue).
 template <typename T>
 static void gather_shape(const gbr_ham *H, int64_t Drows, int64_t Dcols, bool aligned16, bool combine, bool lz,
-                         int nt, int *vec_out, int *tr_out) {
+                         int nt, bool keep_vec, int *vec_out, int *tr_out) {
     const int fpi = sizeof(T) == 8 ? 1 : 0;
     const int vmax = sizeof(T) == 4 ? 4 : 2;
     // widest vector whose column chunk (the rows one wave of CTAs gathers
@@ -986,7 +1177,18 @@ static void gather_shape(const gbr_ham *H, int64_t Drows, int64_t Dcols, bool al
     const int tuned = lz ? H->tune_lz_rows[fpi] : (combine ? H->tune_up_rows[fpi] : H->tune_dn_rows[fpi]);
     // untuned default: 4 rows for the FP32 combine pass (its registers limit
     // occupancy; the tuner's pick on the 4x4 sector), 8 otherwise
-    const int tr_req = tuned ? tuned : ((combine && vec == 4) ? 4 : 8);
+    int tr_req = tuned ? tuned : ((combine && vec == 4) ? 4 : 8);
+    // FP64 on few rows or columns: single columns per thread and fewer rows until
+    // there are 32 warps a multiprocessor (untuned handles).  A warp's FP64
+    // operation occupies its scheduler's pipe for tens of clocks, so it takes
+    // warps to fill four of them: 731,808 states 116 -> 97 us, 853,776 states 56 ->
+    // 48 us, no difference from 3e6 states on; FP32 passes lose (2e6 states 33 -> 38 us).
+    if (sizeof(T) == 8 && !tuned && !keep_vec) {
+        const int64_t want = (int64_t)sm_count() * 32;
+        auto warps = [&](int v) { return (Drows + tr_req - 1) / tr_req * ((Dcols + nt * v - 1) / (nt * v)) * (nt / 32); };
+        while (vec > 1 && warps(vec) < want) vec /= 2;
+        if (tr_req == 8 && warps(vec) < want) tr_req = 4;
+    }
     *vec_out = vec;
     *tr_out = (tr_req == 4 || tr_req == 16) ? tr_req : 8;
 }
@@ -1074,7 +1276,7 @@ static int launch_gather(const gbr_ham *H, const SpinSector &lists, int64_t Drow
     int vec = 1, TR = 8;
     const int fpi = sizeof(T) == 8 ? 1 : 0;
     const int NT = H->gather_nt[MODE >= 2 ? 2 : MODE][fpi] == 64 ? 64 : 128;
-    gather_shape<T>(H, Drows, Dcols, aligned16, COMBINE, MODE >= 2, NT, &vec, &TR);
+    gather_shape<T>(H, Drows, Dcols, aligned16, COMBINE, MODE >= 2, NT, MODE == 3, &vec, &TR);
     if (MODE == 3 && vec != VM) {
         if (declined) *declined = true;
         return GBR_OK;
@@ -1120,6 +1322,12 @@ static int launch_gather(const gbr_ham *H, const SpinSector &lists, int64_t Drow
 }
 
 template <typename T>
+static bool transpose_packs(const T *x, const T *xt, int64_t Dup, int64_t Ddn) {
+    constexpr int V = 16 / (int)sizeof(T);
+    return ((((uintptr_t)x) | ((uintptr_t)xt)) & 15u) == 0 && Dup % V == 0 && Ddn % V == 0;
+}
+
+template <typename T>
 static int stage_transpose(const gbr_ham *H, const T *x, cudaStream_t st, const Scratch *ws = nullptr) {
     if (!ws) {
         int rc = ensure_ws(H, (size_t)H->D * sizeof(T));
@@ -1127,13 +1335,35 @@ static int stage_transpose(const gbr_ham *H, const T *x, cudaStream_t st, const 
     }
     T *xt = ws ? (T *)ws->xt : H->ws_xt.as<T>();
     const int64_t Dup = H->up.D, Ddn = H->dn.D;
-    constexpr int TILE = 64, V = 16 / (int)sizeof(T);
-    dim3 grid((unsigned)((Ddn + TILE - 1) / TILE), (unsigned)((Dup + TILE - 1) / TILE));
+    const dim3 grid((unsigned)((Ddn + kTransposeTile - 1) / kTransposeTile), (unsigned)((Dup + kTransposeTile - 1) / kTransposeTile));
     if (grid.y > 65535) return set_error(GBR_EINVAL, "sector too large for the transpose grid");
-    const bool packs = ((((uintptr_t)x) | ((uintptr_t)xt)) & 15u) == 0 && Dup % V == 0 && Ddn % V == 0;
-    if (packs) k_transpose16<T><<<grid, 256, 0, st>>>(x, xt, Dup, Ddn);
-    else k_transpose<T, TILE><<<grid, dim3(TILE, 4), 0, st>>>(x, xt, Dup, Ddn);
+    if (transpose_packs(x, xt, Dup, Ddn)) k_transpose<T, true><<<grid, kTransposeThreads, 0, st>>>(x, xt, Dup, Ddn);
+    else k_transpose<T, false><<<grid, kTransposeThreads, 0, st>>>(x, xt, Dup, Ddn);
     GBR_LAUNCH_CHECK();
+    count_launches(1);
+    return GBR_OK;
+}
+
+// the ranking pass and the transpose in one launch; *declined: the grid would be
+// too large (stage_hop_lists and stage_transpose then run one after the other)
+template <typename T>
+static int stage_prepare(const gbr_ham *H, const T *x, cudaStream_t st, const Scratch *ws, bool *declined) {
+    const int64_t Dup = H->up.D, Ddn = H->dn.D;
+    const int64_t tc = (Ddn + kTransposeTile - 1) / kTransposeTile, tr = (Dup + kTransposeTile - 1) / kTransposeTile;
+    HopArgs ha;
+    size_t smem = 0;
+    int rc = hop_args<T>(H, &ha, &smem);
+    if (rc) return rc;
+    *declined = tr > 65535 || tc * tr > 0x3FFFFFFF;
+    if (*declined) return GBR_OK;
+    if (!ws && (rc = ensure_ws(H, (size_t)H->D * sizeof(T)))) return rc;
+    T *xt = ws ? (T *)ws->xt : H->ws_xt.as<T>();
+    smem = std::max(smem, sizeof(TransposeTile<T>));
+    auto kern = transpose_packs(x, xt, Dup, Ddn) ? k_prepare<T, true> : k_prepare<T, false>;
+    if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<(unsigned)(ha.nblk + tc * tr), kTransposeThreads, smem, st>>>(ha, H->k, x, xt, Dup, Ddn, (unsigned)tc);
+    GBR_LAUNCH_CHECK();
+    lists_done(H);
     count_launches(1);
     return GBR_OK;
 }
@@ -1181,10 +1411,15 @@ static int launch_factored(const gbr_ham *H, const T *x, T *y, cudaStream_t st, 
                            cudaEvent_t *ev = nullptr, const Scratch *ws = nullptr, const LzHook *hook = nullptr,
                            int *nparts = nullptr, bool xt_ready = false, bool *updated = nullptr) {
     if (ev) cudaEventRecord(ev[0], st);
-    int rc = stage_hop_lists<T>(H, st);
-    if (rc) return rc;
-    if (ev) cudaEventRecord(ev[1], st);
-    if (!xt_ready && (rc = stage_transpose<T>(H, x, st, ws))) return rc;
+    int rc = GBR_OK;
+    bool declined = true;
+    // one launch for the first two stages unless their times are asked for
+    if (!ev && !xt_ready && (rc = stage_prepare<T>(H, x, st, ws, &declined))) return rc;
+    if (declined) {
+        if ((rc = stage_hop_lists<T>(H, st))) return rc;
+        if (ev) cudaEventRecord(ev[1], st);
+        if (!xt_ready && (rc = stage_transpose<T>(H, x, st, ws))) return rc;
+    }
     if (ev) cudaEventRecord(ev[2], st);
     if ((rc = stage_dn<T>(H, st, hd, ws))) return rc;
     if (ev) cudaEventRecord(ev[3], st);
@@ -1197,7 +1432,7 @@ static int launch_factored(const gbr_ham *H, const T *x, T *y, cudaStream_t st, 
 
 // Precision-specific device arrays hang off the handle as extra buffers.
 struct gbr_ham_prec {
-    gbr::DevBuf dup, ddn, uval, bcoef, hcoef;
+    gbr::DevBuf dup, ddn, uval, bcoef, hcoef, ucoef;
 };
 
 namespace gbr {
@@ -1207,7 +1442,7 @@ static gbr_ham_prec *prec_bufs(const gbr_ham *H, int fpi);
 int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, cudaEvent_t *ev) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
     int path = H->path;
     if (path == GBR_HV_AUTO) path = H->D <= (1 << 17) ? GBR_HV_FUSED : GBR_HV_FACTORED;
     if (path == GBR_HV_FUSED) {
@@ -1231,7 +1466,7 @@ int hv_launch_lz(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t 
                  int *nparts, bool xt_ready, bool *updated) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
     if (fp == 64)
         return launch_factored<double>(H, (const double *)x, (double *)y, st, hd, ev, nullptr, &hook, nparts, xt_ready,
                                        updated);
@@ -1256,7 +1491,7 @@ int64_t hv_lz_parts(const gbr_ham *H, int fp) {
 int hv_factored_with_scratch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, void *xt, void *zt) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
     const Scratch ws{xt, zt};
     if (fp == 64) return launch_factored<double>(H, (const double *)x, (double *)y, st, hd, nullptr, &ws);
     return launch_factored<float>(H, (const float *)x, (float *)y, st, hd, nullptr, &ws);
@@ -1274,7 +1509,7 @@ int hv_stage(const gbr_ham *H, const void *x, void *y, int fp, int stage, cudaSt
             return set_error(GBR_EINVAL, "stage %d before stage 2 (scratch) in this precision", stage);
     }
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
     if (fp == 64) {
         if (stage == 1) return stage_hop_lists<double>(H, st);
         if (stage == 2) return stage_transpose<double>(H, (const double *)x, st);
@@ -1303,6 +1538,7 @@ static int build_spin(gbr_ham *H, SpinSector &s, int N) {
         stag_fill(d, tab);
         if (d.wide) return set_error(GBR_EINVAL, "per-spin ranks exceed 32 bits");
         std::vector<uint32_t> t32(tab.begin(), tab.end());
+        t32.resize((t32.size() + 3) & ~(size_t)3, 0);   // whole 16-byte packs: the ranking pass reads those
         if ((rc = (R == 8 ? s.stag : s.stag4).upload(t32.data(), t32.size() * 4))) return rc;
     }
     std::vector<uint64_t> st;
@@ -1350,22 +1586,25 @@ static int upload_prec(gbr_ham *H, gbr_ham_prec *pb) {
     std::vector<double> dup((size_t)H->up.D), ddn((size_t)H->dn.D);
     GBR_CUDA_TRY(cudaMemcpy(dup.data(), H->up.diag.p, dup.size() * 8, cudaMemcpyDeviceToHost));
     GBR_CUDA_TRY(cudaMemcpy(ddn.data(), H->dn.diag.p, ddn.size() * 8, cudaMemcpyDeviceToHost));
-    std::vector<double> uv(kMaxUClasses, 0.0), bc, hc((size_t)H->L * H->L, 0.0);
+    std::vector<double> uv(kMaxUClasses, 0.0), bc, uc, hc((size_t)H->L * H->L, 0.0);
     for (int c = 0; c < H->k.nucls; ++c) uv[(size_t)c] = H->k.uval[c];
     for (int p = 0; p < H->L; ++p)
         for (int q = 0; q < H->L; ++q)
-            if (p != q) hc[(size_t)(p * H->L + q)] = H->h[(size_t)(p * H->L + q)];
-    for (int p = 0; p < H->L; ++p)
-        for (int q = 0; q < H->L; ++q)
-            if (p != q && H->h[(size_t)(p * H->L + q)] != 0.0) bc.push_back(H->h[(size_t)(p * H->L + q)]);
+            if (p != q && H->h[(size_t)(p * H->L + q)] != 0.0) {
+                bc.push_back(H->h[(size_t)(p * H->L + q)]);
+                hc[(size_t)(p * H->L + q)] = bc.back();
+                if (p < q) uc.push_back(bc.back());   // undirected, in the order of ubonds
+            }
     if (bc.empty()) bc.push_back(0.0);
+    if (uc.empty()) uc.push_back(0.0);
     int rc;
-    auto a = conv(dup), b = conv(ddn), u = conv(uv), c = conv(bc), h = conv(hc);
+    auto a = conv(dup), b = conv(ddn), u = conv(uv), c = conv(bc), h = conv(hc), o = conv(uc);
     if ((rc = pb->dup.upload(a.data(), a.size() * sizeof(T)))) return rc;
     if ((rc = pb->ddn.upload(b.data(), b.size() * sizeof(T)))) return rc;
     if ((rc = pb->uval.upload(u.data(), u.size() * sizeof(T)))) return rc;
     if ((rc = pb->bcoef.upload(c.data(), c.size() * sizeof(T)))) return rc;
     if ((rc = pb->hcoef.upload(h.data(), h.size() * sizeof(T)))) return rc;
+    if ((rc = pb->ucoef.upload(o.data(), o.size() * sizeof(T)))) return rc;
     return GBR_OK;
 }
 
@@ -1463,6 +1702,12 @@ extern "C" int gbr_ham_create(int L, const double *h, const double *U, int Nup, 
     std::vector<uint16_t> bonds_blob(pairs);
     bonds_blob.insert(bonds_blob.end(), bidx.begin(), bidx.end());
     int rc = H->bonds.upload(bonds_blob.data(), bonds_blob.size() * 2);
+    std::vector<BondMasks> ub;
+    for (int p = 0; p < L; ++p)
+        for (int q = p + 1; q < L; ++q)
+            if (h[p * L + q] != 0.0) ub.push_back({(1u << p) | (1u << q), ((1u << q) - 1u) & ~((2u << p) - 1u)});
+    if (ub.empty()) ub.push_back({0u, 0u});
+    if (!rc) rc = H->ubonds.upload(ub.data(), ub.size() * sizeof(BondMasks));
     std::vector<uint32_t> bin((size_t)(L + 1) * (L + 1));
     for (int n = 0; n <= L; ++n)
         for (int kk = 0; kk <= L; ++kk) bin[(size_t)(n * (L + 1) + kk)] = (uint32_t)binom(n, kk);
@@ -1553,7 +1798,7 @@ extern "C" int gbr_ham_set_shape(gbr_ham *H, int fp, const int *shape) {
         if (shape[i] != 0 && shape[i] != 64 && shape[i] != 128)
             return set_error(GBR_EINVAL, "threads per CTA %d must be 64 or 128", shape[i]);
     H->rank_R[fpi] = shape[4] ? shape[4] : 8;
-    H->fused_tps[fpi] = shape[5] ? shape[5] : 1;
+    H->fused_tps[fpi] = shape[5];
     H->gather_nt[0][fpi] = shape[6] ? shape[6] : 128;
     H->gather_nt[1][fpi] = shape[7] ? shape[7] : 128;
     H->gather_nt[2][fpi] = shape[8] ? shape[8] : 128;
@@ -1588,7 +1833,7 @@ extern "C" int gbr_ham_get_shape(const gbr_ham *H, int fp, int *shape) {
         shape[3] = plain(H->tune_lz_rows[fpi], 8);
     }
     shape[4] = H->rank_R[fpi];
-    shape[5] = H->fused_tps[fpi];
+    shape[5] = fused_wide(H, fpi) ? 0 : std::max(1, H->fused_tps[fpi]);   // 0: eight, by the rule
     for (int i = 0; i < 3; ++i) shape[6 + i] = on ? 256 : H->gather_nt[i][fpi];
     return GBR_OK;
 }
@@ -1746,7 +1991,8 @@ extern "C" int gbr_ham_tune(gbr_ham *H, int fp, void *stream) {
             float best_fu = 1e30f;
             int bR = 8, bT = 1;
             for (int R : {8, 4})
-                for (int tps : {1, 2, 4}) {
+                for (int tps : {0, 1, 2, 4}) {   // 0: the rule (eight in small sectors)
+                    if (tps == 0 && H->D * kWideTps > (int64_t)sm_count() * 2048) continue;
                     H->rank_R[fpi] = R;
                     H->fused_tps[fpi] = tps;
                     if ((rc = time_it(&ms))) goto done;
