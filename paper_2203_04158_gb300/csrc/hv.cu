@@ -124,7 +124,7 @@ __device__ __forceinline__ void stage_packs(uint32_t *s, const uint32_t *__restr
 // nblk0 blocks take s0).  A thread finds the place of its site's hops in the list
 // by counting those of the lower sites, a few instructions a site; a thread per
 // state ranked its ~10 to 30 hops one after the other on a handful of CTAs.
-// Bound: latency (table staging, one chain of look-ups).  HOPLIST_FIGURES
+// Bound: latency (table staging, one chain of look-ups): 12-site ring 4 us, against 13 us.
 constexpr int kHopThreads = 256;
 
 struct HopOut {
@@ -466,7 +466,8 @@ __global__ void __launch_bounds__(kTransposeThreads) k_transpose(const T *__rest
 
 // Hop lists and X^T, which do not depend on one another, in one launch: the first
 // ha.nblk blocks rank, the others transpose a tile each.
-// PREP_FIGURES
+// 731,808 states: 6.5 us, against 5.7 us for the transpose and 13 us for each species'
+// lists (a thread per state) one after the other.
 template <typename T, bool PACKS>
 __global__ void __launch_bounds__(kTransposeThreads) k_prepare(const HopArgs ha, const HamK hk, const T *__restrict__ in,
                                                                T *__restrict__ out, int64_t rows, int64_t cols,
@@ -520,10 +521,10 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
 // Row stride padding (elements) of the staged Z tile.  The tile is written
 // column by column, TR rows of one column from consecutive threads, so a warp
 // covers 32 / TR columns; a padding of 32 / TR FP32 elements puts all 32 in
-// different banks for TR = 4 and 8.  The rows stay 16-byte aligned for the
+// different banks for TR = 2, 4 and 8.  The rows stay 16-byte aligned for the
 // vector reads, so TR = 16 keeps 4 (two-way conflicts); FP64 keeps 16 bytes.
 __host__ __device__ constexpr int ztile_pad(int elem_bytes, int TR) {
-    return (elem_bytes == 4 && TR == 4) ? 8 : 16 / elem_bytes;
+    return (elem_bytes == 4 && TR <= 4) ? 32 / TR : 16 / elem_bytes;
 }
 
 struct CombineArgs {
@@ -1159,6 +1160,7 @@ static int ensure_ws(const gbr_ham *H, size_t bytes) {
     return rc;
 }
 
+constexpr int kGatherCtas = 6;
 // Vector width and rows per CTA of a gather pass (shared by the launch and
 // the partial-sum sizing of the fused Lanczos epilogue).
 template <typename T>
@@ -1178,19 +1180,22 @@ static void gather_shape(const gbr_ham *H, int64_t Drows, int64_t Dcols, bool al
     // untuned default: 4 rows for the FP32 combine pass (its registers limit
     // occupancy; the tuner's pick on the 4x4 sector), 8 otherwise
     int tr_req = tuned ? tuned : ((combine && vec == 4) ? 4 : 8);
-    // FP64 on few rows or columns: single columns per thread and fewer rows until
-    // there are 32 warps a multiprocessor (untuned handles).  A warp's FP64
-    // operation occupies its scheduler's pipe for tens of clocks, so it takes
-    // warps to fill four of them: 731,808 states 116 -> 97 us, 853,776 states 56 ->
-    // 48 us, no difference from 3e6 states on; FP32 passes lose (2e6 states 33 -> 38 us).
-    if (sizeof(T) == 8 && !tuned && !keep_vec) {
-        const int64_t want = (int64_t)sm_count() * 32;
-        auto warps = [&](int v) { return (Drows + tr_req - 1) / tr_req * ((Dcols + nt * v - 1) / (nt * v)) * (nt / 32); };
-        while (vec > 1 && warps(vec) < want) vec /= 2;
-        if (tr_req == 8 && warps(vec) < want) tr_req = 4;
+    // Few rows and columns (untuned handles): a CTA walks its rows one after the
+    // other, each a round of L2 latency, so rows are taken away while there are fewer
+    // than kGatherCtas CTAs a multiprocessor; and in FP64, where a warp's operation
+    // occupies its scheduler's pipe for tens of clocks and it takes warps to fill four
+    // of them, single columns per thread until there are 32 warps a multiprocessor
+    // (731,808 states 116 -> 97 us; FP32 passes lose by that: 2e6 states 33 -> 38 us).
+    // Two-row CTAs: 731,808 states 33 -> 22 us, 853,776 states 20 -> 15 us FP32.
+    if (!tuned && !keep_vec) {
+        auto ctas = [&](int v) { return (Drows + tr_req - 1) / tr_req * ((Dcols + nt * v - 1) / (nt * v)); };
+        const int64_t sms = sm_count();
+        if (sizeof(T) == 8)
+            while (vec > 1 && ctas(vec) * (nt / 32) < 32 * sms) vec /= 2;
+        while (tr_req > (lz ? 4 : 2) && ctas(vec) < kGatherCtas * sms) tr_req /= 2;
     }
     *vec_out = vec;
-    *tr_out = (tr_req == 4 || tr_req == 16) ? tr_req : 8;
+    *tr_out = (tr_req == 2 || tr_req == 4 || tr_req == 16) ? tr_req : 8;
 }
 
 // Shared memory of a windowed gather pass with TR rows per CTA.
@@ -1305,7 +1310,8 @@ static int launch_gather(const gbr_ham *H, const SpinSector &lists, int64_t Drow
     }
 #define GBR_GV(V)                                                                                            \
     {                                                                                                        \
-        if (TR == 4) GBR_GN(V, 4) else if (TR == 16) GBR_GN(V, 16) else GBR_GN(V, 8)                         \
+        if (TR == 4) GBR_GN(V, 4) else if (TR == 16) GBR_GN(V, 16)                                           \
+        else if (MODE <= 1 && TR == 2) GBR_GN(V, (MODE <= 1 ? 2 : 8)) else GBR_GN(V, 8)                      \
     }
     if constexpr (MODE == 3) {
         GBR_GV(VM)
@@ -1439,12 +1445,17 @@ namespace gbr {
 
 static gbr_ham_prec *prec_bufs(const gbr_ham *H, int fpi);
 
+// Largest sector that the automatic path gives to the fused kernel: 63,504 states
+// 10.1 us FP32 and 11.3 us FP64 there, 11.6 and 13.5 us in the factored path's three
+// launches, whose time hardly grows up to a few hundred thousand states.
+constexpr int64_t kFusedMax = (int64_t)1 << 16;
+
 int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, cudaEvent_t *ev) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
     HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
     int path = H->path;
-    if (path == GBR_HV_AUTO) path = H->D <= (1 << 17) ? GBR_HV_FUSED : GBR_HV_FACTORED;
+    if (path == GBR_HV_AUTO) path = H->D <= kFusedMax ? GBR_HV_FUSED : GBR_HV_FACTORED;
     if (path == GBR_HV_FUSED) {
         int rc;
         if (ev)
@@ -1459,7 +1470,7 @@ int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st,
 }
 
 bool hv_is_factored(const gbr_ham *H) {
-    return H->path == GBR_HV_FACTORED || (H->path == GBR_HV_AUTO && H->D > (1 << 17));
+    return H->path == GBR_HV_FACTORED || (H->path == GBR_HV_AUTO && H->D > kFusedMax);
 }
 
 int hv_launch_lz(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, cudaEvent_t *ev, const LzHook &hook,
