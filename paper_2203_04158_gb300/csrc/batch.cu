@@ -564,20 +564,14 @@ namespace gbr {
 static int g_batch_threads = kBatchThreads, g_batch_per_sm = 0;
 
 template <int NT>
-static int launch_batch(int grid_req_per_sm, int nsec, const SectorDesc *secs, const ModelDev *md, const double *d_start,
-                        const BatchLay &bl, int *ctr, double *E, int *Kout, DevBuf &dx, cudaStream_t st) {
+static int batch_grid(int grid_req_per_sm, int nsec, const BatchLay &bl, int *grid) {
     auto kern = k_batch<NT>;
     GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bl.bytes));
     int per_sm = 0;
     GBR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, (size_t)bl.bytes));
     per_sm = std::max(1, per_sm);
     if (grid_req_per_sm > 0) per_sm = std::min(per_sm, grid_req_per_sm);
-    const int grid = std::max(1, std::min<int>(nsec, sm_count() * per_sm));
-    int rc;
-    if ((rc = dx.alloc((size_t)grid * (size_t)bl.slot * 8))) return rc;
-    kern<<<grid, NT, (size_t)bl.bytes, st>>>(secs, md, d_start, bl, ctr, E, Kout, dx.as<double>());
-    GBR_LAUNCH_CHECK();
-    count_launches(1);
+    *grid = std::max(1, std::min<int>(nsec, sm_count() * per_sm));
     return GBR_OK;
 }
 
@@ -669,30 +663,38 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
     for (int c = 0; c <= kBatchClasses; ++c)
         bl.beg[c] = (int)std::count_if(cls.begin(), cls.end(), [&](int k) { return k < c; });
     for (size_t i = 0; i < idx.size(); ++i) order[i] = secs[(size_t)idx[i]];
-    DevBuf dsec, dmod, dE, dK, dctr, dx;
-    if ((rc = dsec.upload(order.data(), order.size() * sizeof(SectorDesc)))) return rc;
-    if ((rc = dmod.upload(md.data(), md.size() * sizeof(ModelDev)))) return rc;
-    if ((rc = dE.alloc(order.size() * 8))) return rc;
-    if ((rc = dK.alloc(order.size() * 4))) return rc;
-    if ((rc = dctr.alloc(16))) return rc;
-    GBR_CUDA_TRY(cudaMemsetAsync(dctr.p, 0, 16, st));
+    const int nsec = (int)order.size();
+    int grid = 1;
+    rc = threads == 128 ? batch_grid<128>(per_sm_req, nsec, bl, &grid)
+                        : (threads == 512 ? batch_grid<512>(per_sm_req, nsec, bl, &grid) : batch_grid<256>(per_sm_req, nsec, bl, &grid));
+    if (rc) return rc;
+    // one allocation: queue counters, sectors and models (copied together), results, scratch
+    auto r256 = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t at_sec = 256, at_mod = at_sec + r256(order.size() * sizeof(SectorDesc)),
+                 at_E = at_mod + r256(md.size() * sizeof(ModelDev)), at_K = at_E + r256(order.size() * 8),
+                 at_x = at_K + r256(order.size() * 4);
+    DevBuf dev_buf;
+    if ((rc = dev_buf.alloc(at_x + (size_t)grid * (size_t)bl.slot * 8))) return rc;
+    std::vector<unsigned char> blob(at_E, 0);
+    memcpy(blob.data() + at_sec, order.data(), order.size() * sizeof(SectorDesc));
+    memcpy(blob.data() + at_mod, md.data(), md.size() * sizeof(ModelDev));
+    unsigned char *dp = dev_buf.as<unsigned char>();
+    GBR_CUDA_TRY(cudaMemcpyAsync(dp, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
+    int *ctr = reinterpret_cast<int *>(dp), *dK = reinterpret_cast<int *>(dp + at_K);
+    const SectorDesc *dsec = reinterpret_cast<const SectorDesc *>(dp + at_sec);
+    const ModelDev *dmod = reinterpret_cast<const ModelDev *>(dp + at_mod);
+    double *dE = reinterpret_cast<double *>(dp + at_E), *dx = reinterpret_cast<double *>(dp + at_x);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ms_out) {
         GBR_CUDA_TRY(cudaEventCreate(&e0));
         GBR_CUDA_TRY(cudaEventCreate(&e1));
         cudaEventRecord(e0, st);
     }
-    const int nsec = (int)order.size();
-    if (threads == 128)
-        rc = launch_batch<128>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
-                               dE.as<double>(), dK.as<int>(), dx, st);
-    else if (threads == 512)
-        rc = launch_batch<512>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
-                               dE.as<double>(), dK.as<int>(), dx, st);
-    else
-        rc = launch_batch<256>(per_sm_req, nsec, dsec.as<SectorDesc>(), dmod.as<ModelDev>(), d_start, bl, dctr.as<int>(),
-                               dE.as<double>(), dK.as<int>(), dx, st);
-    if (rc) return rc;
+    if (threads == 128) k_batch<128><<<grid, 128, (size_t)bl.bytes, st>>>(dsec, dmod, d_start, bl, ctr, dE, dK, dx);
+    else if (threads == 512) k_batch<512><<<grid, 512, (size_t)bl.bytes, st>>>(dsec, dmod, d_start, bl, ctr, dE, dK, dx);
+    else k_batch<256><<<grid, 256, (size_t)bl.bytes, st>>>(dsec, dmod, d_start, bl, ctr, dE, dK, dx);
+    GBR_LAUNCH_CHECK();
+    count_launches(1);
     if (ms_out) {
         cudaEventRecord(e1, st);
         GBR_CUDA_TRY(cudaEventSynchronize(e1));
@@ -701,7 +703,7 @@ static int batch_run(int n_models, const gbr_model_desc *models, const double *d
         cudaEventDestroy(e1);
     }
     std::vector<double> E(order.size());
-    GBR_CUDA_TRY(cudaMemcpyAsync(E.data(), dE.p, E.size() * 8, cudaMemcpyDeviceToHost, st));
+    GBR_CUDA_TRY(cudaMemcpyAsync(E.data(), dE, E.size() * 8, cudaMemcpyDeviceToHost, st));
     GBR_CUDA_TRY(cudaStreamSynchronize(st));
     std::vector<double> Es(secs.size());
     for (size_t i = 0; i < idx.size(); ++i) Es[(size_t)idx[i]] = E[i];

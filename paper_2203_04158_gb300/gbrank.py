@@ -60,6 +60,8 @@ class ModelDesc(C.Structure):
 def lib():
     """The loaded library; raises if it was not built (no CPU fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -142,11 +144,38 @@ def _check(rc: int):
         raise GbrError(rc, gbr_last_error())
 
 
-def _stream(stream):
-    if stream is not None:
-        return C.c_void_p(stream if isinstance(stream, int) else stream.cuda_stream)
+# Per-call helpers.  A call on a small sector is as short as its marshalling, so
+# these stay off torch's Python layers: device pointers go to ctypes as plain
+# integers, and the current stream comes from the accessor torch's own launchers use.
+_torch = None
+_raw_stream = None
+_REALS = _PATTERNS = _DOUBLES = None
+_RANK_BITS: dict = {}
+
+
+def _load_torch():
+    global _torch, _raw_stream, _REALS, _PATTERNS, _DOUBLES
     import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    _RANK_BITS.update({torch.int32: 32, torch.int64: 64})
+    _REALS = {torch.float32: 32, torch.float64: 64}
+    _PATTERNS, _DOUBLES = (torch.int64,), (torch.float64,)
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _raw_stream = lambda: raw(dev())
+    else:
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+    _torch = torch
+    return torch
+
+
+def _stream(stream):
+    if stream is None:
+        if _raw_stream is None:
+            _load_torch()
+        if not _torch.cuda.is_initialized():
+            return _torch.cuda.current_stream().cuda_stream
+        return _raw_stream()
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def _dptr(t, dtypes=None):
@@ -157,7 +186,7 @@ def _dptr(t, dtypes=None):
         raise ValueError("expected a contiguous tensor")
     if dtypes is not None and t.dtype not in dtypes:
         raise ValueError(f"dtype {t.dtype} not in {dtypes}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _hptr(a: np.ndarray):
@@ -165,12 +194,30 @@ def _hptr(a: np.ndarray):
 
 
 def _rank_bits(t) -> int:
-    import torch
-    if t.dtype == torch.int32:
-        return 32
-    if t.dtype == torch.int64:
-        return 64
-    raise ValueError("rank tensors are int32 (32-bit ranks) or int64 (64-bit ranks)")
+    if _torch is None:
+        _load_torch()
+    bits = _RANK_BITS.get(t.dtype)
+    if bits is None:
+        raise ValueError("rank tensors are int32 (32-bit ranks) or int64 (64-bit ranks)")
+    return bits
+
+
+def _patterns(t):
+    if _torch is None:
+        _load_torch()
+    return _dptr(t, _PATTERNS)
+
+
+def _real_pair(x, y) -> int:
+    """32 or 64: the precision that x and y share."""
+    if _torch is None:
+        _load_torch()
+    if x.dtype != y.dtype:
+        raise ValueError("x and y must have the same dtype")
+    fp = _REALS.get(x.dtype)
+    if fp is None:
+        raise ValueError("x must be float32 or float64")
+    return fp
 
 
 class _Handle:
@@ -230,16 +277,12 @@ def gbr_comb_info(c: Comb):
 
 
 def gbr_comb_rank(c: Comb, pat, out, check: int = 0, stream=None):
-    import torch
-    _check(lib().gbr_comb_rank(c, _dptr(pat, (torch.int64,)), _dptr(out), _rank_bits(out), pat.numel(), int(check),
-                               _stream(stream)))
+    _check(lib().gbr_comb_rank(c, _patterns(pat), _dptr(out), _rank_bits(out), pat.numel(), int(check), _stream(stream)))
     return out
 
 
 def gbr_comb_unrank(c: Comb, rank, out, stream=None):
-    import torch
-    _check(lib().gbr_comb_unrank(c, _dptr(rank), _rank_bits(rank), _dptr(out, (torch.int64,)), rank.numel(),
-                                 _stream(stream)))
+    _check(lib().gbr_comb_unrank(c, _dptr(rank), _rank_bits(rank), _patterns(out), rank.numel(), _stream(stream)))
     return out
 
 
@@ -283,23 +326,17 @@ def gbr_trie_build_host(sorted_members: np.ndarray, M: int, R: int, msb_first: b
 
 
 def gbr_trie_rank(t: Trie, pat, out, check: int = 0, stream=None):
-    import torch
-    _check(lib().gbr_trie_rank(t, _dptr(pat, (torch.int64,)), _dptr(out), _rank_bits(out), pat.numel(), int(check),
-                               _stream(stream)))
+    _check(lib().gbr_trie_rank(t, _patterns(pat), _dptr(out), _rank_bits(out), pat.numel(), int(check), _stream(stream)))
     return out
 
 
 def gbr_trie_rank_bisect(t: Trie, pat, out, check: int = 0, stream=None):
-    import torch
-    _check(lib().gbr_trie_rank_bisect(t, _dptr(pat, (torch.int64,)), _dptr(out), _rank_bits(out), pat.numel(),
-                                      int(check), _stream(stream)))
+    _check(lib().gbr_trie_rank_bisect(t, _patterns(pat), _dptr(out), _rank_bits(out), pat.numel(), int(check), _stream(stream)))
     return out
 
 
 def gbr_trie_unrank(t: Trie, rank, out, stream=None):
-    import torch
-    _check(lib().gbr_trie_unrank(t, _dptr(rank), _rank_bits(rank), _dptr(out, (torch.int64,)), rank.numel(),
-                                 _stream(stream)))
+    _check(lib().gbr_trie_unrank(t, _dptr(rank), _rank_bits(rank), _patterns(out), rank.numel(), _stream(stream)))
     return out
 
 
@@ -370,24 +407,14 @@ def gbr_device_status(clear: bool = True) -> int:
 
 
 def gbr_hv(H: Ham, x, y, stream=None):
-    import torch
-    if x.dtype != y.dtype:
-        raise ValueError("x and y must have the same dtype")
-    fp = {torch.float32: 32, torch.float64: 64}.get(x.dtype)
-    if fp is None:
-        raise ValueError("x must be float32 or float64")
+    fp = _real_pair(x, y)
     _check(lib().gbr_hv(H, _dptr(x), _dptr(y), fp, _stream(stream)))
     return y
 
 
 def gbr_hv_static(H: Ham, x, y, stream=None):
     """gbr_hv that allocates nothing (scratch in a static device array)."""
-    import torch
-    if x.dtype != y.dtype:
-        raise ValueError("x and y must have the same dtype")
-    fp = {torch.float32: 32, torch.float64: 64}.get(x.dtype)
-    if fp is None:
-        raise ValueError("x must be float32 or float64")
+    fp = _real_pair(x, y)
     _check(lib().gbr_hv_static(H, _dptr(x), _dptr(y), fp, _stream(stream)))
     return y
 
@@ -407,14 +434,15 @@ def gbr_launch_count() -> int:
 
 def _lanczos(fn, handle, v0, iters, reorth, prec, refine, store_basis, use_graph, want_ritz, profile, tol,
              ritz_tail, stream) -> dict:
-    import torch
+    if _torch is None:
+        _load_torch()
     o = LanczosOpts(iters, int(bool(reorth)), prec, int(bool(refine)), store_basis, int(bool(use_graph)),
                     int(bool(profile)), float(tol), float(ritz_tail))
     r = LanczosResult()
     a = np.zeros(iters, dtype=np.float64)
     b = np.zeros(max(iters, 1), dtype=np.float64)
     rz = np.zeros(iters, dtype=np.float64) if want_ritz else None
-    _check(fn(handle, C.byref(o), _dptr(v0, (torch.float64,)), C.byref(r), _hptr(a), _hptr(b),
+    _check(fn(handle, C.byref(o), _dptr(v0, _DOUBLES), C.byref(r), _hptr(a), _hptr(b),
               None if rz is None else _hptr(rz), _stream(stream)))
     k = r.iters_done
     return dict(E0=r.E0, E_ritz=r.E_ritz, residual=r.residual, iters=k, breakdown=bool(r.breakdown),
@@ -468,12 +496,7 @@ def gbr_setham_set_bisect(S: SetHam, bisect: bool):
 
 
 def gbr_setham_hv(S: SetHam, x, y, check: int = 1, stream=None):
-    import torch
-    if x.dtype != y.dtype:
-        raise ValueError("x and y must have the same dtype")
-    fp = {torch.float32: 32, torch.float64: 64}.get(x.dtype)
-    if fp is None:
-        raise ValueError("x must be float32 or float64")
+    fp = _real_pair(x, y)
     _check(lib().gbr_setham_hv(S, _dptr(x), _dptr(y), fp, int(check), _stream(stream)))
     return y
 
@@ -513,48 +536,58 @@ def gbr_termham_info(T: TermHam):
 
 
 def gbr_termham_hv(T: TermHam, x, y, check: int = 1, stream=None):
-    import torch
-    if x.dtype != y.dtype:
-        raise ValueError("x and y must have the same dtype")
-    fp = {torch.float32: 32, torch.float64: 64}.get(x.dtype)
-    if fp is None:
-        raise ValueError("x must be float32 or float64")
+    fp = _real_pair(x, y)
     _check(lib().gbr_termham_hv(T, _dptr(x), _dptr(y), fp, int(check), _stream(stream)))
     return y
 
 
 # ---------------------------------------------------------------------- batch
 
+_MODEL = np.dtype([("L", np.int32), ("pad", np.int32), ("h", np.uint64), ("U", np.uint64)])
+
+
 def _models(models):
-    keep = []
-    arr = (ModelDesc * len(models))()
-    for i, (h, U) in enumerate(models):
-        h = np.ascontiguousarray(h, dtype=np.float64)
-        L = h.shape[0]
-        u = np.ascontiguousarray(np.zeros(L) if U is None else U, dtype=np.float64)
-        keep += [h, u]
-        arr[i] = ModelDesc(L, h.ctypes.data, u.ctypes.data)
-    return arr, keep
+    """The models as an array of ModelDesc (as bytes) and the buffers it points into."""
+    hs = [np.asarray(h, dtype=np.float64) for h, _ in models]
+    L = np.array([h.shape[0] for h in hs], dtype=np.int64)
+    us = [np.zeros(n) if U is None else np.asarray(U, dtype=np.float64).reshape(-1) for n, (_, U) in zip(L, models)]
+    hbuf = np.concatenate([h.reshape(-1) for h in hs]) if hs else np.zeros(0)
+    ubuf = np.concatenate(us) if us else np.zeros(0)
+    starts = lambda sizes: np.cumsum(sizes) - sizes
+    arr = np.zeros(len(hs), dtype=_MODEL)
+    arr["L"] = L
+    arr["h"] = hbuf.ctypes.data + 8 * starts(np.array([h.size for h in hs], dtype=np.int64))
+    arr["U"] = ubuf.ctypes.data + 8 * starts(np.array([u.size for u in us], dtype=np.int64))
+    return arr, (hbuf, ubuf)
+
+
+def _layout(arr):
+    ns, nst = C.c_int64(), C.c_int64()
+    _check(lib().gbr_batch_layout(len(arr), _hptr(arr), C.byref(ns), C.byref(nst)))
+    return ns.value, nst.value
 
 
 def gbr_batch_layout(models):
     arr, keep = _models(models)
-    ns, nst = C.c_int64(), C.c_int64()
-    _check(lib().gbr_batch_layout(len(models), arr, C.byref(ns), C.byref(nst)))
-    return ns.value, nst.value
+    return _layout(arr)
+
+
+def _batch_inputs(models, start):
+    if _torch is None:
+        _load_torch()
+    arr, keep = _models(models)
+    ns, nst = _layout(arr)
+    if start.numel() != nst:
+        raise ValueError(f"start has {start.numel()} entries, the batch has {nst} states")
+    return arr, keep, ns, _dptr(start, _DOUBLES)
 
 
 def gbr_batch_solve(models, start, iters: int, stream=None) -> dict:
-    import torch
-    arr, keep = _models(models)
-    ns, nst = gbr_batch_layout(models)
-    if start.numel() != nst:
-        raise ValueError(f"start has {start.numel()} entries, the batch has {nst} states")
+    arr, keep, ns, v0 = _batch_inputs(models, start)
     E0 = np.zeros(len(models))
     arg = np.zeros(2 * len(models), dtype=np.int32)
     sec = np.zeros(ns)
-    _check(lib().gbr_batch_solve(len(models), arr, _dptr(start, (torch.float64,)), iters, _hptr(E0), _hptr(arg),
-                                 _hptr(sec), _stream(stream)))
+    _check(lib().gbr_batch_solve(len(models), _hptr(arr), v0, iters, _hptr(E0), _hptr(arg), _hptr(sec), _stream(stream)))
     return dict(E0=E0, arg=arg.reshape(-1, 2), sector_E=sec)
 
 
@@ -569,13 +602,8 @@ def gbr_batch_get_shape() -> dict:
 
 
 def gbr_batch_tune(models, start, iters: int, stream=None) -> dict:
-    import torch
-    arr, keep = _models(models)
-    ns, nst = gbr_batch_layout(models)
-    if start.numel() != nst:
-        raise ValueError(f"start has {start.numel()} entries, the batch has {nst} states")
+    arr, keep, ns, v0 = _batch_inputs(models, start)
     sh = np.zeros(2, dtype=np.int32)
     ms = np.zeros(9, dtype=np.float32)
-    _check(lib().gbr_batch_tune(len(models), arr, _dptr(start, (torch.float64,)), iters, _hptr(sh), _hptr(ms),
-                                _stream(stream)))
+    _check(lib().gbr_batch_tune(len(models), _hptr(arr), v0, iters, _hptr(sh), _hptr(ms), _stream(stream)))
     return dict(threads=int(sh[0]), ctas_per_sm=int(sh[1]), candidate_ms=ms.tolist())
