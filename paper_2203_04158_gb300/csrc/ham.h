@@ -142,6 +142,23 @@ void *hv_xt_scratch(const gbr_ham *H, int fp);
 // upper bound of the partial sums hv_launch_lz writes for precision fp
 int64_t hv_lz_parts(const gbr_ham *H, int fp);
 
+// The hop lists of one spin species and everything of the H·v that a kernel
+// outside hv.cu needs to apply it to single elements (precision T = fp).
+struct HvLists {
+    const uint16_t *cnt;
+    const uint32_t *tgt;
+    const uint16_t *bond;
+};
+struct HvView {
+    HvLists up, dn;
+    HamK hk;
+    const uint32_t *st_up, *st_dn;
+    const void *dup, *ddn, *uval, *bcoef;
+    int Dup, Ddn;
+};
+// Ranks the hop lists on the stream and fills the view.
+int hv_view(const gbr_ham *H, int fp, cudaStream_t st, HvView *v);
+
 // The operator of a Lanczos solve: the sector Hamiltonian (whose factored
 // H·v carries the fused first update of each step), or any other operator
 // given as y = A x in precision fp (32 or 64) on a stream.

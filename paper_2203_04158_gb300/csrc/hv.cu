@@ -1469,6 +1469,25 @@ int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st,
     return launch_factored<float>(H, (const float *)x, (float *)y, st, hd, ev);
 }
 
+int hv_view(const gbr_ham *H, int fp, cudaStream_t st, HvView *v) {
+    const int rc = fp == 64 ? stage_hop_lists<double>(H, st) : stage_hop_lists<float>(H, st);
+    if (rc) return rc;
+    gbr_ham_prec *pb = prec_bufs(H, fp == 64 ? 1 : 0);
+    auto lists = [](const SpinSector &s) { return HvLists{s.hop_cnt.as<uint16_t>(), s.hop_tgt.as<uint32_t>(), s.hop_bond.as<uint16_t>()}; };
+    v->up = lists(H->up);
+    v->dn = lists(dn_lists(H));
+    v->hk = H->k;
+    v->st_up = H->up.states.as<uint32_t>();
+    v->st_dn = H->dn.states.as<uint32_t>();
+    v->dup = pb->dup.p;
+    v->ddn = pb->ddn.p;
+    v->uval = pb->uval.p;
+    v->bcoef = pb->bcoef.p;
+    v->Dup = (int)H->up.D;
+    v->Ddn = (int)H->dn.D;
+    return GBR_OK;
+}
+
 bool hv_is_factored(const gbr_ham *H) {
     return H->path == GBR_HV_FACTORED || (H->path == GBR_HV_AUTO && H->D > kFusedMax);
 }

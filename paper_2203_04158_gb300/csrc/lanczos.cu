@@ -630,6 +630,262 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
         v[i] = (T)((double)v[i] * inv);
 }
 
+// ------------------------------------- re-orthogonalised solve, one launch
+//
+// The whole recurrence with re-orthogonalisation of a small sector in one cooperative
+// launch.  Every CTA owns m consecutive elements of all vectors and walks through the
+// steps; what the CTAs need from one another goes through global memory between
+// grid barriers, five a step:
+//   gathers of H u_k (from the hop lists, ranked once a solve), first Gram-Schmidt
+//   pass: partial <w, u_j> | c_j, alpha_k | w -= sum c_j u_j, second pass: partials | c_j |
+//   w = u_{k+1} into its slot, partial <w, w> | beta.
+// Every CTA forms beta itself from the same partial sums in the same order.
+//
+// Bound: latency -- the barriers and the chains of FP64 operations (about 150 clocks
+// each when dependent) in the sums.  Thirteen launches a step, each of a few
+// microseconds, took 65 us a step on the 8-site ring (4,900 states, FP64).
+// REORTH_FIGURES
+//
+// 8 warps for the elements, one more for the scalars, which works while the others
+// gather.
+constexpr int kRoWarps = 8, kRoThreads = 32 * (kRoWarps + 1), kRoElems = 256;
+
+struct RoBarrier {
+    unsigned count;
+    int failed;       // a wait ran out: the solve is abandoned
+};
+
+// Grid barrier number `phase` (1, 2, ...) of a cooperative launch; false, once the wait
+// has run out (about a second) here or elsewhere.
+__device__ __forceinline__ bool grid_barrier(RoBarrier *b, unsigned phase) {
+    __shared__ int ok_s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned target = phase * gridDim.x;
+        __threadfence();
+        atomicAdd(&b->count, 1u);
+        int ok = 0;
+        for (int it = 0; it < (1 << 22); ++it) {
+            unsigned c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&b->count) : "memory");
+            if (c >= target) {
+                ok = 1;
+                break;
+            }
+            if (it > 256) __nanosleep(100);
+        }
+        if (!ok) atomicExch(&b->failed, 1);
+        __threadfence();
+        ok_s = ok;
+    }
+    __syncthreads();
+    return ok_s != 0;
+}
+
+// sum of v over the warps that own elements, by warp 0 (valid in its lane 0)
+__device__ __forceinline__ double ro_block_sum(double v, double *red) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if (lane == 0 && warp < kRoWarps) red[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < kRoWarps ? red[lane] : 0.0;
+        for (int o = kRoWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    }
+    return v;
+}
+
+// sum of p[0 .. n) by one warp (all lanes)
+__device__ __forceinline__ double ro_warp_sum(const double *p, int n) {
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(p + i);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const int n, const int m, const int tpe,
+                                                          const int iters, T *basis, double *alpha, double *beta, double *scal,
+                                                          LzState *st, double *npart, double *pdot,
+                                                          double *coef, RoBarrier *bar) {
+    __shared__ T ws[kRoElems];                      // this CTA's w
+    __shared__ T sub[kRoWarps * 32];
+    __shared__ double cs[kRoThreads], red[kRoWarps];
+    __shared__ double ig_s, scale_s, s_b;           // 1 / g_k; running scale; beta_k / g_{k-1}
+    __shared__ int stop_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = (int)gridDim.x, b = (int)blockIdx.x;
+    const int e0 = b * m, mine = max(0, min(m, n - e0));
+    const HamK &hk = hv.hk;
+    const bool worker = warp < kRoWarps;
+    // H·v: tpe threads an element; otherwise thread t owns element t
+    const int he = (int)threadIdx.x / tpe, hg = (int)threadIdx.x % tpe;
+    const bool hlive = worker && he < mine;
+    const int hi = e0 + (hlive ? he : 0), ru = hi / hv.Ddn, rd = hi - ru * hv.Ddn;
+    T dg = 0;
+    int nu = 0, nd = 0;
+    if (hlive) {
+        const uint32_t both = hv.st_up[ru] & hv.st_dn[rd];
+        dg = ((const T *)hv.dup)[ru] + ((const T *)hv.ddn)[rd];
+        for (int c = 0; c < hk.nucls; ++c) dg += ((const T *)hv.uval)[c] * (T)__popc(both & hk.umask[c]);
+        nu = hv.up.cnt[ru];
+        nd = hv.dn.cnt[rd];
+    }
+    const T *bc = (const T *)hv.bcoef;
+    const T hu = (T)hk.hu;
+    if (threadIdx.x == 0) {
+        ig_s = 1.0;
+        s_b = 0.0;
+        scale_s = 0.0;
+        stop_s = 0;
+    }
+    __syncthreads();
+    unsigned phase = 0;
+    int k = 0;
+    for (;; ++k) {
+        const T *u = basis + (int64_t)k * n;
+        // gathers; from step 1 on the scalar warp meanwhile finishes beta_k
+        T acc = 0;
+        if (hlive) {
+            if (hg == 0) acc = dg * u[hi];
+            for (int h = hg; h < nu; h += tpe) {
+                const uint32_t w = hv.up.tgt[(int64_t)h * hv.Dup + ru];
+                const T c = hk.uniform ? hu : bc[hv.up.bond[(int64_t)h * hv.Dup + ru]];
+                const T v = __ldcg(u + (int64_t)(w & 0x7FFFFFFFu) * hv.Ddn + rd);
+                acc += (w >> 31) ? -c * v : c * v;
+            }
+            for (int h = hg; h < nd; h += tpe) {
+                const uint32_t w = hv.dn.tgt[(int64_t)h * hv.Ddn + rd];
+                const T c = hk.uniform ? hu : bc[hv.dn.bond[(int64_t)h * hv.Ddn + rd]];
+                const T v = __ldcg(u + (int64_t)ru * hv.Ddn + (w & 0x7FFFFFFFu));
+                acc += (w >> 31) ? -c * v : c * v;
+            }
+        }
+        for (int o = tpe / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        if (hlive && hg == 0) ws[he] = acc;
+        if (!worker && k > 0) {
+            const double s = ro_warp_sum(npart, G);
+            if (lane == 0) {
+                const double bk = sqrt(fmax(s, 0.0)), igp = ig_s, sc = scale_s;
+                if (!isfinite(s)) stop_s = 3;
+                else if (k >= iters) stop_s = 1;
+                else if (bk <= 1e-13 * sc) stop_s = 2;
+                const double ig = 1.0 / bk;
+                if (isfinite(s)) {
+                    ig_s = ig;
+                    s_b = bk * igp;
+                    scale_s = fmax(sc, bk);
+                    if (b == 0) {
+                        beta[k] = bk;
+                        scal[kScal * k] = ig;
+                        scal[kScal * k + 1] = bk * igp;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (stop_s) break;
+        // w = H u_k / g_k - (beta_k / g_{k-1}) u_{k-1}
+        const int i = (int)threadIdx.x;
+        const bool live = i < mine;
+        T wi = 0;
+        if (live) {
+            wi = ws[i];
+            if (k > 0) wi = lz_rec((T)ig_s, wi, (T)s_b, basis[(int64_t)(k - 1) * n + e0 + i]);
+        }
+        if (live) ws[i] = wi;
+        // two Gram-Schmidt passes against u_0 .. u_k; the first one's <w, u_k> is g_k alpha_k
+        const int J = k + 1;
+        const int split = J <= 32 ? 8 : (J <= 64 ? 4 : (J <= 128 ? 2 : 1));   // threads a vector
+        for (int pass = 0; pass < 2; ++pass) {
+            __syncthreads();
+            if (worker)
+                for (int j0 = 0; j0 < J; j0 += kRoElems / split) {
+                    const int j = j0 + i / split, q = i % split;
+                    DotAcc<T> d0, d1, d2, d3;   // independent chains
+                    if (j < J) {
+                        const T *uj = basis + (int64_t)j * n + e0;
+                        int t = q;
+                        for (; t + 3 * split < mine; t += 4 * split) {
+                            d0.add(ws[t], uj[t]);
+                            d1.add(ws[t + split], uj[t + split]);
+                            d2.add(ws[t + 2 * split], uj[t + 2 * split]);
+                            d3.add(ws[t + 3 * split], uj[t + 3 * split]);
+                        }
+                        for (; t < mine; t += split) d0.add(ws[t], uj[t]);
+                    }
+                    double d = (d0.value() + d1.value()) + (d2.value() + d3.value());
+                    for (int o = split / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
+                    if (j < J && q == 0) pdot[(int64_t)j * G + b] = d;
+                }
+            if (!grid_barrier(bar, ++phase)) return;
+            if (worker)
+                for (int j = b * kRoWarps + warp; j < J; j += G * kRoWarps) {
+                    const double c = ro_warp_sum(pdot + (int64_t)j * G, G);
+                    const double g = __ldcg(scal + kScal * j);
+                    if (lane == 0) {
+                        coef[j] = c * g * g;
+                        if (pass == 0 && j == k) {
+                            alpha[k] = c * g;
+                            scal[kScal * k + 2] = c * g * g;
+                        }
+                    }
+                }
+            if (!grid_barrier(bar, ++phase)) return;
+            if (pass == 0) {
+                if (threadIdx.x == kRoThreads - 1) {
+                    const double a = __ldcg(alpha + k);
+                    scale_s = fmax(scale_s, fabs(a));
+                    if (!isfinite(a)) stop_s = 4;
+                }
+                __syncthreads();
+                if (stop_s) break;
+            }
+            // w -= sum_j c_j u_j, the vectors dealt to the threads of an element
+            const int mp = mine <= 32 ? 32 : (mine <= 64 ? 64 : (mine <= 128 ? 128 : 256)), Q = kRoElems / mp;
+            const int el = i % mp, q = i / mp;
+            T s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+            for (int j0 = 0; j0 < J; j0 += kRoThreads) {
+                __syncthreads();
+                if (j0 + i < J) cs[i] = __ldcg(coef + j0 + i);
+                __syncthreads();
+                if (worker && el < mine) {
+                    const T *ue = basis + (int64_t)j0 * n + e0 + el;
+                    const int je = min(kRoThreads, J - j0);
+                    int j = q;
+                    for (; j + 3 * Q < je; j += 4 * Q) {
+                        s0 += (T)cs[j] * ue[(int64_t)j * n];
+                        s1 += (T)cs[j + Q] * ue[(int64_t)(j + Q) * n];
+                        s2 += (T)cs[j + 2 * Q] * ue[(int64_t)(j + 2 * Q) * n];
+                        s3 += (T)cs[j + 3 * Q] * ue[(int64_t)(j + 3 * Q) * n];
+                    }
+                    for (; j < je; j += Q) s0 += (T)cs[j] * ue[(int64_t)j * n];
+                }
+            }
+            if (worker) sub[i] = (s0 + s1) + (s2 + s3);
+            __syncthreads();
+            if (live) {
+                for (int t = 0; t < Q; ++t) wi -= sub[t * mp + i];
+                ws[i] = wi;
+            }
+        }
+        if (stop_s) break;
+        // w is u_{k+1}
+        if (live) basis[(int64_t)(k + 1) * n + e0 + i] = wi;
+        const double s = ro_block_sum((double)wi * (double)wi, red);
+        if (threadIdx.x == 0) npart[b] = s;
+        if (!grid_barrier(bar, ++phase)) return;
+    }
+    // the step that stopped the recurrence: the one before, by its beta_k, or this
+    // one, by its alpha_k
+    if (b == 0 && threadIdx.x == 0) {
+        st->k = stop_s == 4 ? k : k - 1;
+        st->stop = 1;
+        st->breakdown = stop_s == 2;
+        st->nonfinite = stop_s >= 3;
+        st->scale = scale_s;
+    }
+}
+
 // ------------------------------------------------------------------ driver
 
 struct Lz {
@@ -780,6 +1036,44 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
     return GBR_OK;
 }
 
+// The re-orthogonalised recurrence in one cooperative launch (k_lz_reorth); *done false if the
+// sector is too large for it or the device does not take cooperative launches.
+template <typename T>
+static int lz_reorth(Lz &z, bool *done) {
+    *done = false;
+    const int sms = sm_count();
+    if (!z.op.ham || z.n > (int64_t)sms * kRoElems) return GBR_OK;
+    int dev = 0, coop = 0, per_sm = 0;
+    GBR_CUDA_TRY(cudaGetDevice(&dev));
+    GBR_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    GBR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lz_reorth<T>, kRoThreads, 0));
+    if (!coop || per_sm < 1) return GBR_OK;
+    // a CTA per multiprocessor, with at least a warp's worth of elements each
+    int m = (int)std::max<int64_t>(32, (z.n + sms - 1) / sms);
+    const int G = (int)((z.n + m - 1) / m);
+    int tpe = m <= 32 ? 8 : (m <= 64 ? 4 : (m <= 128 ? 2 : 1)), n = (int)z.n, iters = z.iters;
+    // partial sums: part holds grid x (iters + 1) of the launches it replaces
+    if ((int64_t)G * (z.iters + 2) + 2 > z.part_cap) return GBR_OK;
+    HvView hv;
+    int rc = hv_view(z.op.ham, z.fp, z.st, &hv);
+    if (rc) return rc;
+    double *npart = z.part.as<double>(), *pdot = npart + G, *alpha = z.alpha.as<double>(), *beta = z.beta.as<double>(),
+           *scal = z.scal.as<double>(), *coef = z.coef.as<double>();
+    RoBarrier *bar = reinterpret_cast<RoBarrier *>(pdot + (int64_t)G * z.iters);
+    LzState *st = z.state.as<LzState>();
+    T *basis = z.basis.as<T>();
+    GBR_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(*bar), z.st));
+    void *args[] = {&hv, &n, &m, &tpe, &iters, &basis, &alpha, &beta, &scal, &st, &npart, &pdot, &coef, &bar};
+    GBR_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)k_lz_reorth<T>, dim3(G), dim3(kRoThreads), args, 0, z.st));
+    count_launches(1);
+    RoBarrier hb{};
+    GBR_CUDA_TRY(cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, z.st));
+    GBR_CUDA_TRY(cudaStreamSynchronize(z.st));
+    if (hb.failed) return set_error(GBR_ETIMEOUT, "a grid barrier of the re-orthogonalised solve ran out");
+    *done = true;
+    return GBR_OK;
+}
+
 template <typename T>
 static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_lanczos_opts *o, double *h_alpha,
                   double *h_beta, double *h_ritz) {
@@ -827,7 +1121,9 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
     int rc = GBR_OK;
     int phase = 0;
     const bool want_ritz = h_ritz != nullptr;
-    for (int k = 0; k < z.iters; ++k) {
+    bool one_launch = false;
+    if (z.reorth && !want_ritz && !o->profile && z.tol == 0.0 && (rc = lz_reorth<T>(z, &one_launch))) return rc;
+    for (int k = 0; k < z.iters && !one_launch; ++k) {
         if (graphs && k >= 2) {
             if (!gexec[phase]) {
                 cudaStream_t keep = z.st;
@@ -1281,6 +1577,7 @@ int lanczos_solve(const LzOp &op, const gbr_lanczos_opts *o, const double *d_v0,
     if ((rc = grow(z.scal, sizeof(double) * kScal * (size_t)(z.iters + 2)))) return rc;
     size_t nparts = (size_t)z.grid * (size_t)(z.reorth ? z.iters + 1 : 1);
     if (op.ham) nparts = std::max(nparts, (size_t)hv_lz_parts(op.ham, z.fp));
+    if (z.reorth) nparts = std::max(nparts, (size_t)sm_count() * (size_t)(z.iters + 2) + 2);   // k_lz_reorth's
     z.part_cap = (int64_t)nparts;
     if ((rc = grow(z.part, sizeof(double) * (nparts + kReduceBlocks)))) return rc;
     if ((rc = grow(z.coef, sizeof(double) * (size_t)(z.iters + 2)))) return rc;

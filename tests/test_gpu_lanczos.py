@@ -43,6 +43,33 @@ def test_ring8_fp64_reorth_matches_dense_and_oracle(G):
     assert np.max(np.abs(r["ritz"] - o["ritz"])) <= 1e-9
 
 
+@pytest.mark.parametrize("kind,iters", [("two_states", 5), ("siam6", 290), ("ring8_35", 70), ("ring10_43", 40), ("ring10_55", 40)])
+def test_reorthogonalised_solve_in_one_launch(G, kind, iters):
+    """Sectors of a few states, below and above one warp of elements a CTA, at the
+    four and two threads an element of the hops, and one too large for the single
+    launch; recurrences longer than one block of coefficients (288)."""
+    if kind == "two_states":
+        L, h, U, Nu, Nd = 2, S.chain(2, pbc=False), S.uniform_U(2, 1.5), 1, 0
+    elif kind == "siam6":
+        h, U = S.siam(next(m for m in range(40) if S.siam(m)[0].shape[0] == 6))
+        L, Nu, Nd = 6, 3, 3
+    else:
+        L = 8 if kind.startswith("ring8") else 10
+        h, U, Nu, Nd = S.chain(L), S.uniform_U(L, 4.0), int(kind[-2]), int(kind[-1])
+    D = oracle.sector_dim(L, Nu, Nd)
+    H = G.gbr_ham_create(L, h, U, Nu, Nd)
+    n0 = G.gbr_launch_count()
+    r = G.gbr_lanczos(H, v0(D), iters, reorth=True, prec=G.GBR_PREC_FP64, refine=False)
+    assert (G.gbr_launch_count() - n0 < 12) == (kind != "ring10_55")
+    o = oracle.lanczos(L, h, U, Nu, Nd, S.start_vector(D), min(iters, D), True)
+    k = min(len(r["alpha"]), 60)
+    assert np.max(np.abs(r["alpha"][:k] - o["alpha"][:k])) <= 1e-9
+    assert np.max(np.abs(r["beta"][:k - 1] - o["beta"][:k - 1]), initial=0.0) <= 1e-9
+    assert abs(r["E_ritz"] - o["E0"]) <= 1e-10 * max(1.0, abs(o["E0"]))
+    m = G.gbr_lanczos(H, v0(D), iters, reorth=True, prec=G.GBR_PREC_MIXED, refine=True)
+    assert abs(m["E0"] - o["E0"]) <= (1e-9 if iters >= 70 or D < 500 else 1e-5) * max(1.0, abs(o["E0"]))
+
+
 def test_ring8_mixed_refined_meets_1e9(G):
     L, h, U, Nu, Nd = ring8()
     H = G.gbr_ham_create(L, h, U, Nu, Nd)
