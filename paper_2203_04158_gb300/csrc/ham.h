@@ -33,6 +33,8 @@ struct HamK {
     int nbond;                 // directed bonds (p, q), p != q, h_pq != 0
     int uniform;               // 1: every bond has the same coefficient
     double hu;                 // that coefficient
+    int ncabs;                 // distinct |h_pq| if there are one or two, else 0 ...
+    double cabs[2];            // ... and their values
     int rank_method;           // GBR_RANK_*
     int nucls;                 // U classes
     uint32_t umask[kMaxUClasses];

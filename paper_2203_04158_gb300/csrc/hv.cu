@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "ham.h"
 #include "dot.cuh"
@@ -536,6 +537,113 @@ struct CombineArgs {
     int zrow;                         // 1: the spin-down pass wrote Z row-major (window kernels)
 };
 
+// Sum of a row's hops in FP64, V columns a thread, mostly on the integer pipes.
+//
+// FP64 runs at two lanes a clock and multiprocessor here (the FP64 gathers took 87 %
+// of their time for one FMA a hop), the integer units at 64.  Where the hops have
+// at most two different |h_pq|, a hop's value only needs a sign before it is summed, and
+// the sums of the two classes meet their coefficients once a row.  So two of four
+// values (three, with a single class) are added as integers: relative to the largest
+// exponent E seen so far in the column, the 53-bit significand with three more bits below it is
+// shifted into place, signed and added to the 64-bit sum of its class (which is shifted
+// down when E grows); the others go to FP64 FMAs, which the integer work leaves time for.
+//
+// Bound: instruction issue (73 % of the slots), FP64 pipe 60 %.  4x4 torus with
+// diagonal hops (two classes, 35e6 states): 4.16 -> 2.56 ms; 14-site ring (11.8e6):
+// 510 -> 341 us.  All hops as integers: 3.48 ms and 360 us; one of four to FP64 with two
+// classes: 2.64 ms, two of four with one: 357 us.
+//
+// Error: a shift drops at most 2^-55 of the largest |x| of the sum (for values within
+// 2^3 of it, nothing), an FP64 addition rounds at 2^-53 of the running sum, so the sum
+// is at least as exact as the chain of FMAs it replaces.  Room: 53 + 3 bits and the sign leave 2^7 > kIntHops terms.
+// Infinities and NaN (E all ones) are left to the caller, which sums the row again in
+// FP64; denormals and zeros are exact.
+constexpr int kIntHops = 96;
+
+template <typename T> __device__ __forceinline__ bool int_sums(const HamK &hk, int hmax) {
+    return sizeof(T) == 8 && hk.ncabs > 0 && hmax <= kIntHops;
+}
+
+// a 2^ex rounded to nearest even, assembled with integer instructions (a conversion and
+// a scaling by FP64 ones cost as much as several hops)
+__device__ __forceinline__ double int_to_double(long long a, int ex) {
+    if (a == 0) return 0.0;
+    const unsigned long long mag = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int lz = __clzll((long long)mag), e = 63 - lz + ex + 1023;   // biased exponent
+    if (e < 1 || e > 2045) return scalbn((double)a, ex);
+    const unsigned long long norm = mag << lz;
+    const unsigned long long sig = (norm >> 11) + (((norm & 0x7FFull) + ((norm >> 11) & 1ull)) > 0x400ull ? 1ull : 0ull);
+    const unsigned long long bits = ((unsigned long long)(e - 1) << 52) + sig;   // the significand's top bit adds the one
+    return __longlong_as_double((long long)(bits | (a < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+template <int V, bool TWO> struct RowSum64 {
+    static constexpr int FMA = TWO ? 2 : 1;   // hops of four that go to the FMA
+    long long a0[V], a1[TWO ? V : 1];
+    int E[V];
+    double f[V];
+    __device__ __forceinline__ RowSum64() {
+#pragma unroll
+        for (int c = 0; c < V; ++c) {
+            a0[c] = 0;
+            if (TWO) a1[c] = 0;
+            E[c] = 0x00100000;
+            f[c] = 0.0;
+        }
+    }
+    // N hops: v[i][c] their values, w[i] the second class in bit 31, h[i] the signed coefficients;
+    // of four hops the last FMA go to FP64
+    template <int N> __device__ __forceinline__ void add(const double (&v)[N][V], const uint32_t *w, const double *h) {
+        constexpr int NI = N == 4 ? 4 - FMA : N;
+        uint32_t eight;   // opaque, so that the shift by three stays a multiplication, on the FMA pipe
+        asm volatile("mov.u32 %0, 8;" : "=r"(eight));
+#pragma unroll
+        for (int c = 0; c < V; ++c) {
+            int e = E[c];
+#pragma unroll
+            for (int i = 0; i < NI; ++i) e = max(e, __double2hiint(v[i][c]) & 0x7FF00000);
+            const int d = min((e - E[c]) >> 20, 63);
+            E[c] = e;
+            a0[c] >>= d;
+            if (TWO) a1[c] >>= d;
+            int n0 = 0, n1 = 0;   // minus the number of complemented terms of each class
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                const int hi = __double2hiint(v[i][c]), ex = hi & 0x7FF00000;
+                const uint32_t top = (uint32_t)((hi & 0x000FFFFF) | min(ex, 0x00100000));
+                unsigned long long sig = (unsigned long long)(uint32_t)__double2loint(v[i][c]) * eight;
+                sig += (unsigned long long)(top * eight) << 32;
+                const unsigned long long m = sig >> min((e - max(ex, 0x00100000)) >> 20, 63);
+                const int sg = (hi ^ __double2hiint(h[i])) >> 31;
+                const long long t = (long long)m ^ (long long)sg;
+                if (TWO && (w[i] >> 31)) {
+                    a1[c] += t;
+                    n1 += sg;
+                } else {
+                    a0[c] += t;
+                    n0 += sg;
+                }
+            }
+            a0[c] -= n0;
+            if (TWO) a1[c] -= n1;
+        }
+        if (N == 4)
+#pragma unroll
+            for (int i = NI; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < V; ++c) f[c] = fma(h[i < N ? i : 0], v[i < N ? i : 0][c], f[c]);
+    }
+    // the column's sum; false if a value was not finite
+    __device__ __forceinline__ bool finish(int c, const double *cabs, double *r) const {
+        const int ex = (E[c] >> 20) - 1023 - 52 - 3;   // exponent of the sums' unit
+        if (E[c] == 0x7FF00000) return false;
+        double s = fma(cabs[0], int_to_double(a0[c], ex), f[c]);
+        if (TWO) s = fma(cabs[1], int_to_double(a1[c], ex), s);
+        *r = s;
+        return true;
+    }
+};
+
 // MODE 0: Z = H_lists W.  MODE 1: y = H_up X + Dg o X + Z (combine).  MODE 2:
 // as 1, then the first update of a Lanczos step on unnormalised vectors
 // u_j = g_j v_j (g_0 = 1, g_j = beta_j) in the same epilogue,
@@ -550,8 +658,9 @@ struct CombineArgs {
 // sector: combine 1.16 ms (10 CTAs) against 1.21 ms (free) and 1.25 ms (16).
 // NT threads per CTA (128, or 64 for column chunks half as wide: the
 // gathered rows of a chunk then take half the L2).
+constexpr int kGather64 = 768;   // FP64: 80 registers
 template <typename T, int VEC, int MODE, int TR, int NT>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather(const int64_t Drows, const int64_t Dcols, const int hmax,
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : kGather64 / NT)) k_gather(const int64_t Drows, const int64_t Dcols, const int hmax,
                                                 const int64_t nrb, const uint16_t *__restrict__ cnt,
                                                 const uint32_t *__restrict__ tgt, const uint16_t *__restrict__ bond,
                                                 const T *__restrict__ bcoef, const int uniform, const T hu,
@@ -564,6 +673,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
     // hop-list row stride, a multiple of 4 so that four targets (and four
     // coefficients) are read with one 16-byte broadcast load
     const int hs = (hmax + 3) & ~3;
+    const bool ints = int_sums<T>(ca.hk, hmax), two = ca.hk.ncabs == 2;
     extern __shared__ __align__(128) unsigned char smr[];
     uint32_t *st = reinterpret_cast<uint32_t *>(smr);
     T *sc = reinterpret_cast<T *>(smr + (size_t)TR * hs * 4);
@@ -579,6 +689,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
     __shared__ uint32_t sau[TR];
     __shared__ T sdu[TR];
     __shared__ T suv[kMaxUClasses];
+    // FP64: U_c k for every number k of doubly occupied sites, a look-up instead of a
+    // conversion on the FP64 pipe
+    __shared__ T sut[COMBINE && sizeof(T) == 8 ? kMaxUClasses * (kMaxL + 1) : 1];
     const int64_t rb = blockIdx.x % nrb, cc = blockIdx.x / nrb;
     const int64_t r0 = rb * TR;
     const int nrow = (int)((Drows - r0) < (int64_t)TR ? (Drows - r0) : (int64_t)TR);
@@ -628,6 +741,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
     }
     if (COMBINE && threadIdx.x < kMaxUClasses)
         suv[threadIdx.x] = threadIdx.x < ca.hk.nucls ? ((const T *)ca.uval)[threadIdx.x] : T(0);
+    if (COMBINE && sizeof(T) == 8)
+        for (int e = threadIdx.x; e < ca.hk.nucls * (kMaxL + 1); e += blockDim.x)
+            sut[e] = ((const T *)ca.uval)[e / (kMaxL + 1)] * (T)(e % (kMaxL + 1));
     __syncthreads();
     for (int e = threadIdx.x; e < TR * hmax; e += blockDim.x) {
         const int i = e % TR, k = e / TR;
@@ -635,7 +751,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
             const int64_t g = (int64_t)k * Drows + r0 + i;
             const uint32_t w = tgt[g];
             const T c = uniform ? hu : bcoef[bond[g]];
-            st[i * hs + k] = w & 0x7FFFFFFFu;
+            // FP64 sums by classes: bit 31 of the staged target is the class
+            const uint32_t cls = ints && two && fabs((double)c) != ca.hk.cabs[0] ? 0x80000000u : 0u;
+            st[i * hs + k] = (w & 0x7FFFFFFFu) | cls;
             sc[i * hs + k] = (w >> 31) ? -c : c;
         }
     }
@@ -697,6 +815,48 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
                 }
             }
             acc[0] = a4.x; acc[1] = a4.y; acc[2] = a4.z; acc[3 % VEC] = a4.w;
+        } else if (sizeof(T) == 8 && ints) {
+            if constexpr (sizeof(T) == 8) {
+                auto load = [&](uint32_t t, double *o) {
+                    const T *p = x + (int64_t)(t & 0x7FFFFFFFu) * Dcols + c0;
+                    if constexpr (VEC == 2) {
+                        const double2 q = __ldcg(reinterpret_cast<const double2 *>(p));
+                        o[0] = q.x;
+                        o[1] = q.y;
+                    } else {
+                        o[0] = __ldcg(p);
+                    }
+                };
+                auto sum = [&](auto classes) {
+                    RowSum64<VEC, decltype(classes)::value> rs;
+                    int k = 0;
+                    for (; k + 4 <= n; k += 4) {
+                        const uint4 t4 = *reinterpret_cast<const uint4 *>(ti + k);
+                        const uint32_t w[4] = {t4.x, t4.y, t4.z, t4.w};
+                        double v[4][VEC], h[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) load(w[u], v[u]);
+                        *reinterpret_cast<double2 *>(h) = *reinterpret_cast<const double2 *>(ci + k);
+                        *reinterpret_cast<double2 *>(h + 2) = *reinterpret_cast<const double2 *>(ci + k + 2);
+                        rs.template add<4>(v, w, h);
+                    }
+                    for (; k < n; ++k) {
+                        double v[1][VEC];
+                        const double h = ci[k];
+                        load(ti[k], v[0]);
+                        rs.template add<1>(v, ti + k, &h);
+                    }
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v)
+                        if (!rs.finish(v, ca.hk.cabs, reinterpret_cast<double *>(&acc[v]))) {
+                            T a = 0;
+                            for (int q = 0; q < n; ++q) a += ci[q] * __ldcg(x + (int64_t)(ti[q] & 0x7FFFFFFFu) * Dcols + c0 + v);
+                            acc[v] = a;
+                        }
+                };
+                if (two) sum(std::true_type{});
+                else sum(std::false_type{});
+            }
         } else if (VEC == 2) {
             T a0 = 0, a1 = 0;
 #pragma unroll 4
@@ -744,7 +904,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : 1)) k_gather
 #pragma unroll
                 for (int u = 0; u < kMaxUClasses; ++u) {
                     if (u >= ca.hk.nucls) break;
-                    dg += suv[u] * (T)__popc(both & ca.hk.umask[u]);
+                    if (sizeof(T) == 8) dg += sut[u * (kMaxL + 1) + __popc(both & ca.hk.umask[u])];
+                    else dg += suv[u] * (T)__popc(both & ca.hk.umask[u]);
                 }
                 acc[v] += dg * xo[v] + zv[v];
             }
@@ -887,12 +1048,14 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
     typedef typename WinVec<T>::V V;
     // padded hop-list stride (multiple of 4: four targets per 16-byte load)
     const int hs = (hmax + 3) & ~3;
+    const bool ints = int_sums<T>(ca.hk, hmax), two = ca.hk.ncabs == 2;
     extern __shared__ __align__(128) unsigned char smr[];
     T *win = reinterpret_cast<T *>(smr);
     uint32_t *st = reinterpret_cast<uint32_t *>(smr + win_region_bytes<T, TR>());
     T *sc = reinterpret_cast<T *>(smr + win_region_bytes<T, TR>() + (size_t)TR * hs * 4);
     __shared__ int scnt[TR];
     __shared__ T suv[kMaxUClasses];
+    __shared__ T sut[COMBINE && sizeof(T) == 8 ? kMaxUClasses * (kMaxL + 1) : 1];
     __shared__ __align__(8) uint64_t bar;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t rb = blockIdx.x % nrb, cc = blockIdx.x / nrb;
@@ -925,6 +1088,9 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
     for (int i = threadIdx.x; i < TR; i += blockDim.x) scnt[i] = (i < nrow) ? (int)cnt[r0 + i] : 0;
     if (COMBINE && threadIdx.x < kMaxUClasses)
         suv[threadIdx.x] = threadIdx.x < ca.hk.nucls ? ((const T *)ca.uval)[threadIdx.x] : T(0);
+    if (COMBINE && sizeof(T) == 8)
+        for (int e = threadIdx.x; e < ca.hk.nucls * (kMaxL + 1); e += blockDim.x)
+            sut[e] = ((const T *)ca.uval)[e / (kMaxL + 1)] * (T)(e % (kMaxL + 1));
     __syncthreads();
     for (int e = threadIdx.x; e < TR * hmax; e += blockDim.x) {
         const int i = e % TR, k = e / TR;
@@ -932,7 +1098,9 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
             const int64_t g = (int64_t)k * Drows + r0 + i;
             const uint32_t w = tgt[g];
             const T c = uniform ? hu : bcoef[bond[g]];
-            st[i * hs + k] = w & 0x7FFFFFFFu;
+            // FP64 sums by classes: bit 31 of the staged target is the class
+            const uint32_t cls = ints && two && fabs((double)c) != ca.hk.cabs[0] ? 0x80000000u : 0u;
+            st[i * hs + k] = (w & 0x7FFFFFFFu) | cls;
             sc[i * hs + k] = (w >> 31) ? -c : c;
         }
     }
@@ -980,6 +1148,37 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
                                            : reinterpret_cast<const V *>(xs + (int64_t)t * Dcols);
             };
             int k = 0;
+            if (sizeof(T) == 8 && ints) {
+                if constexpr (sizeof(T) == 8) {
+                    auto sum = [&](auto classes) {
+                        RowSum64<VEC, decltype(classes)::value> rs;
+                        for (; k + 4 <= n; k += 4) {
+                            const uint4 t4 = *reinterpret_cast<const uint4 *>(ti + k);
+                            const uint32_t w[4] = {t4.x, t4.y, t4.z, t4.w};
+                            double v[4][VEC], h[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) WinVec<T>::get(v[u], *row(w[u] & 0x7FFFFFFFu));
+                            WinVec<T>::coef4(h, ci + k);
+                            rs.template add<4>(v, w, h);
+                        }
+                        for (; k < n; ++k) {
+                            double v[1][VEC];
+                            const double h = ci[k];
+                            WinVec<T>::get(v[0], *row(ti[k] & 0x7FFFFFFFu));
+                            rs.template add<1>(v, ti + k, &h);
+                        }
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v)
+                            if (!rs.finish(v, ca.hk.cabs, reinterpret_cast<double *>(&acc[v]))) {
+                                T a = 0;
+                                for (int q = 0; q < n; ++q) a += ci[q] * reinterpret_cast<const T *>(row(ti[q] & 0x7FFFFFFFu))[v];
+                                acc[v] = a;
+                            }
+                    };
+                    if (two) sum(std::true_type{});
+                    else sum(std::false_type{});
+                }
+            }
 #pragma unroll 2
             for (; k + 4 <= n; k += 4) {
                 const uint4 t4 = *reinterpret_cast<const uint4 *>(ti + k);
@@ -1006,7 +1205,8 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
 #pragma unroll
                     for (int u = 0; u < kMaxUClasses; ++u) {
                         if (u >= ca.hk.nucls) break;
-                        dg += suv[u] * (T)__popc(both & ca.hk.umask[u]);
+                        if (sizeof(T) == 8) dg += sut[u * (kMaxL + 1) + __popc(both & ca.hk.umask[u])];
+                        else dg += suv[u] * (T)__popc(both & ca.hk.umask[u]);
                     }
                     acc[v] += dg * xo[v] + zv[v];
                 }
@@ -1378,6 +1578,7 @@ static int stage_prepare(const gbr_ham *H, const T *x, cudaStream_t st, const Sc
 template <typename T>
 static int stage_dn(const gbr_ham *H, cudaStream_t st, const HamDev &hd, const Scratch *ws = nullptr) {
     CombineArgs ca{};
+    ca.hk = H->k;
     T *xt = ws ? (T *)ws->xt : H->ws_xt.as<T>();
     T *zt = ws ? (T *)ws->zt : H->ws_zt.as<T>();
     return launch_gather<T, 0>(H, dn_lists(H), H->dn.D, H->up.D, xt, zt, ca, st, hd);
@@ -1662,6 +1863,17 @@ int build_hamk(int L, const double *h, const double *U, int rank_method, HamK *k
             ++k.nbond;
         }
     k.hu = first;
+    for (int p = 0; p < L && k.ncabs >= 0; ++p)
+        for (int q = 0; q < L; ++q) {
+            const double v = fabs(h[p * L + q]);
+            if (p == q || v == 0.0 || (k.ncabs > 0 && v == k.cabs[0]) || (k.ncabs > 1 && v == k.cabs[1])) continue;
+            if (k.ncabs == 2) {
+                k.ncabs = -1;
+                break;
+            }
+            k.cabs[k.ncabs++] = v;
+        }
+    if (k.ncabs < 0) k.ncabs = 0;
     for (int p = 0; p < L; ++p) {
         const double u = U ? U[p] : 0.0;
         if (u == 0.0) continue;

@@ -296,3 +296,69 @@ def test_quarter_filled_open_chain_sampled_rows(G, fp):
             y = torch.empty_like(x)
             G.gbr_hv(H, x, y)
             assert rel_inf(y[idx].double().cpu().numpy(), y_ref) <= tol, (path, R)
+
+
+@pytest.mark.parametrize("kind", ["wide", "tiny", "zeros", "nonfinite"])
+@pytest.mark.parametrize("model_", ["two_classes", "one_class"])
+def test_fp64_class_sums_over_the_whole_range(G, kind, model_):
+    """The FP64 gathers sum hops of one or two coefficient magnitudes as aligned
+    integers: vectors over 200 decades, denormals, mostly zeros, and with
+    infinities and NaN, on both vector widths (even and odd per-spin sectors) and
+    both gather families.  Every element within 2^-50 of its own sum of
+    magnitudes (an FMA chain of up to 40 terms stays within 40 * 2^-53)."""
+    import torch
+    L = 9
+    h = S.square(3, 3, 1.0, -0.3) if model_ == "two_classes" else S.chain(9)
+    h = h + np.diag(np.linspace(-0.5, 0.5, L))
+    U = S.uniform_U(L, 4.0)
+    for Nu, Nd in ((4, 4), (4, 2)):
+        D = oracle.sector_dim(L, Nu, Nd)
+        rng = np.random.default_rng(5)
+        x = rng.uniform(-1, 1, D)
+        if kind == "wide":
+            x *= 10.0 ** rng.uniform(-100, 100, D)
+        elif kind == "tiny":
+            x *= 2.0 ** rng.integers(-60, 4, D) * 2.0 ** -1030
+        elif kind == "zeros":
+            x[rng.random(D) < 0.97] = 0.0
+        else:
+            x[[3, D // 2]] = np.inf
+            x[D // 3] = np.nan
+        with np.errstate(invalid="ignore"):
+            ref = oracle.hv(L, h, U, Nu, Nd, x)
+        mats = []
+        for N in (Nu, Nd):     # sum of |h x| without the fermion signs
+            st = oracle.enumerate_sector(L, N).astype(np.int64)
+            m = np.zeros((st.size, st.size))
+            for i, a in enumerate(st):
+                m[i, i] = sum(abs(h[p, p]) for p in range(L) if a >> p & 1)
+                for p in range(L):
+                    for q in range(L):
+                        if p != q and h[p, q] and a >> p & 1 and not a >> q & 1:
+                            m[i, np.searchsorted(st, a ^ (1 << p) ^ (1 << q))] = abs(h[p, q])
+            mats.append(m)
+        H = G.gbr_ham_create(L, h, U, Nu, Nd)
+        G.gbr_ham_set_path(H, G.GBR_HV_FACTORED)
+        xd = torch.from_numpy(x).cuda()
+        outs = []
+        for shape in (dict(window=0), dict(window=1), dict(window=0, rows_dn=4, rows_up=16, threads_dn=64)):
+            G.gbr_ham_set_shape(H, 64, **shape)
+            y = torch.full_like(xd, 7.0)
+            G.gbr_hv(H, xd, y)
+            outs.append(y.cpu().numpy())
+        for o in outs[1:]:
+            assert np.array_equal(o, outs[0], equal_nan=True)
+        if kind == "nonfinite":
+            # the per-element kernel forms the same products (0 * inf on the diagonal among them)
+            G.gbr_ham_set_path(H, G.GBR_HV_FUSED)
+            y = torch.empty_like(xd)
+            G.gbr_hv(H, xd, y)
+            ref = y.cpu().numpy()
+            assert np.array_equal(np.isnan(outs[0]), np.isnan(ref))
+            ok = np.isfinite(ref)
+            assert np.array_equal(np.isfinite(outs[0]), ok)
+            assert np.max(np.abs(outs[0][ok] - ref[ok])) <= 1e-12
+            continue
+        X = np.abs(x).reshape(mats[0].shape[0], mats[1].shape[0])
+        total = (mats[0] @ X + X @ mats[1].T + 4.0 * min(Nu, Nd) * X).ravel()
+        assert np.all(np.abs(outs[0] - ref) <= 2.0 ** -49 * total + 2.0 ** -1070), kind
