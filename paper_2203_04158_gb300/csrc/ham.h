@@ -90,9 +90,6 @@ struct gbr_ham {
     gbr::HamK k;
     gbr::SpinSector up, dn;
     gbr::DevBuf bonds;         // nbond x {p, q} uint8 pairs (as uint16), bond order
-    gbr::DevBuf bond_coef64;   // nbond doubles
-    gbr::DevBuf bond_coef32;   // nbond floats
-    gbr::DevBuf ubonds;        // undirected bonds p < q as masks (fused path)
     gbr::DevBuf binom;         // (L+1) x (L+1) uint32 binomials (CNS ranking)
     // tuned launch shape (0 = default): rows per CTA of the gather passes
     int tune_up_rows[2] = {0, 0};

@@ -1260,7 +1260,7 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
 
 struct HamDev {
     // precision-specific copies of the diagonal and coefficients
-    const void *dup, *ddn, *uval, *bcoef, *hcoef, *ucoef;
+    const void *dup, *ddn, *uval, *bcoef, *hcoef, *ucoef, *ubonds;
 };
 
 // When N_up == N_dn both spin species share one sector and one set of hop
@@ -1331,7 +1331,7 @@ static int launch_fused(const gbr_ham *H, const T *x, T *y, cudaStream_t st, con
         if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<blocks, kFusedThreads, smem, st>>>(su, sd, H->k, nub, H->up.states.as<uint32_t>(), H->dn.states.as<uint32_t>(),
                                                   spin_tab(H->up, R), spin_tab(H->dn, R), H->binom.as<uint32_t>(),
-                                                  H->ubonds.as<BondMasks>(), (const T *)hd.ucoef, (const T *)hd.dup,
+                                                  (const BondMasks *)hd.ubonds, (const T *)hd.ucoef, (const T *)hd.dup,
                                                   (const T *)hd.ddn, (const T *)hd.uval, x, y);
     } else {
         auto kern = tps == 4 ? k_hv_fused<T, 4> : (tps == 2 ? k_hv_fused<T, 2> : k_hv_fused<T, 1>);
@@ -1638,8 +1638,13 @@ static int launch_factored(const gbr_ham *H, const T *x, T *y, cudaStream_t st, 
 }  // namespace gbr
 
 // Precision-specific device arrays hang off the handle as extra buffers.
+// One allocation and one upload for all of them.
 struct gbr_ham_prec {
-    gbr::DevBuf dup, ddn, uval, bcoef, hcoef, ucoef;
+    struct Part {
+        void *p = nullptr;
+    };
+    gbr::DevBuf all;
+    Part dup, ddn, uval, bcoef, hcoef, ucoef, ubonds;
 };
 
 namespace gbr {
@@ -1654,7 +1659,7 @@ constexpr int64_t kFusedMax = (int64_t)1 << 16;
 int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, cudaEvent_t *ev) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p, pb->ubonds.p};
     int path = H->path;
     if (path == GBR_HV_AUTO) path = H->D <= kFusedMax ? GBR_HV_FUSED : GBR_HV_FACTORED;
     if (path == GBR_HV_FUSED) {
@@ -1697,7 +1702,7 @@ int hv_launch_lz(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t 
                  int *nparts, bool xt_ready, bool *updated) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p, pb->ubonds.p};
     if (fp == 64)
         return launch_factored<double>(H, (const double *)x, (double *)y, st, hd, ev, nullptr, &hook, nparts, xt_ready,
                                        updated);
@@ -1722,7 +1727,7 @@ int64_t hv_lz_parts(const gbr_ham *H, int fp) {
 int hv_factored_with_scratch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, void *xt, void *zt) {
     const int fpi = fp == 64 ? 1 : 0;
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p, pb->ubonds.p};
     const Scratch ws{xt, zt};
     if (fp == 64) return launch_factored<double>(H, (const double *)x, (double *)y, st, hd, nullptr, &ws);
     return launch_factored<float>(H, (const float *)x, (float *)y, st, hd, nullptr, &ws);
@@ -1740,7 +1745,7 @@ int hv_stage(const gbr_ham *H, const void *x, void *y, int fp, int stage, cudaSt
             return set_error(GBR_EINVAL, "stage %d before stage 2 (scratch) in this precision", stage);
     }
     gbr_ham_prec *pb = prec_bufs(H, fpi);
-    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p};
+    HamDev hd{pb->dup.p, pb->ddn.p, pb->uval.p, pb->bcoef.p, pb->hcoef.p, pb->ucoef.p, pb->ubonds.p};
     if (fp == 64) {
         if (stage == 1) return stage_hop_lists<double>(H, st);
         if (stage == 2) return stage_transpose<double>(H, (const double *)x, st);
@@ -1813,7 +1818,6 @@ static int build_spin(gbr_ham *H, SpinSector &s, int N) {
 
 template <typename T>
 static int upload_prec(gbr_ham *H, gbr_ham_prec *pb) {
-    auto conv = [](const std::vector<double> &v) { return std::vector<T>(v.begin(), v.end()); };
     std::vector<double> dup((size_t)H->up.D), ddn((size_t)H->dn.D);
     GBR_CUDA_TRY(cudaMemcpy(dup.data(), H->up.diag.p, dup.size() * 8, cudaMemcpyDeviceToHost));
     GBR_CUDA_TRY(cudaMemcpy(ddn.data(), H->dn.diag.p, ddn.size() * 8, cudaMemcpyDeviceToHost));
@@ -1827,15 +1831,34 @@ static int upload_prec(gbr_ham *H, gbr_ham_prec *pb) {
                 if (p < q) uc.push_back(bc.back());   // undirected, in the order of ubonds
             }
     if (bc.empty()) bc.push_back(0.0);
-    if (uc.empty()) uc.push_back(0.0);
-    int rc;
-    auto a = conv(dup), b = conv(ddn), u = conv(uv), c = conv(bc), h = conv(hc), o = conv(uc);
-    if ((rc = pb->dup.upload(a.data(), a.size() * sizeof(T)))) return rc;
-    if ((rc = pb->ddn.upload(b.data(), b.size() * sizeof(T)))) return rc;
-    if ((rc = pb->uval.upload(u.data(), u.size() * sizeof(T)))) return rc;
-    if ((rc = pb->bcoef.upload(c.data(), c.size() * sizeof(T)))) return rc;
-    if ((rc = pb->hcoef.upload(h.data(), h.size() * sizeof(T)))) return rc;
-    if ((rc = pb->ucoef.upload(o.data(), o.size() * sizeof(T)))) return rc;
+    // undirected bonds as masks, in the order of their coefficients uc
+    std::vector<BondMasks> ub;
+    for (int p = 0; p < H->L; ++p)
+        for (int q = p + 1; q < H->L; ++q)
+            if (H->h[(size_t)(p * H->L + q)] != 0.0) ub.push_back({(1u << p) | (1u << q), ((1u << q) - 1u) & ~((2u << p) - 1u)});
+    std::vector<unsigned char> blob;
+    std::vector<std::pair<gbr_ham_prec::Part *, size_t>> at;
+    auto add = [&](gbr_ham_prec::Part &part, const void *data, size_t bytes) {
+        at.push_back({&part, blob.size()});
+        const unsigned char *d = static_cast<const unsigned char *>(data);
+        blob.insert(blob.end(), d, d + bytes);
+        blob.resize((blob.size() + 255) & ~(size_t)255, 0);
+    };
+    auto addv = [&](gbr_ham_prec::Part &part, const std::vector<double> &v) {
+        const std::vector<T> t(v.begin(), v.end());
+        add(part, t.data(), t.size() * sizeof(T));
+    };
+    addv(pb->dup, dup);
+    addv(pb->ddn, ddn);
+    addv(pb->uval, uv);
+    addv(pb->bcoef, bc);
+    addv(pb->hcoef, hc);
+    addv(pb->ucoef, uc);
+    add(pb->ubonds, ub.data(), ub.size() * sizeof(BondMasks));
+    blob.resize(blob.size() + 256, 0);   // an empty last part still has an address inside
+    const int rc = pb->all.upload(blob.data(), blob.size());
+    if (rc) return rc;
+    for (auto &x : at) x.first->p = pb->all.as<unsigned char>() + x.second;
     return GBR_OK;
 }
 
@@ -1944,12 +1967,6 @@ extern "C" int gbr_ham_create(int L, const double *h, const double *U, int Nup, 
     std::vector<uint16_t> bonds_blob(pairs);
     bonds_blob.insert(bonds_blob.end(), bidx.begin(), bidx.end());
     int rc = H->bonds.upload(bonds_blob.data(), bonds_blob.size() * 2);
-    std::vector<BondMasks> ub;
-    for (int p = 0; p < L; ++p)
-        for (int q = p + 1; q < L; ++q)
-            if (h[p * L + q] != 0.0) ub.push_back({(1u << p) | (1u << q), ((1u << q) - 1u) & ~((2u << p) - 1u)});
-    if (ub.empty()) ub.push_back({0u, 0u});
-    if (!rc) rc = H->ubonds.upload(ub.data(), ub.size() * sizeof(BondMasks));
     std::vector<uint32_t> bin((size_t)(L + 1) * (L + 1));
     for (int n = 0; n <= L; ++n)
         for (int kk = 0; kk <= L; ++kk) bin[(size_t)(n * (L + 1) + kk)] = (uint32_t)binom(n, kk);
