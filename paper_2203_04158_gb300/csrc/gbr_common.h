@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "gbrank.h"
@@ -100,6 +101,9 @@ struct TriePlan {
     int shift[kMaxChunks];
     std::vector<int64_t> level_off; // H + 1 entries: start of each level
     int64_t size = 0;              // elements without padding
+    // slots whose subtree holds one member, where that first happens on its path,
+    // and the member's rank
+    std::vector<std::pair<int64_t, int64_t>> single;
 };
 
 // Builds the breadth-first packed trie into t (uint64 entries, size + 2^R
@@ -122,6 +126,13 @@ struct gbr_comb {
     uint64_t dim;
 };
 
+namespace gbr {
+constexpr uint32_t kTrieLeaf = 0x80000000u;
+// gbr_trie_create_ordered; leaves = false keeps the table free of kTrieLeaf marks
+// (for kernels that walk every level)
+int trie_create(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first, bool leaves, gbr_trie **out);
+}
+
 struct gbr_trie {
     int M, R, H;
     int msb_first;           // dispatch order of the chunks (trie_build)
@@ -132,6 +143,7 @@ struct gbr_trie {
     int smem_levels;         // number of leading levels copied to shared memory
     int64_t smem_entries;    // entries in those levels
     int64_t hot_entries;     // leading levels read with the L2 evict_last policy
+    int leaf;                // 1: slots of single-member subtrees hold rank | kTrieLeaf
     gbr::DevBuf t;
     gbr::DevBuf members;
 };

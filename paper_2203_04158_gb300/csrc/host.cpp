@@ -195,7 +195,7 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
         for (int d = 0; d < P.H; ++d) k = (k << P.width[d]) | ((a >> P.shift[d]) & ((1ull << P.width[d]) - 1));
         kr[(size_t)i] = {k, (uint64_t)i};
     }
-    std::sort(kr.begin(), kr.end());
+    if (!msb_first) std::sort(kr.begin(), kr.end());   // else the keys are the members, in order
     std::vector<int> below(P.H, 0);
     for (int d = P.H - 2; d >= 0; --d) below[d] = below[d + 1] + P.width[d + 1];
     auto chunk = [&](size_t idx, int d) -> uint64_t {
@@ -208,6 +208,8 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
     std::vector<uint64_t> &T = *t;
     T.clear();
     P.level_off.assign(P.H + 1, 0);
+    P.single.clear();
+    P.single.reserve((size_t)n);
     for (int d = 0; d < P.H; ++d) {
         P.level_off[d] = (int64_t)T.size();
         nxt.clear();
@@ -225,6 +227,7 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
                 int64_t slot = start + (int64_t)(c - cmin);
                 if (d == P.H - 1) T[(size_t)slot] = kr[(size_t)i].second;
                 else nxt.push_back({i, j, slot});
+                if (d < P.H - 1 && j == i + 1 && nd.hi > nd.lo + 1) P.single.push_back({slot, (int64_t)kr[(size_t)i].second});
                 i = j;
             }
         }

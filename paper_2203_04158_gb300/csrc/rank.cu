@@ -328,7 +328,15 @@ template <> __device__ __forceinline__ uint64_t ld_policy<uint64_t>(const uint64
 // interleaved so that their dependent loads overlap.  Entries are unsigned
 // and the pointer arithmetic wraps, so the stored (start - smallest child)
 // works even where it is negative; every index is clamped into the table.
-template <typename E, typename RT, int HT>
+//
+// LEAF (32-bit tables): a slot whose subtree holds a single member has that member's
+// rank, marked in bit 31, in place of the pointer, and a walk ends there.  Below
+// the level where a sparse set's prefixes become unique every further level was a
+// random read (and most of them a DRAM sector) that could lead to one place only.
+// 2^21 members of 40 bits, 2^24 random queries with the check: 518 -> 232 us (DRAM
+// traffic 2.5 GB before); most significant chunk first, without the check: 350 -> 149 us;
+// 20,000 of 46 bits, 1e6 queries: 22 -> 12 us.
+template <typename E, typename RT, int HT, bool LEAF>
 __global__ void __launch_bounds__(kRankThreads) k_trie_rank(const uint64_t *__restrict__ pat, RT *__restrict__ out,
                                                             int64_t n, const TrieK d, const E *__restrict__ t,
                                                             int64_t padded, int64_t smem_entries, int64_t hot_end,
@@ -348,11 +356,13 @@ __global__ void __launch_bounds__(kRankThreads) k_trie_rank(const uint64_t *__re
     for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
         uint64_t a[kRankItems];
         E k[kRankItems];
+        bool done[kRankItems];
 #pragma unroll
         for (int j = 0; j < kRankItems; ++j) {
             const int64_t i = base + threadIdx.x + (int64_t)j * kRankThreads;
             a[j] = i < n ? __ldcs(pat + i) : 0ull;
             k[j] = 0;
+            done[j] = LEAF && i >= n;
         }
 #pragma unroll
         for (int lvl = 0; lvl < (HT > 0 ? HT : kMaxChunks); ++lvl) {
@@ -360,9 +370,14 @@ __global__ void __launch_bounds__(kRankThreads) k_trie_rank(const uint64_t *__re
             const uint32_t mask = (1u << d.width[lvl]) - 1u;
 #pragma unroll
             for (int j = 0; j < kRankItems; ++j) {
+                if (LEAF && done[j]) continue;
                 E idx = k[j] + (E)((uint32_t)(a[j] >> d.shift[lvl]) & mask);
                 idx = idx > last ? last : idx;
                 k[j] = idx < sm_end ? s[idx] : ld_policy<E>(t + idx, idx < hot ? pol_last : pol_first);
+                if (LEAF && lvl + 1 < H && (k[j] & (E)kTrieLeaf)) {
+                    k[j] &= (E)~kTrieLeaf;
+                    done[j] = true;
+                }
             }
         }
 #pragma unroll
@@ -533,7 +548,7 @@ static int launch_trie_rank(const gbr_trie *T, const uint64_t *pat, RT *out, int
     const int grid = grid_for(n, (int64_t)kRankThreads * kRankItems, 4);
 #define GBR_TRIE_CASE(HV)                                                                                  \
     case HV: {                                                                                             \
-        auto kern = k_trie_rank<E, RT, HV>;                                                                \
+        auto kern = T->leaf ? k_trie_rank<E, RT, HV, sizeof(E) == 4> : k_trie_rank<E, RT, HV, false>;      \
         if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
         kern<<<grid, kRankThreads, smem, st>>>(pat, out, n, d, T->t.as<E>(), T->padded, T->smem_entries,   \
                                                T->hot_entries,                                             \
@@ -654,12 +669,13 @@ extern "C" int gbr_comb_unrank(const gbr_comb *c, const void *d_rank, int rank_b
 namespace gbr {
 // Handle from a trie plan and its table (entries as uint64, padding included).
 static int trie_upload(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first, const TriePlan &plan,
-                       std::vector<uint64_t> &t, gbr_trie **out) {
+                       std::vector<uint64_t> &t, bool leaves, gbr_trie **out) {
     int rc = GBR_OK;
     gbr_trie *T = new (std::nothrow) gbr_trie();
     if (!T) return set_error(GBR_ENOMEM, "host allocation failed");
     T->M = M; T->R = R; T->H = plan.H;
     T->msb_first = msb_first;
+    T->leaf = 0;
     for (int l = 0; l < plan.H; ++l) { T->width[l] = plan.width[l]; T->shift[l] = plan.shift[l]; }
     T->n_members = n;
     T->size = plan.size;
@@ -684,7 +700,16 @@ static int trie_upload(const uint64_t *h_sorted, int64_t n, int M, int R, int ms
         rc = T->t.upload(t.data(), t.size() * 8);
     } else {
         std::vector<uint32_t> t32(t.size());
-        for (size_t i = 0; i < t.size(); ++i) t32[i] = (uint32_t)t[i];   // wraps negative offsets on purpose
+        const size_t above = (size_t)plan.level_off[plan.H - 1];   // entries above the last level
+        uint32_t seen = 0;
+        for (size_t i = 0; i < above; ++i) seen |= t32[i] = (uint32_t)t[i];   // wraps negative offsets on purpose
+        for (size_t i = above; i < t.size(); ++i) t32[i] = (uint32_t)t[i];
+        // marks where they end at least a quarter of the members' walks early and every
+        // pointer above the last level leaves bit 31 free
+        T->leaf = leaves && (int64_t)plan.single.size() * 4 >= n && T->padded < (int64_t)kTrieLeaf && n < (int64_t)kTrieLeaf &&
+                  !(seen & kTrieLeaf);
+        if (T->leaf)
+            for (const auto &s : plan.single) t32[(size_t)s.first] = (uint32_t)s.second | kTrieLeaf;
         std::vector<uint64_t>().swap(t);
         rc = T->t.upload(t32.data(), t32.size() * 4);
     }
@@ -695,9 +720,8 @@ static int trie_upload(const uint64_t *h_sorted, int64_t n, int M, int R, int ms
 }
 }  // namespace gbr
 
-extern "C" int gbr_trie_create_ordered(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first,
-                                       gbr_trie **out) {
-    clear_error();
+namespace gbr {
+int trie_create(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first, bool leaves, gbr_trie **out) {
     if (!out) return set_error(GBR_EINVAL, "out is NULL");
     *out = nullptr;
     if (msb_first != 0 && msb_first != 1) return set_error(GBR_EINVAL, "msb_first=%d must be 0 or 1", msb_first);
@@ -705,7 +729,14 @@ extern "C" int gbr_trie_create_ordered(const uint64_t *h_sorted, int64_t n, int 
     std::vector<uint64_t> t;
     int rc = trie_build(h_sorted, n, M, R, &plan, &t, msb_first);
     if (rc) return rc;
-    return trie_upload(h_sorted, n, M, R, msb_first, plan, t, out);
+    return trie_upload(h_sorted, n, M, R, msb_first, plan, t, leaves, out);
+}
+}  // namespace gbr
+
+extern "C" int gbr_trie_create_ordered(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first,
+                                       gbr_trie **out) {
+    clear_error();
+    return trie_create(h_sorted, n, M, R, msb_first, true, out);
 }
 
 extern "C" int gbr_trie_create_from_table(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first,
@@ -723,7 +754,8 @@ extern "C" int gbr_trie_create_from_table(const uint64_t *h_sorted, int64_t n, i
         return set_error(GBR_EINVAL, "table of %lld entries, the member list's trie has %lld", (long long)len,
                          (long long)t.size());
     t.assign(h_t, h_t + len);
-    return trie_upload(h_sorted, n, M, R, msb_first, plan, t, out);
+    // no marks: the walk goes through the caller's entries, whatever they hold
+    return trie_upload(h_sorted, n, M, R, msb_first, plan, t, false, out);
 }
 
 extern "C" int gbr_trie_create(const uint64_t *h_sorted, int64_t n, int M, int R, gbr_trie **out) {

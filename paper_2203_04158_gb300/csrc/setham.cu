@@ -273,7 +273,7 @@ extern "C" int gbr_setham_create_ordered(int L, const double *h, const double *U
     S->n = n;
     std::vector<uint16_t> pairs, bidx;
     int rc = build_hamk(L, h, U, GBR_RANK_STAGGERED, &S->k, &pairs, &bidx);
-    if (!rc) rc = gbr_trie_create_ordered(h_states, n, 2 * L, R, msb_first, &S->trie);   // validates order, duplicates, width
+    if (!rc) rc = trie_create(h_states, n, 2 * L, R, msb_first, false, &S->trie);   // validates order, duplicates, width
     if (rc) { delete S; return rc; }
     // elements: the diagonal plus every hop of every member (for a set closed
     // under H, exactly the matrix elements one H·v visits)

@@ -279,3 +279,26 @@ def test_trie_edge_cases(G):
     assert np.array_equal(as_u64(r64), np.arange(wide.size, dtype=np.uint64))
     G.gbr_trie_rank_bisect(t64, to_dev_u64(wide), r64, check=1)
     assert np.array_equal(as_u64(r64), np.arange(wide.size, dtype=np.uint64))
+
+
+@pytest.mark.parametrize("n,bits,R", [(1, 40, 8), (2, 63, 8), (300, 17, 4), (5000, 40, 8), (60000, 17, 8), (200000, 48, 11)])
+@pytest.mark.parametrize("msb", [False, True])
+def test_trie_walks_that_end_early(G, n, bits, R, msb):
+    """Sparse sets, whose walks end where a subtree holds one member, and dense
+    ones, whose walks do not: members and strangers, in both index widths."""
+    import torch
+    st = S.trie_member_set(n, bits, seed=40 + n)
+    t = G.gbr_trie_create(st, bits, R, msb)
+    rng = np.random.default_rng(n)
+    j = rng.integers(0, n, 3 * 2048 + 11)
+    q = st[j].copy()
+    odd = np.arange(q.size) % 5 == 0
+    q[odd] ^= np.uint64(1) << rng.integers(0, bits, int(odd.sum())).astype(np.uint64)
+    at = np.minimum(np.searchsorted(st, q), n - 1)
+    want = np.where(st[at] == q, at, -1)
+    for dt in (torch.int32, torch.int64):
+        r = torch.empty(q.size, dtype=dt, device="cuda")
+        G.gbr_trie_rank(t, to_dev_u64(q), r, check=1)
+        assert np.array_equal(r.cpu().numpy(), want)
+        G.gbr_trie_rank(t, to_dev_u64(st[j]), r, check=0)
+        assert np.array_equal(r.cpu().numpy(), j)
