@@ -222,12 +222,16 @@ __global__ void __launch_bounds__(kRedThreads) k_norm2(const LzState *st, const 
 }
 
 // which: 0 = alpha_k = sum / g_k; 1 = beta_{k+1} = sqrt(sum) with the
-// stopping test; each also stores the scalars the vector kernels need
+// stopping test and (advance) the next step's number; each also stores the scalars the vector kernels need
 constexpr int kFinThreads = 1024;
 
 __global__ void __launch_bounds__(kFinThreads) k_finalize(LzState *st, double *alpha, double *beta, double *scal,
-                                                          const double *part, int nparts, int which, int iters) {
+                                                          const double *part, int nparts, int which, int iters,
+                                                          int advance) {
     if (st->stop) return;
+    // what the scalars at the end need, loaded beside the partial sums
+    const int k = st->k;
+    const double igk = scal[kScal * k], scale = st->scale;
     // four independent running sums per thread (fixed order), so the loads
     // of one thread are not one dependency chain
     double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
@@ -242,13 +246,12 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(LzState *st, double *a
     for (; i < nparts; i += blockDim.x) v0 += part[i];
     const double s = block_sum<kFinThreads>((v0 + v1) + (v2 + v3));
     if (threadIdx.x != 0) return;
-    const int k = st->k;
     if (which == 0) {
         // the partials hold <w, u_k> = g_k alpha_k
-        const double a = s * scal[kScal * k];
+        const double a = s * igk;
         alpha[k] = a;
-        scal[kScal * k + 2] = a * scal[kScal * k];
-        st->scale = fmax(st->scale, fabs(a));
+        scal[kScal * k + 2] = a * igk;
+        st->scale = fmax(scale, fabs(a));
         if (!isfinite(a)) {
             st->stop = 1;
             st->nonfinite = 1;
@@ -262,14 +265,16 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(LzState *st, double *a
         const double b = sqrt(fmax(s, 0.0));
         beta[k + 1] = b;
         scal[kScal * (k + 1)] = 1.0 / b;
-        scal[kScal * (k + 1) + 1] = b * scal[kScal * k];
+        scal[kScal * (k + 1) + 1] = b * igk;
         if (k + 1 >= iters) {
             st->stop = 1;
-        } else if (b <= 1e-13 * st->scale) {
+        } else if (b <= 1e-13 * scale) {
             st->stop = 1;
             st->breakdown = 1;
+        } else if (advance) {
+            st->k = k + 1;
         }
-        st->scale = fmax(st->scale, b);
+        st->scale = fmax(scale, b);
     }
 }
 
@@ -962,6 +967,8 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
         k_step1<T><<<z.grid, kRedThreads, 0, z.st>>>(st, z.scal.as<double>(), vprev, v, w, n, part, pass2 ? 0 : 1);
         ++nk;
     }
+    // nothing reads the step's number between beta and the next step: beta's kernel advances it
+    const bool separate_advance = pass2 || z.tol > 0.0 || want_ritz;
     // alpha (which 0) or beta (which 1) from np partial sums, through the
     // first-stage reduction when there are many
     auto finalize = [&](int np, int which) {
@@ -974,7 +981,7 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
             np = kReduceBlocks;
         }
         k_finalize<<<1, kFinThreads, 0, z.st>>>(st, z.alpha.as<double>(), z.beta.as<double>(), z.scal.as<double>(), src,
-                                                np, which, z.iters);
+                                                np, which, z.iters, which == 1 && !separate_advance);
         ++nk;
     };
     if (!pass2) finalize(nparts, 0);
@@ -1029,8 +1036,10 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
                                                         z.iters <= kTriSmemRows, z.ritz_tmp.as<double>());
         ++nk;
     }
-    k_advance<<<1, 32, 0, z.st>>>(st);
-    nk += 1;
+    if (separate_advance) {
+        k_advance<<<1, 32, 0, z.st>>>(st);
+        ++nk;
+    }
     count_launches(nk);
     GBR_LAUNCH_CHECK();
     return GBR_OK;
