@@ -159,13 +159,13 @@ __global__ void __launch_bounds__(kRankThreads) k_comb_rank_pairs(const ulonglon
 // only.  The last kLowBits positions are one look-up: the patterns of that
 // many bits listed by popcount, in increasing order within one.
 //
-// Bound: instruction issue (80 % of the slots, 180 warp instructions per 32
-// ranks; DRAM 31 %).  2^25 32-bit ranks of the half-filled 32-orbital sector:
-// 194 us, against 1,782 us for one thread per rank that looked each position's
+// Bound: instruction issue (DRAM 41 %).  2^25 32-bit ranks of the half-filled
+// 32-orbital sector: 146 us, against 1,782 us for one thread per rank that looked each position's
 // binomial up in global memory in a loop of its own length (14.8 of 32 lanes
-// active); 4e6 64-bit ranks of 62 orbitals, 31 set: 78 against 424 us.  The row
-// addresses are 32-bit shared-memory addresses with constant offsets: through
-// C++ indexing the same loop took 228 us, through pointers 257 us.  14 looked-up
+// active); 4e6 64-bit ranks of 62 orbitals, 31 set: 71 against 424 us.  The row
+// addresses are 32-bit shared-memory addresses with constant offsets and the
+// updates predicated: through C++ indexing the same loop took 228 us, through
+// pointers 257 us, with the compiler's selects 194 us.  14 looked-up
 // positions are 32 KiB a block, which still leaves room for the registers' three
 // blocks a multiprocessor.
 constexpr int kLowBits = 14;
@@ -180,25 +180,26 @@ __host__ __device__ constexpr int unrank_low_bits(int M) { return M < kLowBits ?
 // its entries, padded to 16 bytes
 __host__ __device__ constexpr int unrank_list_entries(int low) { return low < 3 ? 8 : 1 << low; }
 
-// loads from a 32-bit shared-memory address plus a constant
-template <int OFF> __device__ __forceinline__ uint32_t lds32(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1 + %2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
+// One position, D rows below the one q points at: five instructions, three of them
+// predicated (left to the compiler the updates became selects).
+template <int D> __device__ __forceinline__ void unrank_step(uint32_t &q, uint32_t &r, uint32_t &bits, uint32_t bit) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .u32 b;\n\t"
+        "ld.shared.u32 b, [%1 + %4];\n\t"
+        "setp.ge.u32 p, %0, b;\n\t"
+        "@p sub.u32 %0, %0, b;\n\t"
+        "@p or.b32 %2, %2, %3;\n\t"
+        "@p sub.u32 %1, %1, 4;\n\t}"
+        : "+r"(r), "+r"(q), "+r"(bits)
+        : "r"(bit), "n"(-D * kUnrankRow * 4));
 }
+
+// load from a 32-bit shared-memory address (64-bit positions; predicated by hand like
+// the others their loop took 81 us in place of 71)
 __device__ __forceinline__ uint64_t lds64(uint32_t a) {
     uint64_t v;
     asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a));
     return v;
-}
-// one position, D rows below the one q points at
-template <int D> __device__ __forceinline__ void unrank_step(uint32_t &q, uint32_t &r, uint32_t &bits, int bit) {
-    const uint32_t b = lds32<-D * kUnrankRow * 4>(q);
-    if (r >= b) {
-        r -= b;
-        bits |= 1u << bit;
-        q -= 4;
-    }
 }
 
 // binom65: 65 x 65 binomials, then (as uint16) the 2^low patterns by popcount
@@ -226,14 +227,17 @@ __global__ void __launch_bounds__(kUnrankThreads) k_comb_unrank(const RT *__rest
     stage_table<uint16_t>(list, reinterpret_cast<const uint16_t *>(binom65 + kUnrankListAt), unrank_list_entries(low));
     const int64_t tile = (int64_t)kUnrankThreads * kUnrankItems;
     for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
+        // this tile's pointers, so that an item is a constant offset away
+        const RT *rp = rank + base + threadIdx.x;
+        uint64_t *pp = pat + base + threadIdx.x;
+        const int left = (int)(n - base < tile ? n - base : tile) - (int)threadIdx.x;
         uint64_t rw[kUnrankItems];
         uint32_t r[kUnrankItems], hi[kUnrankItems], lo[kUnrankItems];
         int k[kUnrankItems];
         bool ok[kUnrankItems];
 #pragma unroll
         for (int j = 0; j < kUnrankItems; ++j) {
-            const int64_t i = base + threadIdx.x + (int64_t)j * kUnrankThreads;
-            rw[j] = i < n ? (uint64_t)__ldcs(rank + i) : 0ull;
+            rw[j] = j * kUnrankThreads < left ? (uint64_t)__ldcs(rp + j * kUnrankThreads) : 0ull;
             // an index beyond the sector walks as 0 and is marked at the end
             ok[j] = rw[j] < dim;
             if (!ok[j]) rw[j] = 0;
@@ -269,23 +273,23 @@ __global__ void __launch_bounds__(kUnrankThreads) k_comb_unrank(const RT *__rest
         int p = narrow - 1;
         for (; p >= 32; --p) {
 #pragma unroll
-            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], hi[j], p - 32);
+            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], hi[j], 1u << (p - 32));
 #pragma unroll
             for (int j = 0; j < kUnrankItems; ++j) q[j] -= kUnrankRow * 4;
         }
         for (; p - 2 >= low; p -= 3) {
 #pragma unroll
-            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], lo[j], p);
+            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], lo[j], 1u << p);
 #pragma unroll
-            for (int j = 0; j < kUnrankItems; ++j) unrank_step<1>(q[j], r[j], lo[j], p - 1);
+            for (int j = 0; j < kUnrankItems; ++j) unrank_step<1>(q[j], r[j], lo[j], 1u << (p - 1));
 #pragma unroll
-            for (int j = 0; j < kUnrankItems; ++j) unrank_step<2>(q[j], r[j], lo[j], p - 2);
+            for (int j = 0; j < kUnrankItems; ++j) unrank_step<2>(q[j], r[j], lo[j], 1u << (p - 2));
 #pragma unroll
             for (int j = 0; j < kUnrankItems; ++j) q[j] -= 3 * kUnrankRow * 4;
         }
         for (; p >= low; --p) {
 #pragma unroll
-            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], lo[j], p);
+            for (int j = 0; j < kUnrankItems; ++j) unrank_step<0>(q[j], r[j], lo[j], 1u << p);
 #pragma unroll
             for (int j = 0; j < kUnrankItems; ++j) q[j] -= kUnrankRow * 4;
         }
@@ -293,10 +297,9 @@ __global__ void __launch_bounds__(kUnrankThreads) k_comb_unrank(const RT *__rest
         for (int j = 0; j < kUnrankItems; ++j) k[j] = (int)(q[j] - (bn - kUnrankRow * 4)) >> 2;
 #pragma unroll
         for (int j = 0; j < kUnrankItems; ++j) {
-            const int64_t i = base + threadIdx.x + (int64_t)j * kUnrankThreads;
-            if (i >= n) break;
+            if (j * kUnrankThreads >= left) break;
             lo[j] |= list[off[k[j]] + r[j]];
-            __stcs(pat + i, ok[j] ? ((uint64_t)hi[j] << 32 | lo[j]) : ~0ull);
+            __stcs(pp + j * kUnrankThreads, ok[j] ? ((uint64_t)hi[j] << 32 | lo[j]) : ~0ull);
         }
     }
 }
