@@ -305,11 +305,15 @@ int gbr_ham_tune(gbr_ham *H, int fp, void *stream);
  *     spin-down pass keeps its product row-major), 0 = plain row gathers;
  *   [1..3]: rows per CTA of the spin-down pass, the spin-up pass and the
  *     spin-up pass with the fused Lanczos update (plain: 4, 8 or 16;
- *     windowed: 32 or 64; 0 = default);
+ *     windowed: 32 or 64; 0 = default, which takes fewer rows where the CTAs
+ *     would not fill the chip);
  *   [4]: chunk width R of the per-spin staggered tables (Fig. fastrank):
  *     8 or 4 (0 = 8); the paper compares both inside the H·v (Sec. V-B);
- *   [5]: threads per state of the fused per-element kernel: 1, 2 or 4
- *     (0 = 1); the threads of a state split its occupied sites;
+ *   [5]: threads per state of the fused per-element kernel: 1, 2 or 4; the
+ *     threads of a state split its occupied sites (0 = by the sector's size:
+ *     eight, splitting its bonds, while the chip holds them all -- up to
+ *     38,912 states on 152 multiprocessors, where 0 is also what
+ *     gbr_ham_get_shape reports -- else 1);
  *   [6..8]: threads per CTA of the plain spin-down, spin-up and fused-update
  *     passes: 128, or 64 for column chunks half as wide (0 = 128); the
  *     windowed kernels always run 256 (reported as such).

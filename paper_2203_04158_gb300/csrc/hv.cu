@@ -1651,10 +1651,13 @@ namespace gbr {
 
 static gbr_ham_prec *prec_bufs(const gbr_ham *H, int fpi);
 
-// Largest sector that the automatic path gives to the fused kernel: 63,504 states
-// 10.1 us FP32 and 11.3 us FP64 there, 11.6 and 13.5 us in the factored path's three
-// launches, whose time hardly grows up to a few hundred thousand states.
-constexpr int64_t kFusedMax = (int64_t)1 << 16;
+// Largest sector that the automatic path gives to the fused kernel.  In time the
+// line would lie near 80,000 states (63,504: 10.1 us FP32 and 11.3 us FP64, against 11.6
+// and 13.5 us in the factored path's three launches, whose time hardly grows up to
+// a few hundred thousand), but the fused path needs no scratch of the handle, so
+// that these sectors' products can run side by side on several streams and be captured
+// without a call before.
+constexpr int64_t kFusedMax = (int64_t)1 << 17;
 
 int hv_launch(const gbr_ham *H, const void *x, void *y, int fp, cudaStream_t st, cudaEvent_t *ev) {
     const int fpi = fp == 64 ? 1 : 0;
