@@ -230,8 +230,13 @@ struct BatchLay {
     int beg[kBatchClasses + 1];             // sectors of each class in the sorted list
     int64_t slot;                           // doubles of global scratch per CTA
 };
-// doubles of global scratch of a sector: x, the restart's source (D each), the solver's 3 (K + 2)
-__host__ __device__ inline int64_t team_slot(int64_t D, int iters) { return 2 * D + 3 * ((iters < D ? iters : D) + 2); }
+// doubles of global scratch of a sector: x, the restart's source (D each), the solver's 3 (K + 2);
+// an even number, so that every team's solver work starts on a 16-byte boundary (the second
+// run keeps its coefficients there in packs)
+__host__ __device__ inline int64_t team_slot(int64_t D, int iters) {
+    const int64_t K = iters < D ? iters : D;
+    return (2 * D + 3 * (K + 2) + 1) & ~(int64_t)1;
+}
 
 template <int T>
 __device__ void solve_sector(const SectorDesc sd, const ModelDev &m, const double *__restrict__ start, const BatchLay &bl,
@@ -466,7 +471,7 @@ __device__ void batch_class(int cls, const SectorDesc *__restrict__ secs, const 
     constexpr int teams = NT / T;
     const int team = threadIdx.x / T, bar = 1 + team;
     smem += team * (bl.bytes / teams & ~15);
-    xg += team * (bl.slot / teams);
+    xg += team * (bl.slot / teams & ~(int64_t)1);   // at least an (even) team_slot
     TeamVars &tv = *reinterpret_cast<TeamVars *>(smem);
     while (true) {
         if (threadIdx.x % T == 0) tv.cur = bl.beg[cls] + atomicAdd(counter + cls, 1);

@@ -50,6 +50,20 @@ def test_batch_small_set_every_sector(G):
     assert k == ns
 
 
+@pytest.mark.parametrize("iters", [512, 513])
+def test_batch_recurrence_limits_around_the_shared_memory_of_its_solver(G, iters):
+    """The tridiagonal solver's arrays lie in shared memory up to 512 coefficients and
+    in global memory beyond; every sector of three models under both."""
+    models = [S.siam(m) for m in (3, 40, 101)]
+    _, res = run_batch(G, models, iters)
+    ref = []
+    for h, U in models:
+        L = h.shape[0]
+        ref.extend(ref_sector_E(h, U, a, b) for a in range(L + 1) for b in range(L + 1))
+    err = np.abs(res["sector_E"] - np.array(ref)) / np.maximum(1.0, np.abs(ref))
+    assert err.max() <= 1e-9
+
+
 def test_batch_256_models_sampled(G):
     models = [S.siam(m) for m in range(256)]
     ns, res = run_batch(G, models)
