@@ -362,3 +362,28 @@ def test_fp64_class_sums_over_the_whole_range(G, kind, model_):
         X = np.abs(x).reshape(mats[0].shape[0], mats[1].shape[0])
         total = (mats[0] @ X + X @ mats[1].T + 4.0 * min(Nu, Nd) * X).ravel()
         assert np.all(np.abs(outs[0] - ref) <= 2.0 ** -49 * total + 2.0 ** -1070), kind
+
+
+@pytest.mark.parametrize("fp", [32, 64])
+@pytest.mark.parametrize("L,Nu,Nd", [(10, 3, 5), (10, 4, 4), (11, 4, 4), (9, 1, 8), (12, 2, 3)])
+def test_hv_of_untuned_handles_around_the_size_rules(G, L, Nu, Nd, fp):
+    """The defaults of an untuned handle: eight threads a state in the per-element
+    kernel while 8 D fits 2,048 threads a multiprocessor, one beyond, and gathers of
+    fewer rows and narrower vectors for small grids; both against the oracle."""
+    import torch
+    h = S.chain(L) + 0.1 * np.eye(L)
+    h[0, 2] = h[2, 0] = -0.4
+    U = S.uniform_U(L, 3.0)
+    H = G.gbr_ham_create(L, h, U, Nu, Nd)
+    D, _ = G.gbr_ham_info(H)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (G.gbr_ham_get_shape(H, fp)["threads_per_state"] == 0) == (8 * D <= 2048 * sms)
+    x = S.start_vector(D, 3)
+    ref = oracle.hv(L, h, U, Nu, Nd, x.astype(np.float32).astype(np.float64) if fp == 32 else x)
+    xd = torch.from_numpy(x).cuda()
+    xd = xd.float() if fp == 32 else xd
+    for path in (G.GBR_HV_AUTO, G.GBR_HV_FUSED, G.GBR_HV_FACTORED):
+        G.gbr_ham_set_path(H, path)
+        y = torch.full_like(xd, 7.0)
+        G.gbr_hv(H, xd, y)
+        assert rel_inf(y.double().cpu().numpy(), ref) <= (TOL64 if fp == 64 else TOL32), path

@@ -364,3 +364,16 @@ def test_ring18_full_size_against_closed_form_and_bethe_ansatz(G, U):
     del s
     G.gbr_release_cache()
     torch.cuda.empty_cache()
+
+
+def test_recurrences_beyond_the_shared_memory_of_the_tridiagonal_solver(G):
+    """Up to 2,000 coefficients the tridiagonal solves work in shared memory (the
+    eigenvector's up to 1,200), beyond that in global memory."""
+    L, h, U, Nu, Nd = ring8()
+    H = G.gbr_ham_create(L, h, U, Nu, Nd)
+    ref = oracle.dense_E0(L, h, U, Nu, Nd)
+    for iters in (2000, 2001, 3400):
+        r = G.gbr_lanczos(H, v0(4900), iters, prec=G.GBR_PREC_FP64, refine=True)
+        assert r["iters"] == iters
+        for E in (r["E_ritz"], r["E0"]):
+            assert abs(E - ref) <= 1e-10 * abs(ref), (iters, E, ref)
