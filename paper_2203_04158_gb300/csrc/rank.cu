@@ -1,7 +1,6 @@
 // Ranking and unranking kernels for fixed-popcount sectors (staggered
 // lookup, Sec. III-B of Wallerberger & Held) and for packed tries (Sec. IV).
 #include <algorithm>
-#include <mutex>
 #include <cstring>
 
 #include "gbr_common.h"
@@ -314,7 +313,12 @@ struct TrieK {
 
 // Loads with an L2 eviction priority: the upper levels of a trie (a few tens
 // of MB, touched by every query) are kept in L2 with evict_last while the
-// deep levels, read once per query at random, go with evict_first.
+// deep levels, read once per query at random, go with evict_first (2^21 members of
+// 40 bits, 2^24 queries: 230 us, 290 with evict_normal for the upper ones).  No
+// persisting set-aside is asked for: it belongs to the whole context and outlives the
+// trie, gave the walk nothing (230 against 232 us; 2^24 members, 2^26 queries 1385
+// against 1362), and took L2 from every later kernel: an 80-step solve of the 14-site
+// ring 13.0 -> 15.1 ms, 2^27 staggered ranks 300 -> 308 us, the 4x4 torus 2.02 -> 2.08 ms.
 template <typename E> __device__ __forceinline__ E ld_policy(const E *p, uint64_t pol);
 template <> __device__ __forceinline__ uint32_t ld_policy<uint32_t>(const uint32_t *p, uint64_t pol) {
     uint32_t v;
@@ -510,39 +514,8 @@ static int launch_comb_unrank(const gbr_comb *c, const RT *rank, uint64_t *pat, 
     return GBR_OK;
 }
 
-// The walk reads the leading ("hot") levels with the L2 evict_last policy.
-// The L2 keeps such lines only inside its persisting set-aside, which is
-// empty unless the context asks for one, so the hot levels were evicted by
-// the random reads of the large levels.  This sizes the set-aside to the hot
-// levels (at most the device's maximum), once per process and device; the
-// set-aside belongs to this process's CUDA context and ends with it.
-static size_t g_persist_done[64] = {0};
-static std::mutex g_persist_mu;
-
-size_t ensure_persisting_l2(size_t bytes) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lock(g_persist_mu);
-    if (g_persist_done[dev] >= bytes) return g_persist_done[dev];
-    int maxp = 0;
-    if (cudaDeviceGetAttribute(&maxp, cudaDevAttrMaxPersistingL2CacheSize, dev) != cudaSuccess || maxp <= 0) {
-        cudaGetLastError();
-        return 0;
-    }
-    size_t cur = 0;
-    cudaDeviceGetLimit(&cur, cudaLimitPersistingL2CacheSize);
-    const size_t want = std::min(bytes, (size_t)maxp);
-    if (cur < want && cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, want) != cudaSuccess) {
-        cudaGetLastError();   // no set-aside on this device (e.g. a MIG slice): the walk still runs
-        return 0;
-    }
-    g_persist_done[dev] = std::max(cur, want);
-    return g_persist_done[dev];
-}
-
 template <typename E, typename RT>
 static int launch_trie_rank(const gbr_trie *T, const uint64_t *pat, RT *out, int64_t n, int check, cudaStream_t st) {
-    ensure_persisting_l2((size_t)T->hot_entries * sizeof(E));
     TrieK d;
     memset(&d, 0, sizeof(d));
     d.H = T->H;
