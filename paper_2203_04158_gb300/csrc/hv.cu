@@ -548,10 +548,10 @@ struct CombineArgs {
 // shifted into place, signed and added to the 64-bit sum of its class (which is shifted
 // down when E grows); the others go to FP64 FMAs, which the integer work leaves time for.
 //
-// Bound: instruction issue (73 % of the slots), FP64 pipe 60 %.  4x4 torus with
-// diagonal hops (two classes, 35e6 states): 4.16 -> 2.56 ms; 14-site ring (11.8e6):
-// 510 -> 341 us.  All hops as integers: 3.48 ms and 360 us; one of four to FP64 with two
-// classes: 2.64 ms, two of four with one: 357 us.
+// Bound: the FP64 pipe (90 % busy, from the FMAs left to it) beside instruction issue
+// (59-66 % of the slots).  4x4 torus with diagonal hops (two classes, 35e6 states):
+// 4.16 -> 2.50 ms; 14-site ring (11.8e6): 510 -> 341 us.  All hops as integers: 3.48 ms
+// and 360 us; one of four to FP64 with two classes: 2.58 ms, two of four with one: 357 us.
 //
 // Error: a shift drops at most 2^-55 of the largest |x| of the sum (for values within
 // 2^3 of it, nothing), an FP64 addition rounds at 2^-53 of the running sum, so the sum
