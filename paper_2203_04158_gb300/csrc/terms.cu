@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(kTermThreads) k_term_hv(const TermK tk, const 
             cnt[s] = 0;
         }
         const int64_t i = i0 + g;
+        // past the end the last member is gone through again, and nothing is stored
+        const E own = (E)(i < tk.n ? i : tk.n - 1);
         W mine = a[0];
 #pragma unroll
         for (int s = 1; s < S; ++s)
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(kTermThreads) k_term_hv(const TermK tk, const 
 #pragma unroll
                 for (int u = 0; u < kTermUnroll; ++u) {
                     if (!d[u].a) {
-                        k[u] = (E)i;   // diagonal term
+                        k[u] = own;   // diagonal term
                     } else if ((check || BISECT) && !(k[u] < (E)tk.n && __ldg(states + k[u]) == (uint64_t)(mine ^ d[u].a))) {
                         on[u] = false;
                     }

@@ -125,3 +125,29 @@ def test_term_tiles_and_members_per_warp(G, M, N, nterms):
         y, x, _ = run(G, M, terms, st, fp=fp)
         y_ref, _ = oracle.hv_ops(terms, st, x)
         assert rel_inf(y, y_ref) <= (TOL64 if fp == 64 else TOL32), (M, N, nterms, fp)
+
+
+@pytest.mark.parametrize("rest", [0, 1, 2, 3])
+def test_last_warp_of_four_members_stays_inside_the_vectors(G, rest):
+    """64 members a multiprocessor and `rest` more: four members a warp, the last
+    warp with `rest` of them, and diagonal terms, which read x at the member's own
+    place.  What lies behind x is NaN and must not reach y, and nothing may be
+    written behind y."""
+    import torch
+    M = 16
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    st = oracle.enumerate_sector(M, 8)
+    n = 64 * sms + rest
+    if n > st.size:
+        pytest.skip("more multiprocessors than the sector has members for")
+    st = st[-n:].copy()    # its last member holds the upper orbitals
+    terms = [(0.5 + p, [2 * p + 1, 2 * p]) for p in range(M)] + _ladder_terms(M, 40, 7)
+    T = G.gbr_termham_create(M, tuples(G, terms), st, 8)
+    for dtype, tol in ((torch.float64, TOL64), (torch.float32, TOL32)):
+        buf = torch.full((n + 32,), float("nan"), dtype=dtype, device="cuda")
+        buf[:n] = torch.from_numpy(S.start_vector(n, 3)).to(dtype)
+        out = torch.full_like(buf, 7.0)
+        G.gbr_termham_hv(T, buf[:n], out[:n])
+        y_ref, _ = oracle.hv_ops(terms, st, buf[:n].double().cpu().numpy())
+        assert rel_inf(out[:n].double().cpu().numpy(), y_ref) <= tol
+        assert bool((out[n:] == 7.0).all())
