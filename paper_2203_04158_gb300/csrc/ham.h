@@ -35,6 +35,7 @@ struct HamK {
     double hu;                 // that coefficient
     int ncabs;                 // distinct |h_pq| if there are one or two, else 0 ...
     double cabs[2];            // ... and their values
+    int apart;                 // 1: two, one of them more than four times the other
     int rank_method;           // GBR_RANK_*
     int nucls;                 // U classes
     uint32_t umask[kMaxUClasses];

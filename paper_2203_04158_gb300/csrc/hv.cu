@@ -547,15 +547,21 @@ struct CombineArgs {
 // exponent E seen so far in the column, the 53-bit significand with three more bits below it is
 // shifted into place, signed and added to the 64-bit sum of its class (which is shifted
 // down when E grows); the others go to FP64 FMAs, which the integer work leaves time for.
+// APART: an exponent of its own for each class, where the larger |h_pq| is more than four
+// times the smaller (HamK::apart): with one for both, a small x behind the strong bonds
+// would be cut against a large x behind the weak ones.
 //
 // Bound: the FP64 pipe (90 % busy, from the FMAs left to it) beside instruction issue
 // (59-66 % of the slots).  4x4 torus with diagonal hops (two classes, 35e6 states):
 // 4.16 -> 2.50 ms; 14-site ring (11.8e6): 510 -> 341 us.  All hops as integers: 3.48 ms
 // and 360 us; one of four to FP64 with two classes: 2.58 ms, two of four with one: 357 us.
+// APART: 2.63 ms (t' = 0.2 t) on the torus and 109 us on its 853,776-state 12-site sibling,
+// against 2.52 ms and 97 us with one exponent (t' = 0.3 t).
 //
-// Error: a shift drops at most 2^-55 of the largest |x| of the sum (for values within
-// 2^3 of it, nothing), an FP64 addition rounds at 2^-53 of the running sum, so the sum
-// is at least as exact as the chain of FMAs it replaces.  Room: 53 + 3 bits and the sign leave 2^7 > kIntHops terms.
+// Error: a shift drops at most 2^-55 of the largest |x| that shares the exponent (for
+// values within 2^3 of it, nothing).  That |x| meets a coefficient at most four times
+// smaller than the sum's own, so a sum of n hops is within n 2^-53 of sum |h x|, the bound of the
+// chain of FMAs it replaces.  Room: 53 + 3 bits and the sign leave 2^7 > kIntHops terms.
 // Infinities and NaN (E all ones) are left to the caller, which sums the row again in
 // FP64; denormals and zeros are exact.
 constexpr int kIntHops = 96;
@@ -577,17 +583,18 @@ __device__ __forceinline__ double int_to_double(long long a, int ex) {
     return __longlong_as_double((long long)(bits | (a < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
-template <int V, bool TWO> struct RowSum64 {
+template <int V, bool TWO, bool APART> struct RowSum64 {
     static constexpr int FMA = TWO ? 2 : 1;   // hops of four that go to the FMA
     long long a0[V], a1[TWO ? V : 1];
-    int E[V];
+    int E0[V], E1[APART ? V : 1];
     double f[V];
     __device__ __forceinline__ RowSum64() {
 #pragma unroll
         for (int c = 0; c < V; ++c) {
             a0[c] = 0;
+            E0[c] = 0x00100000;
             if (TWO) a1[c] = 0;
-            E[c] = 0x00100000;
+            if (APART) E1[c] = 0x00100000;
             f[c] = 0.0;
         }
     }
@@ -599,13 +606,22 @@ template <int V, bool TWO> struct RowSum64 {
         asm volatile("mov.u32 %0, 8;" : "=r"(eight));
 #pragma unroll
         for (int c = 0; c < V; ++c) {
-            int e = E[c];
+            int e0 = E0[c], e1 = APART ? E1[c] : 0;
 #pragma unroll
-            for (int i = 0; i < NI; ++i) e = max(e, __double2hiint(v[i][c]) & 0x7FF00000);
-            const int d = min((e - E[c]) >> 20, 63);
-            E[c] = e;
+            for (int i = 0; i < NI; ++i) {
+                const int ex = __double2hiint(v[i][c]) & 0x7FF00000;
+                if (APART && (w[i] >> 31)) e1 = max(e1, ex);
+                else e0 = max(e0, ex);
+            }
+            const int d = min((e0 - E0[c]) >> 20, 63);
+            E0[c] = e0;
             a0[c] >>= d;
-            if (TWO) a1[c] >>= d;
+            if (APART) {
+                a1[c] >>= min((e1 - E1[c]) >> 20, 63);
+                E1[c] = e1;
+            } else if (TWO) {
+                a1[c] >>= d;
+            }
             int n0 = 0, n1 = 0;   // minus the number of complemented terms of each class
 #pragma unroll
             for (int i = 0; i < NI; ++i) {
@@ -613,6 +629,7 @@ template <int V, bool TWO> struct RowSum64 {
                 const uint32_t top = (uint32_t)((hi & 0x000FFFFF) | min(ex, 0x00100000));
                 unsigned long long sig = (unsigned long long)(uint32_t)__double2loint(v[i][c]) * eight;
                 sig += (unsigned long long)(top * eight) << 32;
+                const int e = APART && (w[i] >> 31) ? e1 : e0;
                 const unsigned long long m = sig >> min((e - max(ex, 0x00100000)) >> 20, 63);
                 const int sg = (hi ^ __double2hiint(h[i])) >> 31;
                 const long long t = (long long)m ^ (long long)sg;
@@ -635,10 +652,10 @@ template <int V, bool TWO> struct RowSum64 {
     }
     // the column's sum; false if a value was not finite
     __device__ __forceinline__ bool finish(int c, const double *cabs, double *r) const {
-        const int ex = (E[c] >> 20) - 1023 - 52 - 3;   // exponent of the sums' unit
-        if (E[c] == 0x7FF00000) return false;
-        double s = fma(cabs[0], int_to_double(a0[c], ex), f[c]);
-        if (TWO) s = fma(cabs[1], int_to_double(a1[c], ex), s);
+        if (E0[c] == 0x7FF00000 || (APART && E1[c] == 0x7FF00000)) return false;
+        constexpr int bias = 1023 + 52 + 3;   // of a sum's unit
+        double s = fma(cabs[0], int_to_double(a0[c], (E0[c] >> 20) - bias), f[c]);
+        if (TWO) s = fma(cabs[1], int_to_double(a1[c], ((APART ? E1[c] : E0[c]) >> 20) - bias), s);
         *r = s;
         return true;
     }
@@ -658,9 +675,12 @@ template <int V, bool TWO> struct RowSum64 {
 // sector: combine 1.16 ms (10 CTAs) against 1.21 ms (free) and 1.25 ms (16).
 // NT threads per CTA (128, or 64 for column chunks half as wide: the
 // gathered rows of a chunk then take half the L2).
-constexpr int kGather64 = 768;   // FP64: 80 registers
+// FP64: threads a multiprocessor, 48 to 80 registers each
+constexpr int gather64_threads(int vec, int mode) {
+    return vec == 1 ? (mode == 0 ? 1280 : mode == 1 ? 1152 : 896) : mode <= 1 ? 896 : 768;
+}
 template <typename T, int VEC, int MODE, int TR, int NT>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : kGather64 / NT)) k_gather(const int64_t Drows, const int64_t Dcols, const int hmax,
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : gather64_threads(VEC, MODE) / NT)) k_gather(const int64_t Drows, const int64_t Dcols, const int hmax,
                                                 const int64_t nrb, const uint16_t *__restrict__ cnt,
                                                 const uint32_t *__restrict__ tgt, const uint16_t *__restrict__ bond,
                                                 const T *__restrict__ bcoef, const int uniform, const T hu,
@@ -827,8 +847,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : kGather64 / 
                         o[0] = __ldcg(p);
                     }
                 };
-                auto sum = [&](auto classes) {
-                    RowSum64<VEC, decltype(classes)::value> rs;
+                auto sum = [&](auto classes, auto apart) {
+                    RowSum64<VEC, decltype(classes)::value, decltype(apart)::value> rs;
                     int k = 0;
                     for (; k + 4 <= n; k += 4) {
                         const uint4 t4 = *reinterpret_cast<const uint4 *>(ti + k);
@@ -854,8 +874,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 1280 / NT : kGather64 / 
                             acc[v] = a;
                         }
                 };
-                if (two) sum(std::true_type{});
-                else sum(std::false_type{});
+                if (!two) sum(std::false_type{}, std::false_type{});
+                else if (ca.hk.apart) sum(std::true_type{}, std::true_type{});
+                else sum(std::true_type{}, std::false_type{});
             }
         } else if (VEC == 2) {
             T a0 = 0, a1 = 0;
@@ -1150,8 +1171,8 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
             int k = 0;
             if (sizeof(T) == 8 && ints) {
                 if constexpr (sizeof(T) == 8) {
-                    auto sum = [&](auto classes) {
-                        RowSum64<VEC, decltype(classes)::value> rs;
+                    auto sum = [&](auto classes, auto apart) {
+                        RowSum64<VEC, decltype(classes)::value, decltype(apart)::value> rs;
                         for (; k + 4 <= n; k += 4) {
                             const uint4 t4 = *reinterpret_cast<const uint4 *>(ti + k);
                             const uint32_t w[4] = {t4.x, t4.y, t4.z, t4.w};
@@ -1175,8 +1196,9 @@ __global__ void __launch_bounds__(256, 2) k_gwin(const int64_t Drows, const int6
                                 acc[v] = a;
                             }
                     };
-                    if (two) sum(std::true_type{});
-                    else sum(std::false_type{});
+                    if (!two) sum(std::false_type{}, std::false_type{});
+                    else if (ca.hk.apart) sum(std::true_type{}, std::true_type{});
+                    else sum(std::true_type{}, std::false_type{});
                 }
             }
 #pragma unroll 2
@@ -1900,6 +1922,7 @@ int build_hamk(int L, const double *h, const double *U, int rank_method, HamK *k
             k.cabs[k.ncabs++] = v;
         }
     if (k.ncabs < 0) k.ncabs = 0;
+    k.apart = k.ncabs == 2 && 0.25 * std::max(k.cabs[0], k.cabs[1]) > std::min(k.cabs[0], k.cabs[1]);
     for (int p = 0; p < L; ++p) {
         const double u = U ? U[p] : 0.0;
         if (u == 0.0) continue;

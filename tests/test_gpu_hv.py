@@ -364,6 +364,49 @@ def test_fp64_class_sums_over_the_whole_range(G, kind, model_):
         assert np.all(np.abs(outs[0] - ref) <= 2.0 ** -49 * total + 2.0 ** -1070), kind
 
 
+def _spin_matrix(h, L, N):
+    """One spin's hopping matrix with its fermion signs (diagonal: h_pp of the occupied sites)."""
+    st = oracle.enumerate_sector(L, N).astype(np.int64)
+    m = np.zeros((st.size, st.size))
+    for i, a in enumerate(st):
+        m[i, i] = sum(h[p, p] for p in range(L) if a >> p & 1)
+        for p in range(L):
+            for q in range(L):
+                if p != q and h[p, q] and a >> p & 1 and not a >> q & 1:
+                    lo, hi = min(p, q), max(p, q)
+                    sign = -1 if bin(int(a) & ((1 << hi) - 1) & ~((2 << lo) - 1)).count("1") & 1 else 1
+                    m[i, np.searchsorted(st, a ^ (1 << p) ^ (1 << q))] = sign * h[p, q]
+    return m
+
+
+@pytest.mark.parametrize("weak", [0.3, 1e-3, 1e-6, 1e-9, 1e4])
+def test_fp64_class_sums_of_unequal_magnitudes(G, weak):
+    """Two hop magnitudes far apart and vectors over six decades, so that some rows
+    have their small elements behind the strong bonds and large ones behind the weak.
+    Against extended precision every element stays within n 2^-53 of its own sum of
+    magnitudes, n the number of its terms: what a chain of FP64 FMAs guarantees."""
+    import torch
+    L, Nu, Nd = 9, 4, 3
+    h = S.square(3, 3, 1.0, -weak)
+    mats = [_spin_matrix(h, L, N).astype(np.longdouble) for N in (Nu, Nd)]
+    D = oracle.sector_dim(L, Nu, Nd)
+    rng = np.random.default_rng(11)
+    x = rng.uniform(-1, 1, D) * 10.0 ** rng.uniform(-6, 0, D)
+    X = x.astype(np.longdouble).reshape(mats[0].shape[0], mats[1].shape[0])
+    ref = (mats[0] @ X + X @ mats[1].T).ravel()
+    total = (abs(mats[0]) @ abs(X) + abs(X) @ abs(mats[1]).T).ravel()
+    n = max(int((mats[0] != 0).sum(1).max() + (mats[1] != 0).sum(1).max()) + 2, 1)
+    H = G.gbr_ham_create(L, h, None, Nu, Nd)
+    G.gbr_ham_set_path(H, G.GBR_HV_FACTORED)
+    xd = torch.from_numpy(x).cuda()
+    for window in (0, 1):
+        G.gbr_ham_set_shape(H, 64, window)
+        y = torch.empty_like(xd)
+        G.gbr_hv(H, xd, y)
+        err = np.abs(y.cpu().numpy().astype(np.longdouble) - ref)
+        assert np.all(err <= n * 2.0 ** -53 * total), float(np.max(err / total))
+
+
 @pytest.mark.parametrize("fp", [32, 64])
 @pytest.mark.parametrize("L,Nu,Nd", [(10, 3, 5), (10, 4, 4), (11, 4, 4), (9, 1, 8), (12, 2, 3)])
 def test_hv_of_untuned_handles_around_the_size_rules(G, L, Nu, Nd, fp):
