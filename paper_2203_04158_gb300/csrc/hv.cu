@@ -562,8 +562,8 @@ struct CombineArgs {
 // values within 2^3 of it, nothing).  That |x| meets a coefficient at most four times
 // smaller than the sum's own, so a sum of n hops is within n 2^-53 of sum |h x|, the bound of the
 // chain of FMAs it replaces.  Room: 53 + 3 bits and the sign leave 2^7 > kIntHops terms.
-// Infinities and NaN (E all ones) are left to the caller, which sums the row again in
-// FP64; denormals and zeros are exact.
+// Infinities, NaN and values from 2^1017 on are left to the caller, which sums the row
+// again in FP64; denormals and zeros are exact.
 constexpr int kIntHops = 96;
 
 template <typename T> __device__ __forceinline__ bool int_sums(const HamK &hk, int hmax) {
@@ -650,9 +650,11 @@ template <int V, bool TWO, bool APART> struct RowSum64 {
 #pragma unroll
                 for (int c = 0; c < V; ++c) f[c] = fma(h[i < N ? i : 0], v[i < N ? i : 0][c], f[c]);
     }
-    // the column's sum; false if a value was not finite
+    // the column's sum; false if a value was not finite, or so large that the sum of 2^7 of them
+    // leaves the FP64 range, where their products with coefficients below one need not
     __device__ __forceinline__ bool finish(int c, const double *cabs, double *r) const {
-        if (E0[c] == 0x7FF00000 || (APART && E1[c] == 0x7FF00000)) return false;
+        constexpr int top = (2046 - 7) << 20;
+        if (E0[c] > top || (APART && E1[c] > top)) return false;
         constexpr int bias = 1023 + 52 + 3;   // of a sum's unit
         double s = fma(cabs[0], int_to_double(a0[c], (E0[c] >> 20) - bias), f[c]);
         if (TWO) s = fma(cabs[1], int_to_double(a1[c], ((APART ? E1[c] : E0[c]) >> 20) - bias), s);

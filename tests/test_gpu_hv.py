@@ -407,6 +407,30 @@ def test_fp64_class_sums_of_unequal_magnitudes(G, weak):
         assert np.all(err <= n * 2.0 ** -53 * total), float(np.max(err / total))
 
 
+def test_fp64_class_sums_near_the_largest_number(G):
+    """Elements of 1e308 and coefficients of 0.1 and 0.03: the elements' own sum
+    leaves the FP64 range, the products' sums stay inside and come out as such."""
+    import torch
+    L = 9
+    h = S.square(3, 3, 0.1, -0.03)
+    m = _spin_matrix(h, L, 1).astype(np.longdouble)
+    D = L * L
+    H = G.gbr_ham_create(L, h, None, 1, 1)
+    G.gbr_ham_set_path(H, G.GBR_HV_FACTORED)
+    x = np.full(D, 1e308)
+    x[::7] *= -0.5
+    X = x.astype(np.longdouble).reshape(L, L)
+    ref = (m @ X + X @ m.T).ravel()
+    xd = torch.from_numpy(x).cuda()
+    for window in (0, 1):
+        G.gbr_ham_set_shape(H, 64, window)
+        y = torch.empty_like(xd)
+        G.gbr_hv(H, xd, y)
+        yh = y.cpu().numpy()
+        assert np.all(np.isfinite(yh))
+        assert np.max(np.abs(yh.astype(np.longdouble) - ref)) <= 20 * 2.0 ** -53 * 1.1e308
+
+
 @pytest.mark.parametrize("fp", [32, 64])
 @pytest.mark.parametrize("L,Nu,Nd", [(10, 3, 5), (10, 4, 4), (11, 4, 4), (9, 1, 8), (12, 2, 3)])
 def test_hv_of_untuned_handles_around_the_size_rules(G, L, Nu, Nd, fp):
