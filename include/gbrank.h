@@ -305,8 +305,10 @@ int gbr_ham_tune(gbr_ham *H, int fp, void *stream);
  *     spin-down pass keeps its product row-major), 0 = plain row gathers;
  *   [1..3]: rows per CTA of the spin-down pass, the spin-up pass and the
  *     spin-up pass with the fused Lanczos update (plain: 4, 8 or 16;
- *     windowed: 32 or 64; 0 = default, which takes fewer rows where the CTAs
- *     would not fill the chip);
+ *     windowed: 32 or 64; 0 = default: of the plain gathers fewer rows, and
+ *     in FP64 narrower vectors, where the CTAs would not fill the chip;
+ *     gbr_ham_get_shape reports the plain default as 0, and gbr_ham_tune keeps
+ *     it where it is the fastest);
  *   [4]: chunk width R of the per-spin staggered tables (Fig. fastrank):
  *     8 or 4 (0 = 8); the paper compares both inside the H·v (Sec. V-B);
  *   [5]: threads per state of the fused per-element kernel: 1, 2 or 4; the

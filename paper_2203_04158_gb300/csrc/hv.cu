@@ -2114,10 +2114,9 @@ extern "C" int gbr_ham_get_shape(const gbr_ham *H, int fp, int *shape) {
         shape[2] = gwin_rows(H->win_up[fpi]);
         shape[3] = gwin_rows(H->win_lz[fpi]);
     } else {
-        auto plain = [](int v, int dflt) { return (v == 4 || v == 8 || v == 16) ? v : dflt; };
-        shape[1] = plain(H->tune_dn_rows[fpi], 8);
-        shape[2] = plain(H->tune_up_rows[fpi], 8);
-        shape[3] = plain(H->tune_lz_rows[fpi], 8);
+        shape[1] = H->tune_dn_rows[fpi];
+        shape[2] = H->tune_up_rows[fpi];
+        shape[3] = H->tune_lz_rows[fpi];
     }
     shape[4] = H->rank_R[fpi];
     shape[5] = fused_wide(H, fpi) ? 0 : std::max(1, H->fused_tps[fpi]);   // 0: eight, by the rule
@@ -2186,13 +2185,13 @@ extern "C" int gbr_ham_tune(gbr_ham *H, int fp, void *stream) {
     for (int pass = 0; pass < 2; ++pass) {
         int *knob = pass == 0 ? &H->tune_up_rows[fpi] : &H->tune_dn_rows[fpi];
         int *nt_knob = &H->gather_nt[pass == 0 ? 1 : 0][fpi];
-        int best_tr = 8, best_nt = 128;
+        int best_tr = 0, best_nt = 128;
         for (int nt : {128, 64})
-            for (int tr : {4, 8, 16}) {
+            for (int tr : {0, 4, 8, 16}) {   // 0: the rule of gather_shape
                 *knob = tr;
                 *nt_knob = nt;
                 if ((rc = time_it(&ms))) goto done;
-                if (ms < best_plain || (tr == 8 && nt == 128 && ms <= best_plain)) {
+                if (ms < best_plain) {
                     best_plain = ms;
                     best_tr = tr;
                     best_nt = nt;
@@ -2249,7 +2248,7 @@ extern "C" int gbr_ham_tune(gbr_ham *H, int fp, void *stream) {
         float best_lz = 1e30f;
         int best_tr = 0, best_nt = 128;
         for (int nt : {128, 64})
-            for (int tr : {4, 8, 16, 32, 64}) {
+            for (int tr : {0, 4, 8, 16, 32, 64}) {   // 0 (plain gathers): the rule of gather_shape
                 if (winmode != (tr >= 32) || (winmode && nt != 128)) continue;
                 (winmode ? H->win_lz[fpi] : H->tune_lz_rows[fpi]) = tr;
                 H->gather_nt[2][fpi] = nt;
