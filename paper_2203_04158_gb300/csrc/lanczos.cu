@@ -910,7 +910,6 @@ struct Lz {
     DevBuf &state, &alpha, &beta, &scal, &part, &coef, &tri, &svec, &work, &ritz_tmp;
     DevBuf *buf;
     DevBuf &basis, &x, &hx;
-    std::vector<cudaEvent_t> evs;   // profile: 5 events per H·v (stage boundaries)
     explicit Lz(const LzOp &o)
         : op(o), state(o.work->state), alpha(o.work->alpha), beta(o.work->beta), scal(o.work->scal),
           part(o.work->part), coef(o.work->coef), tri(o.work->tri), svec(o.work->svec), work(o.work->work),
@@ -1086,6 +1085,31 @@ static int lz_reorth(Lz &z, bool *done) {
     return GBR_OK;
 }
 
+// What one run creates in the runtime, given back on every way out of it.
+struct LzRun {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    std::vector<cudaEvent_t> evs;   // profile: 5 events per H·v (stage boundaries)
+    cudaStream_t cap = nullptr;     // graph mode: the capture's stream and a graph per buffer phase
+    cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};
+    LzRun() = default;
+    LzRun(const LzRun &) = delete;
+    LzRun &operator=(const LzRun &) = delete;
+    void drop_graphs() {
+        for (cudaGraphExec_t &g : gexec) {
+            if (g) cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+        if (cap) cudaStreamDestroy(cap);
+        cap = nullptr;
+    }
+    ~LzRun() {
+        drop_graphs();
+        for (cudaEvent_t ev : evs) cudaEventDestroy(ev);
+        if (e0) cudaEventDestroy(e0);
+        if (e1) cudaEventDestroy(e1);
+    }
+};
+
 template <typename T>
 static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_lanczos_opts *o, double *h_alpha,
                   double *h_beta, double *h_ritz) {
@@ -1107,9 +1131,10 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
     GBR_LAUNCH_CHECK();
     count_launches(4);
 
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0); cudaEventCreate(&e1);
-    cudaEventRecord(e0, s);
+    LzRun run;
+    GBR_CUDA_TRY(cudaEventCreate(&run.e0));
+    GBR_CUDA_TRY(cudaEventCreate(&run.e1));
+    cudaEventRecord(run.e0, s);
     // graph mode: one graph per buffer phase, captured on a private stream
     // after two eager steps (which also set kernel attributes), replayed on s
     const bool graphs = o->use_graph && !o->profile;
@@ -1126,35 +1151,33 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
         z.xt = z.fuse_t ? hv_xt_scratch(z.op.ham, z.fp) : nullptr;
         if (z.fuse_t && !z.xt) return set_error(GBR_ENOMEM, "scratch for X^T");
     }
-    cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};
     int64_t gnodes[3] = {0, 0, 0};
-    cudaStream_t cap = nullptr;
-    if (graphs) GBR_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     int rc = GBR_OK;
     int phase = 0;
     const bool want_ritz = h_ritz != nullptr;
     bool one_launch = false;
     if (z.reorth && !want_ritz && !o->profile && z.tol == 0.0 && (rc = lz_reorth<T>(z, &one_launch))) return rc;
+    if (graphs && !one_launch) GBR_CUDA_TRY(cudaStreamCreateWithFlags(&run.cap, cudaStreamNonBlocking));
     for (int k = 0; k < z.iters && !one_launch; ++k) {
         if (graphs && k >= 2) {
-            if (!gexec[phase]) {
+            if (!run.gexec[phase]) {
                 cudaStream_t keep = z.st;
-                z.st = cap;
+                z.st = run.cap;
                 const int64_t before = launch_count();
-                GBR_CUDA_TRY(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+                GBR_CUDA_TRY(cudaStreamBeginCapture(run.cap, cudaStreamCaptureModeThreadLocal));
                 rc = lz_step<T>(z, phase, false, nullptr, want_ritz);
                 cudaGraph_t g = nullptr;
-                cudaError_t ce = cudaStreamEndCapture(cap, &g);
+                cudaError_t ce = cudaStreamEndCapture(run.cap, &g);
                 z.st = keep;
                 gnodes[phase] = launch_count() - before;   // captured, not yet run
                 set_launch_count(before);
                 if (rc) { if (g) cudaGraphDestroy(g); break; }
                 if (ce != cudaSuccess) { rc = set_error(GBR_ECUDA, "graph capture failed: %s", cudaGetErrorString(ce)); break; }
-                ce = cudaGraphInstantiate(&gexec[phase], g, 0);
+                ce = cudaGraphInstantiate(&run.gexec[phase], g, 0);
                 cudaGraphDestroy(g);
                 if (ce != cudaSuccess) { rc = set_error(GBR_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(ce)); break; }
             }
-            cudaError_t le = cudaGraphLaunch(gexec[phase], s);
+            cudaError_t le = cudaGraphLaunch(run.gexec[phase], s);
             if (le != cudaSuccess) { rc = set_error(GBR_ECUDA, "graph launch failed: %s", cudaGetErrorString(le)); break; }
             count_launches(gnodes[phase]);
         } else {
@@ -1163,9 +1186,9 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
                 for (int e = 0; e < 5; ++e) {
                     cudaEvent_t ev;
                     GBR_CUDA_TRY(cudaEventCreate(&ev));
-                    z.evs.push_back(ev);
+                    run.evs.push_back(ev);
                 }
-                ev4 = z.evs.data() + z.evs.size() - 5;
+                ev4 = run.evs.data() + run.evs.size() - 5;
             }
             rc = lz_step<T>(z, phase, false, ev4, want_ritz, k, k == 0);
             if (rc) break;
@@ -1179,10 +1202,8 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
             if (hs.stop) break;
         }
     }
-    for (int p = 0; p < 3; ++p)
-        if (gexec[p]) cudaGraphExecDestroy(gexec[p]);
-    if (cap) cudaStreamDestroy(cap);
     if (rc) return rc;
+    run.drop_graphs();
     LzState hs;
     GBR_CUDA_TRY(cudaMemcpyAsync(&hs, z.state.p, sizeof(hs), cudaMemcpyDeviceToHost, s));
     GBR_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1342,24 +1363,21 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
         res->E0 = E;
         res->residual = sqrt(fmax(r2, 0.0) / hd[1]);
     }
-    cudaEventRecord(e1, s);
-    cudaEventSynchronize(e1);
+    cudaEventRecord(run.e1, s);
+    cudaEventSynchronize(run.e1);
     float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
+    cudaEventElapsedTime(&ms, run.e0, run.e1);
     res->seconds = ms * 1e-3;
     res->hv_seconds = 0.0;
-    for (size_t e = 0; e + 4 < z.evs.size(); e += 5) {
+    for (size_t e = 0; e + 4 < run.evs.size(); e += 5) {
         for (int st3 = 0; st3 < 4; ++st3) {
             float t = 0.f;
-            cudaEventElapsedTime(&t, z.evs[e + st3], z.evs[e + st3 + 1]);
+            cudaEventElapsedTime(&t, run.evs[e + st3], run.evs[e + st3 + 1]);
             res->stage_seconds[st3] += t * 1e-3;
             res->stage_launches[st3] += 1;
             res->hv_seconds += t * 1e-3;
         }
     }
-    for (cudaEvent_t ev : z.evs) cudaEventDestroy(ev);
-    z.evs.clear();
-    cudaEventDestroy(e0); cudaEventDestroy(e1);
     if (h_alpha) GBR_CUDA_TRY(cudaMemcpy(h_alpha, z.alpha.p, sizeof(double) * (size_t)kdone, cudaMemcpyDeviceToHost));
     if (h_beta && kdone > 1)
         GBR_CUDA_TRY(cudaMemcpy(h_beta, z.beta.as<double>() + 1, sizeof(double) * (size_t)(kdone - 1), cudaMemcpyDeviceToHost));
