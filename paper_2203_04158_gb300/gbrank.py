@@ -147,6 +147,8 @@ def _check(rc: int):
 # Per-call helpers.  A call on a small sector is as short as its marshalling, so
 # these stay off torch's Python layers: device pointers go to ctypes as plain
 # integers, and the current stream comes from the accessor torch's own launchers use.
+# _torch is the sign that the others are set: _load_torch assigns it last, every helper
+# looks at it first, and threads that load at the same time assign the same things.
 _torch = None
 _raw_stream = None
 _REALS = _PATTERNS = _DOUBLES = None
@@ -170,7 +172,7 @@ def _load_torch():
 
 def _stream(stream):
     if stream is None:
-        if _raw_stream is None:
+        if _torch is None:
             _load_torch()
         if not _torch.cuda.is_initialized():
             return _torch.cuda.current_stream().cuda_stream

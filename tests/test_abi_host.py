@@ -286,3 +286,38 @@ def test_term_and_set_hamiltonians_reject_bad_input_on_the_host(G):
     hbad = np.zeros((3, 3)); hbad[0, 1] = 1.0                   # not symmetric
     with pytest.raises(G.GbrError):
         G.gbr_setham_create(3, hbad, None, np.array([1, 2], dtype=np.uint64))
+
+
+def test_a_thread_that_loads_torch_beside_another_never_sees_half_of_it(monkeypatch):
+    """The helpers' globals are published one after the other; stopped behind each of
+    them, as another thread may find them, the stream accessor works."""
+    import sys
+    torch = pytest.importorskip("torch")
+    from paper_2203_04158_gb300 import gbrank as B
+    names = ("_torch", "_raw_stream", "_REALS", "_PATTERNS", "_DOUBLES")
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 77, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+    for name in names:
+        monkeypatch.setattr(B, name, None)
+    seen = []
+
+    def trace(frame, event, arg):
+        if frame.f_code is not B._load_torch.__code__:
+            return None
+        if event == "line":
+            state = {n: getattr(B, n) for n in names}
+            if not any(state == s for s in seen):
+                seen.append(state)
+        return trace
+
+    sys.settrace(trace)
+    try:
+        B._load_torch()
+    finally:
+        sys.settrace(None)
+    assert len(seen) >= 3      # nothing, some, ... of the globals
+    for state in seen:
+        for n, v in state.items():
+            setattr(B, n, v)
+        assert B._stream(None) == 77, state
