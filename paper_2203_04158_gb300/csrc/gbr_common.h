@@ -102,7 +102,7 @@ struct TriePlan {
     std::vector<int64_t> level_off; // H + 1 entries: start of each level
     int64_t size = 0;              // elements without padding
     // slots whose subtree holds one member, where that first happens on its path,
-    // and the member's rank
+    // and the member's rank (collected on request)
     std::vector<std::pair<int64_t, int64_t>> single;
 };
 
@@ -113,7 +113,7 @@ struct TriePlan {
 // in value share their walk down to the last levels.  Returns GBR_OK or
 // GBR_EINVAL (message set).
 int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, std::vector<uint64_t> *t,
-               int msb_first = 0);
+               int msb_first = 0, bool singles = false);
 
 }  // namespace gbr
 

@@ -169,7 +169,7 @@ void enumerate_combinations(int L, int N, std::vector<uint64_t> &out) {
 // ------------------------------------------------------------------ trie
 
 int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, std::vector<uint64_t> *t,
-               int msb_first) {
+               int msb_first, bool singles) {
     if (M < 1 || M > 64) return set_error(GBR_EINVAL, "trie: M=%d out of range 1..64", M);
     if (R < 1 || R > 16) return set_error(GBR_EINVAL, "trie: R=%d out of range 1..16", R);
     if (n < 1) return set_error(GBR_EINVAL, "trie: empty member set");
@@ -209,7 +209,7 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
     T.clear();
     P.level_off.assign(P.H + 1, 0);
     P.single.clear();
-    P.single.reserve((size_t)n);
+    if (singles) P.single.reserve((size_t)n);
     for (int d = 0; d < P.H; ++d) {
         P.level_off[d] = (int64_t)T.size();
         nxt.clear();
@@ -227,7 +227,7 @@ int trie_build(const uint64_t *sorted, int64_t n, int M, int R, TriePlan *plan, 
                 int64_t slot = start + (int64_t)(c - cmin);
                 if (d == P.H - 1) T[(size_t)slot] = kr[(size_t)i].second;
                 else nxt.push_back({i, j, slot});
-                if (d < P.H - 1 && j == i + 1 && nd.hi > nd.lo + 1) P.single.push_back({slot, (int64_t)kr[(size_t)i].second});
+                if (singles && d < P.H - 1 && j == i + 1 && nd.hi > nd.lo + 1) P.single.push_back({slot, (int64_t)kr[(size_t)i].second});
                 i = j;
             }
         }

@@ -703,7 +703,7 @@ int trie_create(const uint64_t *h_sorted, int64_t n, int M, int R, int msb_first
     if (msb_first != 0 && msb_first != 1) return set_error(GBR_EINVAL, "msb_first=%d must be 0 or 1", msb_first);
     TriePlan plan;
     std::vector<uint64_t> t;
-    int rc = trie_build(h_sorted, n, M, R, &plan, &t, msb_first);
+    int rc = trie_build(h_sorted, n, M, R, &plan, &t, msb_first, leaves);
     if (rc) return rc;
     return trie_upload(h_sorted, n, M, R, msb_first, plan, t, leaves, out);
 }

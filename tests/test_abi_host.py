@@ -321,3 +321,52 @@ def test_a_thread_that_loads_torch_beside_another_never_sees_half_of_it(monkeypa
         for n, v in state.items():
             setattr(B, n, v)
         assert B._stream(None) == 77, state
+
+
+def test_host_trie_memory_is_the_keys_and_the_table(tmp_path):
+    """Building a table on the host takes the dispatch keys (16 bytes a member), the
+    growing table (at most twice its length beside the half that it grows from, 8 bytes an
+    entry) and the nodes of a level; the places that only marked tries need are not
+    collected.  The C++ allocations are counted by a replacement of new and delete."""
+    import subprocess
+    import sys
+    import __graft_entry__
+    __graft_entry__.build()
+    src, so = tmp_path / "count.cpp", tmp_path / "count.so"
+    src.write_text("""
+#include <cstdlib>
+#include <malloc.h>
+#include <new>
+static long live, peak;
+static void *take(std::size_t n) {
+    void *p = std::malloc(n);
+    live += (long)malloc_usable_size(p);
+    if (live > peak) peak = live;
+    return p;
+}
+void *operator new(std::size_t n) { return take(n); }
+void operator delete(void *p) noexcept { if (p) live -= (long)malloc_usable_size(p); std::free(p); }
+void operator delete(void *p, std::size_t) noexcept { if (p) live -= (long)malloc_usable_size(p); std::free(p); }
+extern "C" void count_reset() { peak = live; }
+extern "C" long count_peak() { return peak; }
+""")
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-o", str(so), str(src)])
+    child = """
+import ctypes as C, sys
+import numpy as np
+from paper_2203_04158_gb300 import gbrank as B
+c = C.CDLL(sys.argv[1])
+c.count_peak.restype = C.c_long
+n = 1 << 20
+m, size = np.arange(n, dtype=np.uint64), C.c_int64()
+for order in (0, 1):
+    c.count_reset()
+    start = c.count_peak()
+    assert B.lib().gbr_trie_build_host_ordered(C.c_void_p(m.ctypes.data), n, 24, 8, order, None, 0, C.byref(size)) == 0
+    print(n, size.value, c.count_peak() - start)
+"""
+    out = subprocess.check_output([sys.executable, "-c", child, str(so)], text=True, timeout=120,
+                                  env=dict(os.environ, LD_PRELOAD=str(so), PYTHONPATH=os.path.dirname(os.path.dirname(__file__))))
+    for line in out.split("\n")[:2]:
+        n, size, peak = (int(v) for v in line.split())
+        assert 16 * n < peak <= 16 * n + 8 * 3 * size + n, line
