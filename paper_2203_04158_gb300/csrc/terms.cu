@@ -112,8 +112,6 @@ __global__ void __launch_bounds__(kTermThreads) k_term_hv(const TermK tk, const 
             cnt[s] = 0;
         }
         const int64_t i = i0 + g;
-        // past the end the last member is gone through again, and nothing is stored
-        const E own = (E)(i < tk.n ? i : tk.n - 1);
         W mine = a[0];
 #pragma unroll
         for (int s = 1; s < S; ++s)
@@ -143,7 +141,8 @@ __global__ void __launch_bounds__(kTermThreads) k_term_hv(const TermK tk, const 
 #pragma unroll
             for (int s = 1; s < S; ++s)
                 if (g == s) have = cnt[s];
-            const int todo = end ? have : have - have % UG;
+            // (none for lanes past the last member: a diagonal term reads x at the member's place)
+            const int todo = i >= tk.n ? 0 : end ? have : have - have % UG;
             for (int e = gl; e < todo; e += UG) {
                 MaskPair<W> d[kTermUnroll];
                 T v[kTermUnroll];
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(kTermThreads) k_term_hv(const TermK tk, const 
 #pragma unroll
                 for (int u = 0; u < kTermUnroll; ++u) {
                     if (!d[u].a) {
-                        k[u] = own;   // diagonal term
+                        k[u] = (E)i;   // diagonal term
                     } else if ((check || BISECT) && !(k[u] < (E)tk.n && __ldg(states + k[u]) == (uint64_t)(mine ^ d[u].a))) {
                         on[u] = false;
                     }
