@@ -646,18 +646,27 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
 //   w = u_{k+1} into its slot, partial <w, w> | beta.
 // Every CTA forms beta itself from the same partial sums in the same order.
 //
+// The first pass is the recurrence's w -= (alpha_k / g_k) u_k as well, so there is one
+// projection fewer than in the route with separate launches.  That is enough while the
+// second pass takes less out of w than it leaves, since a pass leaves rounding errors in
+// proportion to what it takes.  Where the first pass leaves little but those
+// (vectors in single precision under a large diagonal shift, the end of the Krylov space),
+// the launch gives up and the solve takes the other route.
+//
 // Bound: latency -- the barriers and the chains of FP64 operations (about 150 clocks
 // each when dependent) in the sums.  Thirteen launches a step, each of a few
 // microseconds, took 65 us a step on the 8-site ring (4,900 states, FP64); one launch
 // takes 22 us a step (100 steps: 6.6 -> 2.2 ms on the device).
 //
 // 8 warps for the elements, one more for the scalars, which works while the others
-// gather.
+// gather.  One CTA a multiprocessor, so that nothing of the 117 registers is spilled
+// (2.61 -> 2.58 ms for the 8-site ring's 100 steps).
 constexpr int kRoWarps = 8, kRoThreads = 32 * (kRoWarps + 1), kRoElems = 256;
 
 struct RoBarrier {
     unsigned count;
     int failed;       // a wait ran out: the solve is abandoned
+    int gave_up;      // the second pass is not enough here
 };
 
 // Grid barrier number `phase` (1, 2, ...) of a cooperative launch; false, once the wait
@@ -709,7 +718,7 @@ __device__ __forceinline__ double ro_warp_sum(const double *p, int n) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const int n, const int m, const int tpe,
+__global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, const int n, const int m, const int tpe,
                                                           const int iters, T *basis, double *alpha, double *beta, double *scal,
                                                           LzState *st, double *npart, double *pdot,
                                                           double *coef, RoBarrier *bar) {
@@ -746,6 +755,7 @@ __global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const
     __syncthreads();
     unsigned phase = 0;
     int k = 0;
+    int took = 0;         // the scalar warp's: largest |<w, v_j>| of the second pass (high word)
     for (;; ++k) {
         const T *u = basis + (int64_t)k * n;
         // gathers; from step 1 on the scalar warp meanwhile finishes beta_k
@@ -773,6 +783,7 @@ __global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const
                 const double bk = sqrt(fmax(s, 0.0)), igp = ig_s, sc = scale_s;
                 if (!isfinite(s)) stop_s = 3;
                 else if (k >= iters) stop_s = 1;
+                else if (took >= __double2hiint(bk)) stop_s = 5;   // or both are zero
                 else if (bk <= 1e-13 * sc) stop_s = 2;
                 const double ig = 1.0 / bk;
                 if (isfinite(s)) {
@@ -866,7 +877,15 @@ __global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const
                     for (; j < je; j += Q) s0 += (T)cs[j] * ue[(int64_t)j * n];
                 }
             }
-            if (worker) sub[i] = (s0 + s1) + (s2 + s3);
+            if (worker) {
+                sub[i] = (s0 + s1) + (s2 + s3);
+            } else if (pass == 1) {
+                // by the high words, since positive numbers order like their bits
+                unsigned hi = 0;
+                for (int j = lane; j < J; j += 32)
+                    hi = max(hi, (unsigned)__double2hiint(fabs(__ldcg(coef + j) * (j ? __ldcg(beta + j) : 1.0))));
+                took = (int)__reduce_max_sync(0xFFFFFFFFu, hi);
+            }
             __syncthreads();
             if (live) {
                 for (int t = 0; t < Q; ++t) wi -= sub[t * mp + i];
@@ -886,8 +905,9 @@ __global__ void __launch_bounds__(kRoThreads) k_lz_reorth(const HvView hv, const
         st->k = stop_s == 4 ? k : k - 1;
         st->stop = 1;
         st->breakdown = stop_s == 2;
-        st->nonfinite = stop_s >= 3;
+        st->nonfinite = stop_s == 3 || stop_s == 4;
         st->scale = scale_s;
+        bar->gave_up = stop_s == 5;
     }
 }
 
@@ -1047,8 +1067,21 @@ static int lz_step(Lz &z, int phase, bool pass2, cudaEvent_t *ev4, bool want_rit
     return GBR_OK;
 }
 
+// state and scalars of a recurrence at step 0
+static int lz_init(Lz &z) {
+    static const LzState zero{};
+    static const double scal0 = 1.0;   // 1/g_0
+    GBR_CUDA_TRY(cudaMemcpyAsync(z.state.p, &zero, sizeof(zero), cudaMemcpyHostToDevice, z.st));
+    GBR_CUDA_TRY(cudaMemsetAsync(z.beta.p, 0, sizeof(double) * (size_t)(z.iters + 2), z.st));
+    GBR_CUDA_TRY(cudaMemsetAsync(z.alpha.p, 0, sizeof(double) * (size_t)(z.iters + 2), z.st));
+    GBR_CUDA_TRY(cudaMemsetAsync(z.scal.p, 0, sizeof(double) * kScal * (size_t)(z.iters + 2), z.st));
+    GBR_CUDA_TRY(cudaMemcpyAsync(z.scal.p, &scal0, sizeof(double), cudaMemcpyHostToDevice, z.st));
+    return GBR_OK;
+}
+
 // The re-orthogonalised recurrence in one cooperative launch (k_lz_reorth); *done false if the
-// sector is too large for it or the device does not take cooperative launches.
+// sector is too large for it, the device does not take cooperative launches or the launch
+// gave up, with the scalars of the recurrence as before it.
 template <typename T>
 static int lz_reorth(Lz &z, bool *done) {
     *done = false;
@@ -1081,8 +1114,8 @@ static int lz_reorth(Lz &z, bool *done) {
     GBR_CUDA_TRY(cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, z.st));
     GBR_CUDA_TRY(cudaStreamSynchronize(z.st));
     if (hb.failed) return set_error(GBR_ETIMEOUT, "a grid barrier of the re-orthogonalised solve ran out");
-    *done = true;
-    return GBR_OK;
+    *done = !hb.gave_up;
+    return *done ? GBR_OK : lz_init(z);
 }
 
 // What one run creates in the runtime, given back on every way out of it.
@@ -1115,13 +1148,8 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
                   double *h_beta, double *h_ritz) {
     const int64_t n = z.n;
     cudaStream_t s = z.st;
-    LzState zero{};
-    GBR_CUDA_TRY(cudaMemcpyAsync(z.state.p, &zero, sizeof(zero), cudaMemcpyHostToDevice, s));
-    GBR_CUDA_TRY(cudaMemsetAsync(z.beta.p, 0, sizeof(double) * (size_t)(z.iters + 2), s));
-    GBR_CUDA_TRY(cudaMemsetAsync(z.alpha.p, 0, sizeof(double) * (size_t)(z.iters + 2), s));
-    GBR_CUDA_TRY(cudaMemsetAsync(z.scal.p, 0, sizeof(double) * kScal * (size_t)(z.iters + 2), s));
-    static const double scal0 = 1.0;   // 1/g_0
-    GBR_CUDA_TRY(cudaMemcpyAsync(z.scal.p, &scal0, sizeof(double), cudaMemcpyHostToDevice, s));
+    int rc = lz_init(z);
+    if (rc) return rc;
     T *B0 = z.buf[0].as<T>();
     k_cast_start<T><<<z.grid, kRedThreads, 0, s>>>(d_v0, B0, n);
     k_norm2<T><<<z.grid, kRedThreads, 0, s>>>(z.state.as<LzState>(), B0, n, z.part.as<double>());
@@ -1152,7 +1180,6 @@ static int lz_run(Lz &z, const double *d_v0, gbr_lanczos_result *res, const gbr_
         if (z.fuse_t && !z.xt) return set_error(GBR_ENOMEM, "scratch for X^T");
     }
     int64_t gnodes[3] = {0, 0, 0};
-    int rc = GBR_OK;
     int phase = 0;
     const bool want_ritz = h_ritz != nullptr;
     bool one_launch = false;

@@ -70,6 +70,30 @@ def test_reorthogonalised_solve_in_one_launch(G, kind, iters):
     assert abs(m["E0"] - o["E0"]) <= (1e-9 if iters >= 70 or D < 500 else 1e-5) * max(1.0, abs(o["E0"]))
 
 
+@pytest.mark.parametrize("shift,iters", [(1e6, 400), (1e8, 20), (1e8, 60)])
+def test_reorthogonalised_solve_where_the_first_pass_leaves_rounding_errors(G, shift, iters):
+    """A large one-body shift leaves single-precision vectors w of alpha_k v_k and its
+    rounding errors, which the second pass of the one-launch route takes most of again:
+    it gives up and the launches with one projection more solve, up to the last of the 400
+    vectors.  Recurrence and energies to within the vectors' precision of the shifted
+    ones, without and with per-step Ritz values (which take the other route at once)."""
+    import torch
+    L, Nu, Nd = 6, 3, 3
+    rng = np.random.default_rng(1)
+    h, U = S.chain(L) + np.diag(rng.uniform(-0.5, 0.5, L)), S.uniform_U(L, 4.0)
+    D, off = oracle.sector_dim(L, Nu, Nd), shift * (Nu + Nd)
+    E = oracle.dense_E0(L, h, U, Nu, Nd)
+    H = G.gbr_ham_create(L, h + shift * np.eye(L), U, Nu, Nd)
+    for seed in range(4):
+        v = torch.from_numpy(np.random.default_rng(seed).uniform(-1, 1, D)).cuda()
+        for want_ritz in (False, True):
+            r = G.gbr_lanczos(H, v, iters, reorth=True, prec=G.GBR_PREC_MIXED, refine=True, want_ritz=want_ritz)
+            a, b = np.atleast_1d(r["alpha"]), np.atleast_1d(r["beta"])
+            assert np.all(np.abs(a - off) <= 8 * 2.0 ** -24 * off + 30), (seed, want_ritz)
+            assert np.all(np.abs(b) <= 8 * 2.0 ** -24 * off + 30), (seed, want_ritz)
+            assert abs(r["E_ritz"] - off - E) <= 4 * 2.0 ** -24 * off, (seed, want_ritz)
+
+
 def test_ring8_mixed_refined_meets_1e9(G):
     L, h, U, Nu, Nd = ring8()
     H = G.gbr_ham_create(L, h, U, Nu, Nd)
