@@ -1523,7 +1523,8 @@ static int launch_gather(const gbr_ham *H, const SpinSector &lists, int64_t Drow
 #define GBR_G(V, R, N)                                                                                       \
     {                                                                                                        \
         auto kern = k_gather<T, V, MODE, R, N>;                                                              \
-        if (smem > 48 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        /* beyond 48 KiB with the kernel's static arrays, which are below 3 KiB */                           \
+        if (smem > 45 * 1024) GBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
         kern<<<(int)blocks, N, smem, st>>>(Drows, Dcols, hmax, nrb, lists.hop_cnt.as<uint16_t>(),            \
                                            lists.hop_tgt.as<uint32_t>(), lists.hop_bond.as<uint16_t>(),      \
                                            (const T *)hd.bcoef, H->k.uniform, (T)H->k.hu, w, z, ca);          \

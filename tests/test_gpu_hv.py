@@ -130,6 +130,33 @@ def test_the_default_rows_survive_a_round_trip_and_the_tuner(G, fp):
     assert torch.equal(y, z)
 
 
+@pytest.mark.parametrize("fp", [32, 64])
+@pytest.mark.parametrize("rows", [4, 8, 16])
+def test_gathers_of_long_hop_lists_near_48_kib_of_shared_memory(G, rows, fp):
+    """Every pair of sites connected: 48 to 64 hops a state, whose staged lists and tiles,
+    with 16 rows a CTA in double precision, lie on both sides of the 48 KiB that a launch has without
+    asking for more (the kernels' own arrays count too)."""
+    import torch
+    for L in (14, 15, 16):
+        h, U = np.ones((L, L)) - np.eye(L), S.uniform_U(L, 4.0)
+        H = G.gbr_ham_create(L, h, U, L // 2, 1)
+        D, _ = G.gbr_ham_info(H)
+        G.gbr_ham_set_path(H, G.GBR_HV_FACTORED)
+        x = torch.from_numpy(S.start_vector(D)).cuda()
+        x = x.float() if fp == 32 else x
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        G.gbr_ham_set_shape(H, fp, 0)
+        G.gbr_hv(H, x, y)
+        G.gbr_ham_set_shape(H, fp, 0, rows, rows, rows)
+        G.gbr_hv(H, x, z)
+        assert torch.equal(y, z)
+        prec = G.GBR_PREC_FP64 if fp == 64 else G.GBR_PREC_MIXED
+        a = G.gbr_lanczos(H, x.double(), 8, prec=prec, refine=False)
+        G.gbr_ham_set_shape(H, fp, 0)
+        b = G.gbr_lanczos(H, x.double(), 8, prec=prec, refine=False)
+        assert np.allclose(a["alpha"], b["alpha"], rtol=0, atol=1e-4 if fp == 32 else 1e-11)
+
+
 def test_hv_rejects_overlap_and_bad_dtype(G):
     import torch
     L, h, U, Nu, Nd = model("ring8")
