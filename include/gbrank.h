@@ -443,8 +443,14 @@ enum { GBR_PREC_FP64 = 0, GBR_PREC_MIXED = 1 };
 
 typedef struct {
     int iters;        /* H·v steps (>= 1) */
-    int reorth;       /* 1 = full re-orthogonalisation (two classical Gram-Schmidt
-                         passes in FP64 against every stored vector) */
+    int reorth;       /* 1 = full re-orthogonalisation: after w -= alpha_k v_k two
+                         classical Gram-Schmidt passes, summed in FP64, against
+                         every stored vector.  gbr_lanczos on sectors of up to 256
+                         states a multiprocessor, with h_ritz NULL, profile 0 and
+                         tol 0, runs in one launch, whose first pass takes alpha_k
+                         v_k off as well (two projections instead of three); where
+                         its second pass takes more out of w than it leaves, the
+                         solve starts again with the three */
     int prec;         /* GBR_PREC_FP64: FP64 vectors and H·v;
                          GBR_PREC_MIXED: FP32 vectors and H·v, FP64 scalars */
     int refine;       /* 1 = form the Ritz vector and return the FP64 Rayleigh

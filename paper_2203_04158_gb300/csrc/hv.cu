@@ -602,7 +602,7 @@ template <int V, bool TWO, bool APART> struct RowSum64 {
     // of four hops the last FMA go to FP64
     template <int N> __device__ __forceinline__ void add(const double (&v)[N][V], const uint32_t *w, const double *h) {
         constexpr int NI = N == 4 ? 4 - FMA : N;
-        uint32_t eight;   // opaque, so that the shift by three stays a multiplication, on the FMA pipe
+        uint32_t eight;   // the shift by three as a multiplication by a value known at run time
         asm volatile("mov.u32 %0, 8;" : "=r"(eight));
 #pragma unroll
         for (int c = 0; c < V; ++c) {
@@ -677,7 +677,11 @@ template <int V, bool TWO, bool APART> struct RowSum64 {
 // sector: combine 1.16 ms (10 CTAs) against 1.21 ms (free) and 1.25 ms (16).
 // NT threads per CTA (128, or 64 for column chunks half as wide: the
 // gathered rows of a chunk then take half the L2).
-// FP64: threads a multiprocessor, 48 to 80 registers each
+// FP64: threads a multiprocessor, so that a thread takes 46 to 78 registers, as it would
+// without the sums with two exponents (with them and one limit of 768 threads the 12-site
+// Anderson model at N = 5, 7, single columns and no class sums, took 41.4 us, now 39.3; the
+// 4x4 torus 2.525, now 2.518 ms).  Models with three magnitudes, whose FMA loop has the limit
+// too: 4x4 torus 5.07 ms without any limit, 4.82 now; 14-site ring of random hops 526 and 445 us.
 constexpr int gather64_threads(int vec, int mode) {
     return vec == 1 ? (mode == 0 ? 1280 : mode == 1 ? 1152 : 896) : mode <= 1 ? 896 : 768;
 }

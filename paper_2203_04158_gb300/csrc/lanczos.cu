@@ -1,7 +1,8 @@
 // Lanczos ground state on the GPU (the paper cites the method in Sec. I and
 // V-B without stating it; this is the textbook three-term recurrence):
 //   v_0 = s/|s|;  w = H v_k - beta_k v_{k-1};  alpha_k = <w, v_k>;
-//   w -= alpha_k v_k;  [two classical Gram-Schmidt passes against v_0..v_k];
+//   w -= alpha_k v_k;  [two classical Gram-Schmidt passes against v_0..v_k; a
+//   small sector's solve in one launch takes alpha_k v_k off in the first of them];
 //   beta_{k+1} = |w|;  stop if beta_{k+1} <= 1e-13 max_j(|alpha_j|, beta_j);
 //   v_{k+1} = w / beta_{k+1};  E = lowest eigenvalue of T_k.
 // The vectors are kept unnormalised, u_j = g_j v_j with g_0 = 1 and

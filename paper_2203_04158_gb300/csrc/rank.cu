@@ -158,15 +158,14 @@ __global__ void __launch_bounds__(kRankThreads) k_comb_rank_pairs(const ulonglon
 // only.  The last kLowBits positions are one look-up: the patterns of that
 // many bits listed by popcount, in increasing order within one.
 //
-// Bound: instruction issue (DRAM 41 %).  2^25 32-bit ranks of the half-filled
-// 32-orbital sector: 146 us, against 1,782 us for one thread per rank that looked each position's
-// binomial up in global memory in a loop of its own length (14.8 of 32 lanes
-// active); 4e6 64-bit ranks of 62 orbitals, 31 set: 71 against 424 us.  The row
-// addresses are 32-bit shared-memory addresses with constant offsets and the
-// updates predicated: through C++ indexing the same loop took 228 us, through
-// pointers 257 us, with the compiler's selects 194 us.  14 looked-up
-// positions are 32 KiB a block, which still leaves room for the registers' three
-// blocks a multiprocessor.
+// Bound: instruction issue (89 % of the slots, DRAM 29 %).  2^25 32-bit ranks of the
+// half-filled 32-orbital sector: 146 us (0.41 of HBM by its bytes), against 1,782 us for one
+// thread per rank that looked each position's binomial up in global memory in a loop of its own
+// length (14.8 of 32 lanes active); 4e6 64-bit ranks of 62 orbitals, 31 set: 71 against 424 us.
+// The row addresses are 32-bit shared-memory addresses with constant offsets and the updates
+// predicated: through C++ indexing the same loop took 228 us, through pointers 257 us, with
+// the updates written as conditional expressions 194 us.  14 looked-up positions are 32 KiB a
+// block, which still leaves room for the registers' three blocks a multiprocessor.
 constexpr int kLowBits = 14;
 constexpr int kNarrowBits = 34;   // C(34, 17) < 2^32 <= C(35, 17): ranks left below position 34 fit 32 bits
 constexpr int kUnrankRow = 65;      // binomials of one position, k = 0 .. 64
@@ -180,7 +179,7 @@ __host__ __device__ constexpr int unrank_low_bits(int M) { return M < kLowBits ?
 __host__ __device__ constexpr int unrank_list_entries(int low) { return low < 3 ? 8 : 1 << low; }
 
 // One position, D rows below the one q points at: five instructions, three of them
-// predicated (left to the compiler the updates became selects).
+// predicated (written in C++ the kernel took 194 us in place of 146).
 template <int D> __device__ __forceinline__ void unrank_step(uint32_t &q, uint32_t &r, uint32_t &bits, uint32_t bit) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .u32 b;\n\t"

@@ -360,7 +360,7 @@ def test_fp64_class_sums_over_the_whole_range(G, kind, model_):
     """The FP64 gathers sum hops of one or two coefficient magnitudes as aligned
     integers: vectors over 200 decades, denormals, mostly zeros, and with
     infinities and NaN, on both vector widths (even and odd per-spin sectors) and
-    both gather families.  Every element within 2^-50 of its own sum of
+    both gather families.  Every element within 2^-49 = 16 * 2^-53 of its own sum of
     magnitudes (an FMA chain of up to 40 terms stays within 40 * 2^-53)."""
     import torch
     L = 9
