@@ -552,8 +552,8 @@ struct CombineArgs {
 // would be cut against a large x behind the weak ones.
 //
 // Bound: the FP64 pipe (90 % busy, from the FMAs left to it) beside instruction issue
-// (59-66 % of the slots).  4x4 torus with diagonal hops (two classes, 35e6 states):
-// 4.16 -> 2.50 ms; 14-site ring (11.8e6): 510 -> 341 us.  All hops as integers: 3.48 ms
+// (60-67 % of the slots).  4x4 torus with diagonal hops (two classes, 35e6 states):
+// 4.16 -> 2.52 ms; 14-site ring (11.8e6): 510 -> 337 us.  All hops as integers: 3.48 ms
 // and 360 us; one of four to FP64 with two classes: 2.58 ms, two of four with one: 357 us.
 // APART: 2.63 ms (t' = 0.2 t) on the torus and 109 us on its 853,776-state 12-site sibling,
 // against 2.52 ms and 97 us with one exponent (t' = 0.3 t).

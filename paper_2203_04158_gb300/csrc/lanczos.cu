@@ -657,7 +657,7 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
 // Bound: latency -- the barriers and the chains of FP64 operations (about 150 clocks
 // each when dependent) in the sums.  Thirteen launches a step, each of a few
 // microseconds, took 65 us a step on the 8-site ring (4,900 states, FP64); one launch
-// takes 22 us a step (100 steps: 6.6 -> 2.2 ms on the device).
+// takes 21 us a step (100 steps: 6.6 -> 2.1 ms on the device).
 //
 // 8 warps for the elements, one more for the scalars, which works while the others
 // gather.  One CTA a multiprocessor, so that nothing of the 117 registers is spilled
