@@ -677,11 +677,11 @@ template <int V, bool TWO, bool APART> struct RowSum64 {
 // sector: combine 1.16 ms (10 CTAs) against 1.21 ms (free) and 1.25 ms (16).
 // NT threads per CTA (128, or 64 for column chunks half as wide: the
 // gathered rows of a chunk then take half the L2).
-// FP64: threads a multiprocessor, so that a thread takes 46 to 78 registers, as it would
-// without the sums with two exponents (with them and one limit of 768 threads the 12-site
-// Anderson model at N = 5, 7, single columns and no class sums, took 41.4 us, now 39.3; the
-// 4x4 torus 2.525, now 2.518 ms).  Models with three magnitudes, whose FMA loop has the limit
-// too: 4x4 torus 5.07 ms without any limit, 4.82 now; 14-site ring of random hops 526 and 445 us.
+// FP64: threads a multiprocessor, so that a thread takes 46 to 78 registers instead of 53 to
+// 101.  Without limits the 12-site Anderson model at N = 5, 7 (single columns) took 41.4 us,
+// now 39.4; one class of hops on the 4x4 torus 1.392, now 1.378 ms, two 2.516 and 2.519, two
+// with an exponent each 2.594 and 2.633.  Models with three magnitudes, whose FMA loop has
+// the limits too: 4x4 torus 4.82 ms both, its 12-site sibling 108.4 and 106.1 us.
 constexpr int gather64_threads(int vec, int mode) {
     return vec == 1 ? (mode == 0 ? 1280 : mode == 1 ? 1152 : 896) : mode <= 1 ? 896 : 768;
 }
