@@ -448,9 +448,9 @@ typedef struct {
                          every stored vector.  gbr_lanczos on sectors of up to 256
                          states a multiprocessor, with h_ritz NULL, profile 0 and
                          tol 0, runs in one launch, whose first pass takes alpha_k
-                         v_k off as well (two projections instead of three); where
-                         its second pass takes more out of w than it leaves, the
-                         solve starts again with the three */
+                         v_k off as well; a third pass follows where the second
+                         takes much out of w beside what it leaves, and where
+                         that is not enough the solve starts again the other way */
     int prec;         /* GBR_PREC_FP64: FP64 vectors and H·v;
                          GBR_PREC_MIXED: FP32 vectors and H·v, FP64 scalars */
     int refine;       /* 1 = form the Ritz vector and return the FP64 Rayleigh

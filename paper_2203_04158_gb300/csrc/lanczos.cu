@@ -649,10 +649,11 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
 //
 // The first pass is the recurrence's w -= (alpha_k / g_k) u_k as well, so there is one
 // projection fewer than in the route with separate launches.  That is enough while the
-// second pass takes less out of w than it leaves, since a pass leaves rounding errors in
-// proportion to what it takes.  Where the first pass leaves little but those
-// (vectors in single precision under a large diagonal shift, the end of the Krylov space),
-// the launch gives up and the solve takes the other route.
+// second pass takes little out of w beside what it leaves, since a pass leaves rounding
+// errors in proportion to what it takes.  Where the first pass leaves little but those (vectors in
+// single precision at the end of the Krylov space or under a large diagonal shift) a third
+// follows, and if that one still takes much, the launch gives up and the solve takes the
+// other route from the start.
 //
 // Bound: latency -- the barriers and the chains of FP64 operations (about 150 clocks
 // each when dependent) in the sums.  Thirteen launches a step, each of a few
@@ -660,14 +661,17 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
 // takes 21 us a step (100 steps: 6.6 -> 2.1 ms on the device).
 //
 // 8 warps for the elements, one more for the scalars, which works while the others
-// gather.  One CTA a multiprocessor, so that nothing of the 117 registers is spilled
-// (2.61 -> 2.58 ms for the 8-site ring's 100 steps).
+// gather.  One CTA a multiprocessor, so that nothing of the 122 registers is spilled
+// (2.62 -> 2.57 ms for the 8-site ring's 100 steps, in the call).
 constexpr int kRoWarps = 8, kRoThreads = 32 * (kRoWarps + 1), kRoElems = 256;
+
+// "much": the largest |<w, v_j>| above 2^-3 of the |w| that is left (high words of doubles)
+constexpr int kRoThird = 3 << 20;
 
 struct RoBarrier {
     unsigned count;
     int failed;       // a wait ran out: the solve is abandoned
-    int gave_up;      // the second pass is not enough here
+    int gave_up;      // three passes are not enough
 };
 
 // Grid barrier number `phase` (1, 2, ...) of a cooperative launch; false, once the wait
@@ -756,7 +760,8 @@ __global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, co
     __syncthreads();
     unsigned phase = 0;
     int k = 0;
-    int took = 0;         // the scalar warp's: largest |<w, v_j>| of the second pass (high word)
+    int took = 0;         // the scalar warp's: largest |<w, v_j>| of the last pass (high word)
+    bool third = false;   // u_k has had a third pass
     for (;; ++k) {
         const T *u = basis + (int64_t)k * n;
         // gathers; from step 1 on the scalar warp meanwhile finishes beta_k
@@ -782,12 +787,14 @@ __global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, co
             const double s = ro_warp_sum(npart, G);
             if (lane == 0) {
                 const double bk = sqrt(fmax(s, 0.0)), igp = ig_s, sc = scale_s;
+                const bool down = bk <= 1e-13 * sc;
                 if (!isfinite(s)) stop_s = 3;
                 else if (k >= iters) stop_s = 1;
-                else if (took >= __double2hiint(bk)) stop_s = 5;   // or both are zero
-                else if (bk <= 1e-13 * sc) stop_s = 2;
+                else if (down && sizeof(T) == 8) stop_s = 2;
+                else if (took >= __double2hiint(bk) - kRoThird) stop_s = third ? 5 : -1;   // or both are zero
+                else if (down) stop_s = 2;
                 const double ig = 1.0 / bk;
-                if (isfinite(s)) {
+                if (stop_s != -1 && isfinite(s)) {
                     ig_s = ig;
                     s_b = bk * igp;
                     scale_s = fmax(sc, bk);
@@ -800,20 +807,22 @@ __global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, co
             }
         }
         __syncthreads();
-        if (stop_s) break;
-        // w = H u_k / g_k - (beta_k / g_{k-1}) u_{k-1}
+        if (stop_s > 0) break;
+        third = stop_s == -1;
+        // w = H u_k / g_k - (beta_k / g_{k-1}) u_{k-1}, or u_k once more
         const int i = (int)threadIdx.x;
         const bool live = i < mine;
         T wi = 0;
         if (live) {
-            wi = ws[i];
-            if (k > 0) wi = lz_rec((T)ig_s, wi, (T)s_b, basis[(int64_t)(k - 1) * n + e0 + i]);
+            wi = third ? basis[(int64_t)k * n + e0 + i] : ws[i];
+            if (k > 0 && !third) wi = lz_rec((T)ig_s, wi, (T)s_b, basis[(int64_t)(k - 1) * n + e0 + i]);
         }
         if (live) ws[i] = wi;
-        // two Gram-Schmidt passes against u_0 .. u_k; the first one's <w, u_k> is g_k alpha_k
-        const int J = k + 1;
+        // two Gram-Schmidt passes against u_0 .. u_k; the first one's <w, u_k> is g_k alpha_k;
+        // or the third against u_0 .. u_{k-1}
+        const int J = third ? k : k + 1;
         const int split = J <= 32 ? 8 : (J <= 64 ? 4 : (J <= 128 ? 2 : 1));   // threads a vector
-        for (int pass = 0; pass < 2; ++pass) {
+        for (int pass = third ? 2 : 0; pass < (third ? 3 : 2); ++pass) {
             __syncthreads();
             if (worker)
                 for (int j0 = 0; j0 < J; j0 += kRoElems / split) {
@@ -880,7 +889,7 @@ __global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, co
             }
             if (worker) {
                 sub[i] = (s0 + s1) + (s2 + s3);
-            } else if (pass == 1) {
+            } else if (pass > 0) {
                 // by the high words, since positive numbers order like their bits
                 unsigned hi = 0;
                 for (int j = lane; j < J; j += 32)
@@ -893,7 +902,11 @@ __global__ void __launch_bounds__(kRoThreads, 1) k_lz_reorth(const HvView hv, co
                 ws[i] = wi;
             }
         }
-        if (stop_s) break;
+        if (stop_s > 0) break;
+        if (third) {
+            --k;   // u_{k+1} in its place again, and the step after it from the start
+            if (threadIdx.x == 0) stop_s = 0;
+        }
         // w is u_{k+1}
         if (live) basis[(int64_t)(k + 1) * n + e0 + i] = wi;
         const double s = ro_block_sum((double)wi * (double)wi, red);

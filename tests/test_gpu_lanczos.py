@@ -70,11 +70,11 @@ def test_reorthogonalised_solve_in_one_launch(G, kind, iters):
     assert abs(m["E0"] - o["E0"]) <= (1e-9 if iters >= 70 or D < 500 else 1e-5) * max(1.0, abs(o["E0"]))
 
 
-@pytest.mark.parametrize("shift,iters", [(1e6, 400), (1e8, 20), (1e8, 60)])
+@pytest.mark.parametrize("shift,iters", [(1e6, 400), (1e8, 20), (1e8, 60), (1e8, 400)])
 def test_reorthogonalised_solve_where_the_first_pass_leaves_rounding_errors(G, shift, iters):
     """A large one-body shift leaves single-precision vectors w of alpha_k v_k and its
-    rounding errors, which the second pass of the one-launch route takes most of again:
-    it gives up and the launches with one projection more solve, up to the last of the 400
+    rounding errors, of which the second pass of the one-launch route takes much again: it
+    makes a third, or gives up for the route with one projection more, up to the last of 400
     vectors.  Recurrence and energies to within the vectors' precision of the shifted
     ones, without and with per-step Ritz values (which take the other route at once)."""
     import torch
@@ -84,7 +84,7 @@ def test_reorthogonalised_solve_where_the_first_pass_leaves_rounding_errors(G, s
     D, off = oracle.sector_dim(L, Nu, Nd), shift * (Nu + Nd)
     E = oracle.dense_E0(L, h, U, Nu, Nd)
     H = G.gbr_ham_create(L, h + shift * np.eye(L), U, Nu, Nd)
-    for seed in range(4):
+    for seed in range(8):
         v = torch.from_numpy(np.random.default_rng(seed).uniform(-1, 1, D)).cuda()
         for want_ritz in (False, True):
             r = G.gbr_lanczos(H, v, iters, reorth=True, prec=G.GBR_PREC_MIXED, refine=True, want_ritz=want_ritz)
@@ -92,6 +92,34 @@ def test_reorthogonalised_solve_where_the_first_pass_leaves_rounding_errors(G, s
             assert np.all(np.abs(a - off) <= 8 * 2.0 ** -24 * off + 30), (seed, want_ritz)
             assert np.all(np.abs(b) <= 8 * 2.0 ** -24 * off + 30), (seed, want_ritz)
             assert abs(r["E_ritz"] - off - E) <= 4 * 2.0 ** -24 * off, (seed, want_ritz)
+
+
+@pytest.mark.parametrize("L,Nu,Nd", [(4, 2, 2), (5, 2, 3), (8, 1, 1), (8, 8, 4)])
+def test_reorthogonalised_solve_to_the_end_of_the_krylov_space(G, L, Nu, Nd):
+    """Rings whose Krylov space is smaller than the sector (degenerate levels): double
+    precision breaks down there, in single precision the recurrence goes on with rounding
+    errors; both stay one launch.  The outermost Ritz values are the sector's levels."""
+    import torch
+    h, U = S.chain(L), S.uniform_U(L, 4.0)
+    D = oracle.sector_dim(L, Nu, Nd)
+    E = oracle.dense_E0(L, h, U, Nu, Nd)
+    H = G.gbr_ham_create(L, h, U, Nu, Nd)
+    for seed in range(4):
+        v = torch.from_numpy(np.random.default_rng(seed).uniform(-1, 1, D)).cuda()
+        for prec, tol in ((G.GBR_PREC_FP64, 1e-10), (G.GBR_PREC_MIXED, 1e-5)):
+            n0 = G.gbr_launch_count()
+            r = G.gbr_lanczos(H, v, D, reorth=True, prec=prec, refine=True)
+            assert G.gbr_launch_count() - n0 < 30
+            assert abs(r["E0"] - E) <= 1e-9 * max(1.0, abs(E))
+            assert abs(r["E_ritz"] - E) <= tol * max(1.0, abs(E))
+            if prec == G.GBR_PREC_FP64:
+                assert r["breakdown"] or r["iters"] == D
+            a, b = np.atleast_1d(r["alpha"]), np.atleast_1d(r["beta"])[:r["iters"] - 1]
+            t = np.linalg.eigvalsh(np.diag(a) + np.diag(b, 1) + np.diag(b, -1))
+            o = oracle.lanczos(L, h, U, Nu, Nd, np.random.default_rng(seed).uniform(-1, 1, D), D, True)
+            oa, ob = np.asarray(o["alpha"]), np.asarray(o["beta"])
+            levels = np.linalg.eigvalsh(np.diag(oa) + np.diag(ob[:oa.size - 1], 1) + np.diag(ob[:oa.size - 1], -1))
+            assert abs(t[-1] - levels[-1]) <= 10 * tol * max(1.0, abs(levels[-1]))
 
 
 def test_ring8_mixed_refined_meets_1e9(G):
