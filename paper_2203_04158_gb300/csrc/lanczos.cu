@@ -650,15 +650,15 @@ __global__ void k_scale_start(T *__restrict__ v, const double *nrm2, int64_t n) 
 // The first pass is the recurrence's w -= (alpha_k / g_k) u_k as well, so there is one
 // projection fewer than in the route with separate launches.  That is enough while the
 // second pass takes little out of w beside what it leaves, since a pass leaves rounding
-// errors in proportion to what it takes.  Where the first pass leaves little but those (vectors in
-// single precision at the end of the Krylov space or under a large diagonal shift) a third
-// follows, and if that one still takes much, the launch gives up and the solve takes the
-// other route from the start.
+// errors in proportion to what it takes.  Where the first pass leaves little but those
+// (vectors in single precision at the end of the Krylov space or under a large diagonal
+// shift) a third follows, and if that one still takes much, the launch gives up and the
+// solve takes the other route from the start.
 //
 // Bound: latency -- the barriers and the chains of FP64 operations (about 150 clocks
 // each when dependent) in the sums.  Thirteen launches a step, each of a few
 // microseconds, took 65 us a step on the 8-site ring (4,900 states, FP64); one launch
-// takes 21 us a step (100 steps: 6.6 -> 2.1 ms on the device).
+// takes 22 us a step (100 steps: 6.6 -> 2.2 ms on the device).
 //
 // 8 warps for the elements, one more for the scalars, which works while the others
 // gather.  One CTA a multiprocessor, so that nothing of the 122 registers is spilled
